@@ -419,7 +419,7 @@ spl_status build_pack(spl_geometry *g, cudaStream_t st)
                        "plane nnz");
     if (s == SPL_OK) s = cuda_check(cudaStreamSynchronize(st), "plane nnz");
     char *b2 = nullptr;
-    const size_t bytes2 = align256((size_t)nnz * (2 * sizeof(int) + 2 * sizeof(float))) + 256;
+    const size_t bytes2 = 4 * align256((size_t)nnz * sizeof(float));  // four arrays, each on a 256-byte boundary
     if (s == SPL_OK && cudaMalloc(&b2, bytes2) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(b1);

@@ -764,3 +764,29 @@ def test_cuda_graph_capture_of_mixed_geometry(env):
         assert torch.isfinite(y_g).all() and torch.isfinite(c_g).all()
         assert torch.allclose(y_g, y_e, rtol=0, atol=1e-5 * float(y_e.abs().max()))
         assert torch.allclose(c_g, c_e, rtol=0, atol=1e-5 * float(c_e.abs().max()))
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+def test_plane_matrix_arrays_are_whole(env, degree):
+    """The four entry arrays of a plane matrix lie on 256-byte boundaries in
+    one allocation that holds all of them, whatever the entry count leaves
+    over: with other geometries built around it, the last column's adjoint
+    equals that of the plain march (the last array once ended up to 320
+    bytes outside the allocation)."""
+    torch, spl = env
+    keep = []
+    for it in range(10):
+        dims = (19, 32, 20 + it)
+        geo = I.tilt_series(9 + it, 35, 29, 0.7)
+        pair = [spl.Geometry(dims, I.centred_origin(dims), geo) for _ in range(2)]
+        for g in pair:
+            spl.prepare(g, spl.basis(degree))
+        y = torch.randn(geo.n_rays, device="cuda")
+        for g in pair:
+            a, b = (torch.empty(g.coeff_shape, device="cuda") for _ in range(2))
+            spl.adjoint(g, y, a, spl.basis(degree))
+            spl.adjoint(g, y, b, spl.basis(degree, separable=spl.SPL_SEP_OFF))
+            g.status()
+            # the same footprint values, another FP32 summation order
+            assert float((a - b).abs().max()) <= 1e-5 * float(b.abs().max())
+        keep.append(pair)
