@@ -164,7 +164,12 @@ typedef struct {
  * three layouts (x, y and z fast) of four shifted copies each (about
  * 48 nx ny nz bytes; not for a parallel geometry whose views are all in the
  * flat class) and, for more than 48 views or 2^22 explicit rays, an FP64
- * accumulator (8 nx ny nz bytes).
+ * accumulator (8 nx ny nz bytes).  Scratch of the forward, for geometries
+ * with rays outside the flat class: the coefficients resampled along each
+ * axis that is the dominant one of some ray, 16 bytes per coefficient and
+ * axis on a grid padded by 3 (left out where few rays cross a large grid,
+ * where explicit rays would need more than 320 MB, above 24 GB, and when it
+ * cannot be allocated: spl_forward then takes the form without scratch).
  * Uses the current CUDA device.
  * Errors: SPL_ERR_ARG, SPL_ERR_NONFINITE, SPL_ERR_UNSUPPORTED, SPL_ERR_OOM,
  * SPL_ERR_CUDA; *out is NULL on error. */
@@ -223,11 +228,17 @@ spl_status spl_prepare(spl_geometry *g, const spl_basis_desc *basis, void *strea
 /* ---------------------------------------------------------------- operators */
 
 /* Forward projection y = A c (Algorithm 2; Eq. 4 summed over all pairs).
- * One GPU thread per ray marches the unit cells of the ray's dominant axis
- * (Definition 2.1); an (n+1)^3 window holds the bases whose support contains
- * the current point (Algorithm 3's neighbourhood, de-duplicated by
- * construction), and each basis the ray crosses adds c_k * Pphi(w, s - X(k))
- * once.  Slice-separable views of a parallel geometry go through the plane
+ * Rays are marched over the unit cells of their dominant axis (Definition
+ * 2.1), cut into the pieces on which every basis is one polynomial.  Degrees
+ * 1 to 3 integrate f itself on each piece (Eq. 2) from the coefficients
+ * resampled once per call into the power basis of the dominant axis; degree
+ * 0, calls captured into a CUDA graph and geometries without the scratch
+ * keep an (n+1)^3 window of the bases whose support contains the current
+ * point (Algorithm 3's neighbourhood, de-duplicated by construction), and
+ * each basis the ray crosses adds c_k * Pphi(w, s - X(k)) once.  The two are
+ * the same matrix and agree to FP32 rounding.  Calls on one geometry from
+ * several streams or threads may overlap: the library orders their use of
+ * the scratch on the GPU.  Slice-separable views of a parallel geometry go through the plane
  * matrices instead (see spl_prepare), with the same footprint values.
  *   Cone views: every ray is walked with the general (three-factor) form
  *   of the march, so a ray's values do not depend on its direction class.
@@ -239,8 +250,10 @@ spl_status spl_forward(const spl_geometry *g, const spl_basis_desc *basis, const
                        void *stream);
 
 /* Adjoint (back-projection) c = A^T y: the transpose of the matrix of Eq. 6,
- * matched exactly to spl_forward (Sec. 2.3): it visits the same
- * (ray, basis) pairs and evaluates bit-identical footprint values.  View
+ * matched to spl_forward (Sec. 2.3): the exact footprint of every (ray,
+ * basis) pair of Eq. 4, integrated over the same pieces (the two agree to
+ * FP32 rounding; the footprint form of spl_forward evaluates bit-identical
+ * values).  View
  * geometries use the form chosen by basis->adjoint (SPL_ADJ_*): a
  * ray-driven scatter with float atomics (the default) or a gather over
  * coefficient bricks that loops over views and the detector window of the

@@ -520,6 +520,7 @@ extern "C" spl_status spl_make_geometry(const spl_geometry_desc *desc, spl_geome
             }
         }
     }
+    line_create(g, d.ray_omega);
     *out = g;
     return SPL_OK;
 }
@@ -529,6 +530,7 @@ extern "C" void spl_destroy_geometry(spl_geometry *g)
     if (!g) return;
     plane_free(g->plane);
     table_free(g->table);
+    line_free(g->line);
     free(g->vconst);
     if (g->acc64) cudaFree(g->acc64);
     for (int L = 0; L < 3; ++L)

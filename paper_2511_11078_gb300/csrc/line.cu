@@ -1,0 +1,662 @@
+// line.cu -- forward projection A as line integrals of f itself (Eq. 2), on
+// coefficients resampled once per call into the power basis of the rays'
+// dominant axis.
+//
+// f = sum_k c_k phi(x - k) is, on every cell [c, c+1) of axis d (v = u + W,
+// the cells of the cell march), a polynomial in the position along d for
+// each pair of transverse indices (la, lb):
+//   sum_{l_d} c(l_d, la, lb) beta^n(v_d - W - l_d) = sum_j p_j(c, la, lb) tau^j,
+// tau = v_d - c - 1/2 in [-1/2, 1/2].  k_line_resample writes p_0 .. p_n of
+// every cell and column as one float4 (float2 for n = 1).  A ray is cut into
+// the pieces of the piece march (spl_march.cuh: cells along its dominant
+// axis, split at the knot planes of the other two, r <= 1) and each piece is
+// integrated with the same Gauss-Legendre rule; a node needs two weight sets
+// instead of three and contracts (n+1)^2 columns:
+//   f(tau) = sum_i wa_i sum_k wb_k (p_0 + p_2 tau^2 + tau (p_1 + p_3 tau^2)),
+// the even and the odd part as one packed FP32x2 value (n = 1: the two
+// coefficients with weights 1/2 -+ tau).
+//
+// The footprint form (march in spl_march.cuh) carries an (n+1)^3 register
+// window that an event shifts by selects and flushes face by face; that is
+// half of its instructions, and it must keep the adjoint's order.  Here a
+// piece loads its (n+1)^2 columns afresh, always as aligned 16-byte vectors
+// (neighbouring lanes and successive pieces share them in L1), so there is
+// no window to shift, no face to pick, and a piece does not depend on the
+// one before: pieces of one ray may be walked by several threads.
+#include <math.h>
+
+#include <mutex>
+#include <new>
+
+#include "spl_host.h"
+
+namespace spl {
+
+// The transverse axes of dominant axis d: p (rows) and q (contiguous).  q is
+// z where it can be: the detector columns of tilt series and of circular and
+// helical orbits about z run along it, and eight lanes along q then load one
+// run of columns (see line_lanes_along_v).
+__host__ __device__ constexpr int line_p(int d) { return d == 1 ? 0 : 1; }
+__host__ __device__ constexpr int line_q(int d) { return d == 2 ? 0 : 2; }
+
+// (selects: a run-time index would put the array into local memory)
+template <class T> __host__ __device__ inline T sel3(int i, const T &a, const T &b, const T &c)
+{
+    return i == 0 ? a : (i == 1 ? b : c);
+}
+
+// Resampled array of axis d at degree n: cells c = 0 .. n_d + n - 1, columns
+// padded by n zeros on every side (a piece's window then never leaves the
+// array).  The row stride is 3 vectors above a multiple of 8: lanes of a
+// warp that sit in neighbouring rows or cells then load from different banks
+// (8 helical views 51.3 ms with rows on 128-byte boundaries, 49.7 with 3; 64
+// general parallel views 5.72 and 4.99 ms).
+struct LineDims {
+    int nd, np, nq;
+};
+__host__ __device__ inline LineDims line_dims(const int (&n)[3], int d, int degree)
+{
+    LineDims L;
+    L.nd = sel3(d, n[0], n[1], n[2]) + degree;
+    L.np = sel3(line_p(d), n[0], n[1], n[2]) + 2 * degree;
+    L.nq = (sel3(line_q(d), n[0], n[1], n[2]) + 2 * degree + 7) / 8 * 8 + 3;
+    return L;
+}
+
+template <int N> struct LineVec { using T = float4; };
+template <> struct LineVec<1> { using T = float2; };
+
+struct LineArrays {
+    void *a[3];  // per dominant axis, NULL where no ray has it
+};
+
+// ---------------------------------------------------------------- resampling
+template <int N>
+__device__ __forceinline__ typename LineVec<N>::T line_poly(const float (&c)[N + 1])
+{
+    if constexpr (N == 1) {
+        // the two coefficients themselves: weights 1/2 - tau, 1/2 + tau
+        return make_float2(c[0], c[1]);
+    } else if constexpr (N == 2) {
+        return make_float4(0.125f * ((c[0] + c[2]) + 6.0f * c[1]), 0.5f * (c[2] - c[0]),
+                           0.5f * ((c[0] - c[1]) - (c[1] - c[2])), 0.0f);
+    } else {
+        const float so = c[0] + c[3], si = c[1] + c[2], dq = c[3] - c[0], di = c[2] - c[1];
+        // (divisions: 1/48 and 1/6 rounded to FP32 would scale every value by 1 + 2e-8, 1 + 3e-8)
+        return make_float4(__fdiv_rn(fmaf(23.0f, si, so), 48.0f), 0.125f * fmaf(5.0f, di, dq), 0.25f * (so - si),
+                           __fdiv_rn(fmaf(-3.0f, di, dq), 6.0f));
+    }
+}
+
+// One thread per column (ip, iq) and chunk of kLineChunk cells, sliding
+// along d: one load per cell.  blockIdx.z: (axis, chunk).
+constexpr int kLineChunk = 32;
+template <int N>
+__global__ void __launch_bounds__(256) k_line_resample(DevGeom g, const float *__restrict__ c, LineArrays out, int3 zc)
+{
+    int d = 0, z = blockIdx.z;
+    if (z >= zc.x) {
+        z -= zc.x;
+        d = 1;
+        if (z >= zc.y) {
+            z -= zc.y;
+            d = 2;
+        }
+    }
+    const LineDims L = line_dims(g.n, d, N);
+    const int iq = blockIdx.x * 32 + (threadIdx.x & 31), ip = blockIdx.y * 8 + (threadIdx.x >> 5);
+    const int c0 = z * kLineChunk;
+    if (iq >= L.nq || ip >= L.np || c0 >= L.nd) return;
+    const long long sy = g.n[0], sz = (long long)g.n[0] * g.n[1];
+    const int nd = L.nd - N, np = L.np - 2 * N, nq = sel3(line_q(d), g.n[0], g.n[1], g.n[2]);
+    auto stride = [&](int e) { return e == 0 ? 1LL : (e == 1 ? sy : sz); };
+    const long long sd = stride(d), sp = stride(line_p(d)), sq = stride(line_q(d));
+    const bool in = ip >= N && ip - N < np && iq >= N && iq - N < nq;
+    const float *src = c + (in ? (ip - N) * sp + (iq - N) * sq : 0);
+    typename LineVec<N>::T *o =
+        reinterpret_cast<typename LineVec<N>::T *>(d == 0 ? out.a[0] : (d == 1 ? out.a[1] : out.a[2])) +
+        ((long long)c0 * L.np + ip) * L.nq + iq;
+    const long long so = (long long)L.np * L.nq;
+    float w[N + 1];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int l = c0 - N + i;  // cell c0 holds l = c0 - N .. c0
+        w[i + 1] = in && l >= 0 && l < nd ? __ldg(src + l * sd) : 0.0f;
+    }
+    const int c1 = min(c0 + kLineChunk, L.nd);
+#pragma unroll 4
+    for (int cc = c0; cc < c1; ++cc) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) w[i] = w[i + 1];
+        w[N] = in && cc < nd ? __ldg(src + cc * sd) : 0.0f;
+        *o = line_poly<N>(w);
+        o += so;
+    }
+}
+
+// ---------------------------------------------------------------- ray set-up
+// Transverse coordinates are carried as 64-bit fixed point with kLineFrac
+// fraction bits: the start is exact to 2^-41 and the step is off by at most
+// 2^-41 per cell, 2^-30 over the longest ray, so a cell's fraction is its
+// FP32 rounding everywhere on the ray, for one 64-bit add per cell.
+constexpr int kLineFrac = 40;
+
+// A ray, in shared memory: set up by one thread, read by the 2^ls threads
+// that share it.
+struct __align__(16) LineRay {
+    long long A, B;           // v_p, v_q at the start of cell c
+    long long RA, RB;         // and their steps
+    float ia, ib;             // reciprocals of ra, rb
+    float ea, eb;             // the fraction at which the ray leaves its cell: 1 (r > 0), 0 (r < 0)
+    float ra, rb;             // steps per cell
+    float scale, scale_lo;    // 1 / |w_d| as a sum of two floats
+    int d, c, cl, pad;        // dominant axis, first and last cell (none: c > cl)
+};
+
+// The FP32 constants 2/3 and 1/6 of the cubic weights (bweights<3>) are
+// 1.987e-8 and 4.97e-9 too large, so the four weights of an axis sum to
+// 1 + 2 (1.987e-8) + 4.97e-9 (g^3 + t^3), on average 1 + 4.22e-8, and every
+// integral over two axes comes out 8.44e-8 too large.  The ray's scale takes
+// that out (it was most of the error against FP64).
+template <int N> __device__ __forceinline__ constexpr float line_excess() { return N == 3 ? 8.44e-8f : 0.0f; }
+
+// The line {s + t w} (w of any length).  The two orientations of a line are
+// the same line: w_d > 0 is implied by dividing by w_d, and the transverse
+// steps keep their signs.  FP64, about 45 operations; GB300 has 1/64 of the
+// FP32 rate for them, so a ray is set up once for all its threads.  L comes
+// with an empty cell range and keeps it when the line meets no support.
+template <int N>
+__device__ __forceinline__ void line_setup(const DevGeom &g, const double (&s)[3], const double (&w)[3], LineRay &L)
+{
+    constexpr double W = 0.5 * (N + 1);
+    int d = 0;
+    if (fabs(w[1]) > fabs(w[d])) d = 1;
+    if (fabs(w[2]) > fabs(w[d])) d = 2;
+    L.d = d;
+    // p and q by selects (no local-memory indexing)
+    const int ap = line_p(d), aq = line_q(d);
+    const double u0 = s[0] - g.org[0], u1 = s[1] - g.org[1], u2 = s[2] - g.org[2];
+    const double wd = sel3(d, w[0], w[1], w[2]), wp = sel3(ap, w[0], w[1], w[2]), wq = sel3(aq, w[0], w[1], w[2]);
+    const double sd = sel3(d, u0, u1, u2), sp = sel3(ap, u0, u1, u2), sq = sel3(aq, u0, u1, u2);
+    const int nd = sel3(d, g.n[0], g.n[1], g.n[2]), np = sel3(ap, g.n[0], g.n[1], g.n[2]),
+              nq = sel3(aq, g.n[0], g.n[1], g.n[2]);
+    const double iw = 1.0 / wd;
+    double ra = wp * iw, rb = wq * iw;
+    // steps below 1e-30 move nothing over 2048 cells
+    if (fabs(ra) < 1e-30) ra = 0.0;
+    if (fabs(rb) < 1e-30) rb = 0.0;
+    // |w| / |w_d| = sqrt(1 + ra^2 + rb^2): the FP32 root and its correction
+    // from the FP64 residual
+    const double q2 = fma(ra, ra, fma(rb, rb, 1.0));
+    L.scale = sqrtf((float)q2);
+    L.scale_lo = fmaf(-line_excess<N>(), L.scale, (float)fma(-(double)L.scale, (double)L.scale, q2) * (0.5f / L.scale));
+    // transverse coordinates at v_d = 0
+    const double a0 = fma(-(W + sd), ra, sp) + W, b0 = fma(-(W + sd), rb, sq) + W;
+    L.ra = (float)ra;
+    L.rb = (float)rb;
+    // an axis that the ray does not move along: crossing at 3 - fraction, never inside a cell
+    L.ia = ra != 0.0 ? 1.0f / L.ra : 1.0f;
+    L.ib = rb != 0.0 ? 1.0f / L.rb : 1.0f;
+    L.ea = ra != 0.0 ? (ra > 0.0 ? 1.0f : 0.0f) : 3.0f;
+    L.eb = rb != 0.0 ? (rb > 0.0 ? 1.0f : 0.0f) : 3.0f;
+    // cells whose window can hold a basis: v_p in (0, n_p + N), v_q in
+    // (0, n_q + N); one cell of margin (the bounds are FP32 quotients)
+    float vmin = 0.0f, vmax = (float)(nd + N);
+    if (ra != 0.0) {
+        const float t0 = (float)(0.0 - a0) * L.ia, t1 = (float)((double)(np + N) - a0) * L.ia;
+        vmin = fmaxf(vmin, fminf(t0, t1));
+        vmax = fminf(vmax, fmaxf(t0, t1));
+    } else if (!(a0 > 0.0 && a0 < (double)(np + N))) {
+        return;
+    }
+    if (rb != 0.0) {
+        const float t0 = (float)(0.0 - b0) * L.ib, t1 = (float)((double)(nq + N) - b0) * L.ib;
+        vmin = fmaxf(vmin, fminf(t0, t1));
+        vmax = fminf(vmax, fmaxf(t0, t1));
+    } else if (!(b0 > 0.0 && b0 < (double)(nq + N))) {
+        return;
+    }
+    if (!(vmax >= vmin - 1.0f)) return;
+    const int c = max((int)floorf(vmin) - 1, 0);
+    L.c = c;
+    L.cl = min((int)floorf(vmax) + 1, nd + N - 1);
+    constexpr double kOne = (double)(1LL << kLineFrac);
+    L.RA = __double2ll_rn(ra * kOne);
+    L.RB = __double2ll_rn(rb * kOne);
+    L.A = __double2ll_rn(fma((double)c, ra, a0) * kOne);
+    L.B = __double2ll_rn(fma((double)c, rb, b0) * kOne);
+}
+
+// 16 bytes of a ray, not to be kept in registers: next to 64 column values
+// the cubic march has none for the constants that only its events need (with
+// them in registers it spills: 8 helical views 51.9 ms, 49.5 without), so
+// the load is volatile and stays in the loop.
+__device__ __forceinline__ uint4 lds128(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+    return v;
+}
+
+// ---------------------------------------------------------------- the march
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+
+// Integral of f over part `seg` of 2^ls equal parts of the cells of L, in
+// units of the d axis (times scale outside), as the FP32 sum over the pieces
+// and its Kahan compensation (the integral is sum - comp).  Returns false if
+// the event bound was reached.
+template <int N>
+__device__ __forceinline__ bool line_march(const LineRay &L, int seg, int ls, const LineArrays &arr, const int (&n)[3],
+                                           const QuadRule &qr, bool kahan, float &sum, float &comp)
+{
+    using V = typename LineVec<N>::T;
+    constexpr int M = GL<N>::M;
+    constexpr bool KEEP = N < 3;  // the events' constants in registers
+    sum = comp = 0.0f;
+    const int cells = L.cl - L.c + 1, k0 = (int)(((long long)cells * seg) >> ls),
+              k1 = (int)(((long long)cells * (seg + 1)) >> ls);
+    if (k0 >= k1) return true;
+    const int d = L.d;
+    long long A = L.A + L.RA * k0, B = L.B + L.RB * k0;
+    int left = k1 - k0;  // cells to go
+    const float ra = L.ra, rb = L.rb;
+    const LineDims D = line_dims(n, d, N);
+    const V *__restrict__ P = reinterpret_cast<const V *>(sel3(d, arr.a[0], arr.a[1], arr.a[2]));
+    if (!P) return false;  // an axis that line_axes ruled out (not expected)
+    const unsigned lim_p = (unsigned)(D.np - N), lim_q = (unsigned)(sel3(line_q(d), n[0], n[1], n[2]) + N);
+    const size_t slab = (size_t)D.np * D.nq;
+    const V *row = P + (size_t)(L.c + k0) * slab;
+    uint4 kr, ke;
+    if (KEEP) {
+        kr = lds128(&L.RA);
+        ke = lds128(&L.ia);
+    }
+    int QA, QB;
+    float ga, gb, ta, tb, t0;
+    // position in the cell: column (QA, QB) and the fractions at the cell's
+    // middle (tau = 0); ta, tb: tau of the crossings (beyond 1/2: none)
+    auto cell = [&]() {
+        constexpr float kUnit = 1.0f / 4294967296.0f;
+        QA = (int)(A >> kLineFrac);
+        QB = (int)(B >> kLineFrac);
+        ga = fmaf(0.5f, ra, __uint2float_rn((unsigned)(A >> (kLineFrac - 32))) * kUnit);
+        gb = fmaf(0.5f, rb, __uint2float_rn((unsigned)(B >> (kLineFrac - 32))) * kUnit);
+        const uint4 e = KEEP ? ke : lds128(&L.ia);
+        ta = (__uint_as_float(e.z) - ga) * __uint_as_float(e.x);
+        tb = (__uint_as_float(e.w) - gb) * __uint_as_float(e.y);
+        t0 = -0.5f;
+    };
+    cell();
+    int ev = 0;
+#pragma unroll 1
+    while (true) {
+        const float t1 = fminf(fminf(ta, tb), 0.5f);
+        if (t1 > t0 && (unsigned)QA < lim_p && (unsigned)QB < lim_q) {
+            const float half = 0.5f * (t1 - t0), mid = 0.5f * (t0 + t1);
+            V col[N + 1][N + 1];
+            const V *r = row + ((unsigned)QA * (unsigned)D.nq + (unsigned)QB);
+#pragma unroll
+            for (int i = 0; i <= N; ++i)
+#pragma unroll
+                for (int k = 0; k <= N; ++k) col[i][k] = __ldg(r + (size_t)i * D.nq + k);
+            float2 S = make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int q = 0; q < M; ++q) {
+                const float tau = fmaf(half, qr.x[q], mid);
+                float wa[N + 1], wb[N + 1];
+                bweights<N>(fmaf(ra, tau, ga), wa);
+                bweights<N>(fmaf(rb, tau, gb), wb);
+                const float2 t2 = dup(tau * tau);
+                float2 h = make_float2(0.0f, 0.0f);
+#pragma unroll
+                for (int i = 0; i <= N; ++i) {
+                    float2 gk;
+#pragma unroll
+                    for (int k = 0; k <= N; ++k) {
+                        float2 e;
+                        if constexpr (N == 3)
+                            e = __ffma2_rn(make_float2(col[i][k].z, col[i][k].w), t2,
+                                           make_float2(col[i][k].x, col[i][k].y));
+                        else if constexpr (N == 2)
+                            e = make_float2(fmaf(col[i][k].z, t2.x, col[i][k].x), col[i][k].y);
+                        else
+                            e = make_float2(col[i][k].x, col[i][k].y);
+                        gk = k == 0 ? __fmul2_rn(dup(wb[0]), e) : __ffma2_rn(dup(wb[k]), e, gk);
+                    }
+                    h = i == 0 ? __fmul2_rn(dup(wa[0]), gk) : __ffma2_rn(dup(wa[i]), gk, h);
+                }
+                if constexpr (N == 1) S = __ffma2_rn(make_float2(qr.w[q] * (0.5f - tau), qr.w[q] * (0.5f + tau)), h, S);
+                else S = __ffma2_rn(make_float2(qr.w[q], qr.w[q] * tau), h, S);
+            }
+            const float v = half * (S.x + S.y);
+            if (kahan) kahan_add(sum, comp, v);
+            else sum += v;
+        }
+        t0 = fmaxf(t0, t1);
+        if (++ev > qr.cap) return false;
+        const bool evA = ta <= tb && ta < 0.5f, evB = !evA && tb < 0.5f;
+        if (evA || evB) {
+            // the column's neighbour along the crossed axis, once per cell
+            const int step = (evA ? ra : rb) > 0.0f ? 1 : -1;
+            QA += evA ? step : 0;
+            ga -= evA ? (float)step : 0.0f;
+            ta = evA ? 2.0f : ta;
+            QB += evB ? step : 0;
+            gb -= evB ? (float)step : 0.0f;
+            tb = evB ? 2.0f : tb;
+        } else {
+            if (--left == 0) break;
+            const uint4 e = KEEP ? kr : lds128(&L.RA);
+            A += (long long)(((unsigned long long)e.y << 32) | e.x);
+            B += (long long)(((unsigned long long)e.w << 32) | e.z);
+            row += slab;
+            cell();
+            ev = 0;
+        }
+    }
+    return true;
+}
+
+// ---------------------------------------------------------------- kernels
+// blocks per SM the registers are sized for
+template <int N> struct LineBlocks { static constexpr int value = N == 3 ? 4 : (N == 2 ? 5 : 8); };
+
+// The value of thread (seg, ray p of the block): the march over its share of
+// the ray's cells, and the sum of the ray's 2^ls shares (adjacent lanes; every
+// lane of the warp calls this).  The shares and the scale are carried as
+// float pairs and rounded once at the end: rounded one by one they would
+// cost as much accuracy as the march itself (5.1e-8 against 2.8e-8).
+template <int N>
+__device__ __forceinline__ float line_value(const DevGeom &g, const LineRay &L, const LineArrays &arr,
+                                            const QuadRule &qr, int kahan, int seg, int ls)
+{
+    float hi, lo;
+    if (!line_march<N>(L, seg, ls, arr, g.n, qr, kahan != 0, hi, lo)) atomicOr(g.err, 1);
+    lo = -lo;
+    for (int o = 1; o < (1 << ls); o <<= 1) {
+        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float s = __fadd_rn(hi, h2), bb = __fsub_rn(s, hi);  // TwoSum
+        lo += l2 + __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(h2, bb));
+        hi = s;
+    }
+    const float p = __fmul_rn(hi, L.scale);
+    return p + fmaf(hi, L.scale_lo, fmaf(lo, L.scale, fmaf(hi, L.scale, -p)));
+}
+
+// Whether a warp's eight consecutive lanes run along detector v (4 x 8
+// pixels) or u (8 x 4): along the axis that moves more along q, so that they
+// load one run of columns (8 cone views 7.9 ms against 6.5 the other way
+// round, 8 helical views 99 against 51).  Decided for the view's central ray.
+__device__ __forceinline__ bool line_lanes_along_v(const DevGeom &g, const ViewPose &P)
+{
+    float w[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) w[e] = fabsf((float)(g.kind == SPL_PARALLEL ? P.src[e] : P.dc[e] - P.src[e]));
+    const int d = w[1] > w[0] ? (w[2] > w[1] ? 2 : 1) : (w[2] > w[0] ? 2 : 0);
+    const int q = line_q(d);
+    return fabs(q == 2 ? P.dv[2] : P.dv[0]) >= fabs(q == 2 ? P.du[2] : P.du[0]);
+}
+
+// view geometries: view blockIdx.z (of order[], when given); the block's 128
+// >> ls pixels form a tile of 16 x 8, 8 x 8, 8 x 4 or 4 x 4
+template <int N>
+__global__ void __launch_bounds__(128, LineBlocks<N>::value)
+    k_line_views(DevGeom g, LineArrays arr, float *__restrict__ y, QuadRule qr, int kahan, const int *order, int ls)
+{
+    const int seg = threadIdx.x & ((1 << ls) - 1), p = threadIdx.x >> ls;
+    const int lane = p & 31, wid = p >> 5;
+    const int k = order ? order[blockIdx.z] : (int)blockIdx.z;
+    int iu, iv;
+    if (ls == 0) {
+        if (line_lanes_along_v(g, g.views[k])) {
+            iu = blockIdx.x * 16 + wid * 4 + (lane >> 3);
+            iv = blockIdx.y * 8 + (lane & 7);
+        } else {
+            iu = blockIdx.x * 16 + (wid & 1) * 8 + (lane & 7);
+            iv = blockIdx.y * 8 + (wid >> 1) * 4 + (lane >> 3);
+        }
+    } else {
+        // tile of 8 x 8, 8 x 4, 4 x 4
+        const int lw = ls == 3 ? 2 : 3;
+        iu = (blockIdx.x << lw) + (p & ((1 << lw) - 1));
+        iv = blockIdx.y * (ls == 1 ? 8 : 4) + (p >> lw);
+    }
+    __shared__ LineRay rays[128];
+    auto setup = [&](LineRay &L, int u, int v) {
+        L.c = 0;
+        L.cl = -1;
+        if (u >= g.nu || v >= g.nv) return;  // beyond the detector
+        const ViewPose &P = g.views[k];
+        const double a = u - 0.5 * (g.nu - 1), b = v - 0.5 * (g.nv - 1);
+        double s[3], w[3];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const double q = fma(b, P.dv[e], fma(a, P.du[e], P.dc[e])), src = P.src[e];
+            s[e] = q;
+            w[e] = g.kind == SPL_PARALLEL ? src : q - src;
+        }
+        line_setup<N>(g, s, w, L);
+    };
+    if (ls == 0) {
+        setup(rays[p], iu, iv);
+        __syncwarp();
+    } else {
+        // thread t sets up ray t of the block
+        const int t = threadIdx.x, lw = ls == 3 ? 2 : 3;
+        if (t < (128 >> ls))
+            setup(rays[t], (blockIdx.x << lw) + (t & ((1 << lw) - 1)), blockIdx.y * (ls == 1 ? 8 : 4) + (t >> lw));
+        __syncthreads();
+    }
+    const bool in = iu < g.nu && iv < g.nv;
+    const float v = line_value<N>(g, rays[p], arr, qr, kahan, seg, ls);
+    if (seg == 0 && in) y[((long long)k * g.nv + iv) * g.nu + iu] = v;
+}
+
+template <int N>
+__global__ void __launch_bounds__(128, LineBlocks<N>::value)
+    k_line_rays(DevGeom g, LineArrays arr, float *__restrict__ y, QuadRule qr, int kahan, int ls)
+{
+    __shared__ LineRay rays[128];
+    const long long r0 = ((long long)blockIdx.x * 128) >> ls;
+    const int t = threadIdx.x, p = t >> ls, seg = t & ((1 << ls) - 1);
+    if (t < (128 >> ls)) {
+        rays[t].c = 0;
+        rays[t].cl = -1;
+        if (r0 + t < g.n_rays) {
+            double s[3], w[3];
+            explicit_ray(g, r0 + t, s, w);
+            line_setup<N>(g, s, w, rays[t]);
+        }
+    }
+    __syncthreads();
+    const float v = line_value<N>(g, rays[p], arr, qr, kahan, seg, ls);
+    if (seg == 0 && r0 + p < g.n_rays) y[r0 + p] = v;
+}
+
+// ---------------------------------------------------------------- host side
+// The resampled arrays of a geometry.  Calls on one geometry from several
+// streams or threads take turns on them: each call makes its stream wait for
+// the previous one's event, under the mutex.
+struct LineScratch {
+    LineArrays arr;
+    void *block;
+    cudaEvent_t last;
+    bool used;
+    std::mutex mu;
+};
+
+// Where the resampled form is the faster one (both sides measured on GB300):
+//  * the arrays are written once per call, 4.7e-12 s a vector, and a piece of
+//    a view's ray costs 2.9e-11 s in the footprint form and 1.9e-11 s here:
+//    it pays from half a piece per vector on, and a ray crosses about half of
+//    nx + ny + nz cells (20 000 rays through 256^3: 1.46 against 1.22 ms, two
+//    views of 395 x 263 through 293 x 335 x 320: 2.47 against 3.07);
+//  * explicit rays need not lie side by side, and then every lane loads its
+//    own 32-byte sectors: the arrays have to stay mostly in the L2 (300 000
+//    random rays, cubic, 192^3 = 365 MB: 4.6 against 6.0 ms; 256^3 = 850 MB:
+//    12.6 against 7.6; quadratic 192^3: 2.97 against 2.94);
+//  * all three axes of a 512^3 grid take 6.7 GB; beyond 24 GB the scratch is
+//    out of proportion.
+constexpr size_t kLineMaxBytes = (size_t)24 << 30;
+constexpr size_t kLineMaxBytesRays = (size_t)320 << 20;
+
+// Axes that can be the dominant one of a line of the geometry (a superset):
+// |w_e| over a view's pixels lies between bounds taken at its corners, since
+// a pixel's direction is affine in (u, v).
+static unsigned line_axes(const spl_geometry *g, const double *raw_rays)
+{
+    const DevGeom &dg = g->dev;
+    unsigned mask = 0;
+    auto add = [&](const double (&lo)[3], const double (&hi)[3]) {
+        for (int e = 0; e < 3; ++e) {
+            bool can = true;
+            for (int f = 0; f < 3; ++f) can = can && hi[e] * (1.0 + 1e-9) >= lo[f];
+            if (can) mask |= 1u << e;
+        }
+    };
+    if (dg.kind == SPL_RAYS) {
+        for (long long r = 0; r < dg.n_rays && mask != 7u; ++r) {
+            double m[3];
+            for (int e = 0; e < 3; ++e) m[e] = fabs(raw_rays[3 * r + e]);
+            add(m, m);
+        }
+        return mask;
+    }
+    for (int k = 0; k < dg.n_views && mask != 7u; ++k) {
+        const ViewPose &P = g->views_host[k];
+        double lo[3], hi[3];
+        for (int e = 0; e < 3; ++e) {
+            double mn = INFINITY, mx = -INFINITY;
+            for (int corner = 0; corner < 4; ++corner) {
+                const double a = ((corner & 1) ? 0.5 : -0.5) * (dg.nu - 1), b = ((corner & 2) ? 0.5 : -0.5) * (dg.nv - 1);
+                const double v = dg.kind == SPL_PARALLEL ? P.src[e] : P.dc[e] + a * P.du[e] + b * P.dv[e] - P.src[e];
+                mn = fmin(mn, v);
+                mx = fmax(mx, v);
+            }
+            lo[e] = mn <= 0.0 && mx >= 0.0 ? 0.0 : fmin(fabs(mn), fabs(mx)) * (1.0 - 1e-9);
+            hi[e] = fmax(fabs(mn), fabs(mx));
+        }
+        add(lo, hi);
+    }
+    return mask;
+}
+
+void line_create(spl_geometry *g, const double *ray_dirs)
+{
+    const DevGeom &dg = g->dev;
+    g->line = nullptr;
+    // parallel views of the flat class take the plane matrices or the flat march
+    if (dg.n_rays == 0 || (dg.kind == SPL_PARALLEL && dg.n_flat == dg.n_views)) return;
+    const unsigned mask = line_axes(g, ray_dirs);
+    size_t off[3], total = 0;
+    for (int d = 0; d < 3; ++d) {
+        off[d] = total;
+        if (!((mask >> d) & 1u)) continue;
+        // sized for cubic splines, the largest
+        const LineDims L = line_dims(dg.n, d, 3);
+        total += ((size_t)L.nd * L.np * L.nq * sizeof(float4) + 255) & ~(size_t)255;
+    }
+    if (total == 0 || total > (dg.kind == SPL_RAYS ? kLineMaxBytesRays : kLineMaxBytes)) return;
+    const long long marched = dg.kind == SPL_PARALLEL ? (long long)(dg.n_views - dg.n_flat) * dg.nu * dg.nv : dg.n_rays;
+    if ((double)marched * (dg.n[0] + dg.n[1] + dg.n[2]) < (double)(total / sizeof(float4))) return;
+    LineScratch *ls = new (std::nothrow) LineScratch();
+    if (!ls) return;
+    if (cudaMalloc(&ls->block, total) != cudaSuccess) {
+        cudaGetLastError();
+        delete ls;
+        return;
+    }
+    if (cudaEventCreateWithFlags(&ls->last, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(ls->block);
+        delete ls;
+        return;
+    }
+    ls->used = false;
+    for (int d = 0; d < 3; ++d) ls->arr.a[d] = ((mask >> d) & 1u) ? (char *)ls->block + off[d] : nullptr;
+    g->line = ls;
+}
+
+void line_free(LineScratch *ls)
+{
+    if (!ls) return;
+    cudaEventDestroy(ls->last);
+    cudaFree(ls->block);
+    delete ls;
+}
+
+bool line_usable(const spl_geometry *g, int degree, cudaStream_t st)
+{
+    if (!g->line || degree < 1) return false;
+    // a captured call cannot take its turn against calls outside the graph
+    // (an event of the one cannot be waited for in the other): it keeps the
+    // footprint form, which has no scratch
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cap == cudaStreamCaptureStatusNone;
+}
+
+// Threads per ray, 2^ls: the fewest that give every SM its resident threads,
+// at most 8 (a thread keeps at least a few cells of the ray).
+static int line_split(long long rays, int blocks_per_sm)
+{
+    const long long fill = (long long)sm_count() * blocks_per_sm * 128;
+    int ls = 0;
+    while (ls < 3 && (rays << ls) < fill) ++ls;
+    return ls;
+}
+
+template <int N>
+static spl_status line_forward_n(const spl_geometry *g, int kahan, const float *c, float *y, cudaStream_t st)
+{
+    const DevGeom &dg = g->dev;
+    LineScratch &S = *g->line;
+    const QuadRule qr = quad_rule(N);
+    std::lock_guard<std::mutex> lock(S.mu);
+    spl_status s = SPL_OK;
+    if (S.used) s = cuda_check(cudaStreamWaitEvent(st, S.last, 0), "line scratch wait");
+    if (s != SPL_OK) return s;
+    int gx = 0, gy = 0, zc[3];
+    for (int d = 0; d < 3; ++d) {
+        zc[d] = 0;
+        if (!S.arr.a[d]) continue;
+        const LineDims L = line_dims(dg.n, d, N);
+        zc[d] = (L.nd + kLineChunk - 1) / kLineChunk;
+        gx = (L.nq + 31) / 32 > gx ? (L.nq + 31) / 32 : gx;
+        gy = (L.np + 7) / 8 > gy ? (L.np + 7) / 8 : gy;
+    }
+    k_line_resample<N><<<dim3(gx, gy, zc[0] + zc[1] + zc[2]), 256, 0, st>>>(dg, c, S.arr, make_int3(zc[0], zc[1], zc[2]));
+    if (dg.kind == SPL_RAYS) {
+        const int ls = line_split(dg.n_rays, LineBlocks<N>::value);
+        const long long blocks = ((dg.n_rays << ls) + 127) / 128;
+        k_line_rays<N><<<(unsigned)blocks, 128, 0, st>>>(dg, S.arr, y, qr, kahan, ls);
+    } else {
+        const int v0 = dg.kind == SPL_PARALLEL ? dg.n_flat : 0, nview = dg.n_views - v0;
+        const int *order = dg.kind == SPL_PARALLEL ? dg.view_order + v0 : nullptr;
+        const int ls = line_split((long long)nview * dg.nu * dg.nv, LineBlocks<N>::value);
+        const int tw = ls == 0 ? 16 : (ls == 3 ? 4 : 8), th = ls < 2 ? 8 : 4;
+        const dim3 grid((dg.nu + tw - 1) / tw, (dg.nv + th - 1) / th, nview);
+        k_line_views<N><<<grid, 128, 0, st>>>(dg, S.arr, y, qr, kahan, order, ls);
+    }
+    s = cuda_check(cudaGetLastError(), "line forward launch");
+    // recorded also after a failed launch: what did start still uses the scratch
+    const spl_status e = cuda_check(cudaEventRecord(S.last, st), "line scratch record");
+    S.used = true;
+    return s != SPL_OK ? s : e;
+}
+
+spl_status line_forward(const spl_geometry *g, int degree, int kahan, const float *c, float *y, cudaStream_t st)
+{
+    switch (degree) {
+    case 1: return line_forward_n<1>(g, kahan, c, y, st);
+    case 2: return line_forward_n<2>(g, kahan, c, y, st);
+    default: return line_forward_n<3>(g, kahan, c, y, st);
+    }
+}
+
+}  // namespace spl

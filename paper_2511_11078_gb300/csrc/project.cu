@@ -777,6 +777,8 @@ static spl_status forward_quad_t(const spl_geometry *g, const spl_basis_desc *b,
     const QuadRule qr = quad_rule(N);
     const int kahan = b->kahan;
     if (dg.n_rays == 0) return SPL_OK;
+    const bool line = line_usable(g, N, st);
+    if (line && dg.kind != SPL_PARALLEL) return line_forward(g, N, kahan, c, y, st);
     if (dg.kind == SPL_RAYS) {
         const long long blocks = (dg.n_rays + 127) / 128;
         k_forward_rays<N, DIRECT><<<(unsigned)blocks, 128, 0, st>>>(dg, c, y, qr, kahan);
@@ -813,13 +815,15 @@ static spl_status forward_quad_t(const spl_geometry *g, const spl_basis_desc *b,
         for_view_chunks(g, v0, dg.n_flat - v0, [&](const ViewChunk &ch, int n) {
             k_forward_pviews<N, VM_FLAT, false><<<dim3(gx, gy, n), 128, 0, st>>>(dg, c, y, qr, kahan, ch);
         });
-        for_view_chunks(g, dg.n_flat, dg.n_views - dg.n_flat, [&](const ViewChunk &ch, int n) {
+        if (line) s = line_forward(g, N, kahan, c, y, st);
+        else for_view_chunks(g, dg.n_flat, dg.n_views - dg.n_flat, [&](const ViewChunk &ch, int n) {
             k_forward_pviews<N, VM_GENERAL, DIRECT><<<dim3(gx, gy, n), 128, 0, st>>>(dg, c, y, qr, kahan, ch);
         });
         if (overlap) {
-            s = cuda_check(cudaStreamWaitEvent(st, g->plane->join, 0), "join wait");
-            if (s != SPL_OK) return s;
+            const spl_status sj = cuda_check(cudaStreamWaitEvent(st, g->plane->join, 0), "join wait");
+            if (s == SPL_OK) s = sj;
         }
+        if (s != SPL_OK) return s;
     } else {
         dim3 grid((dg.nu + 15) / 16, (dg.nv + 7) / 8, dg.n_views);
         k_forward_views<N, DIRECT><<<grid, 128, 0, st>>>(dg, c, y, qr, kahan);

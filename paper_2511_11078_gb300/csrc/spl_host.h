@@ -10,6 +10,7 @@
 namespace spl {
 struct PlaneGroup;
 struct TableSet;
+struct LineScratch;
 }
 
 struct spl_geometry {
@@ -25,6 +26,7 @@ struct spl_geometry {
     float *lay[3];                // the scatter adjoint's targets: c in the x-fast [0], y-fast [1] and z-fast [2]
                                   // layouts, four copies each shifted by 0..3 floats (4 * dev.lay_cs floats),
                                   // or NULL (no rays; parallel geometries whose views are all flat)
+    spl::LineScratch *line;       // the forward's resampled coefficients (line.cu), or NULL (not needed or too large)
 };
 
 namespace spl {
@@ -125,5 +127,15 @@ spl_status table_build(spl_geometry *g, int degree, cudaStream_t st);
 spl_status table_forward(const spl_geometry *g, const spl_basis_desc *b, const float *c, float *y, cudaStream_t st);
 spl_status table_adjoint(const spl_geometry *g, const spl_basis_desc *b, const float *y, float *c, cudaStream_t st);
 void table_free(TableSet *ts);
+
+// The forward as line integrals of f on resampled coefficients (line.cu),
+// for explicit rays, cone views and the parallel views outside the flat
+// class.  line_create allocates its arrays with the geometry (leaves
+// g->line NULL when they are not needed, too large or not to be had);
+// line_usable: whether a call of this degree on this stream takes it.
+void line_create(spl_geometry *g, const double *ray_dirs);
+void line_free(LineScratch *ls);
+bool line_usable(const spl_geometry *g, int degree, cudaStream_t st);
+spl_status line_forward(const spl_geometry *g, int degree, int kahan, const float *c, float *y, cudaStream_t st);
 
 }  // namespace spl

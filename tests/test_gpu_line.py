@@ -1,0 +1,139 @@
+"""The forward on resampled coefficients (csrc/line.cu): the shapes at which
+its dispatch changes, against the FP64 oracle.
+
+Tolerance: a ray is a Kahan sum of at most ~90 pieces here, each a chain of
+about 4 + 4 + 4 + 5 roundings of 2^-24 on terms no larger than the window's
+absolute sum; with random signs that is about 17 * 2^-24 = 1e-6 of a piece
+and less of the sum, so the relative L2 error stays below 2e-6.
+"""
+import numpy as np
+import pytest
+
+from paper_2511_11078_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+TOL = 2e-6
+DIMS = (13, 21, 18)
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+
+    from paper_2511_11078_gb300 import build as B
+    from paper_2511_11078_gb300 import spl
+
+    B.build()
+    spl.lib()
+    return torch, spl
+
+
+def geom_of(orc, geo):
+    if geo.kind == "rays":
+        return orc.Geometry("rays", omega=geo.omega, s=geo.s)
+    key = "direction" if geo.kind == "parallel" else "source"
+    return orc.Geometry(geo.kind, det_center=geo.det_center, det_u=geo.det_u, det_v=geo.det_v, nu=geo.nu, nv=geo.nv,
+                        **{key: geo.src})
+
+
+def check(env, orc, geo, degree, seed, dims=DIMS):
+    torch, spl = env
+    rng = np.random.default_rng(seed)
+    origin = I.centred_origin(dims)
+    c = rng.normal(size=dims[::-1]).astype(np.float32)
+    g = spl.Geometry(dims, origin, geo)
+    y = torch.full((g.n_rays,), float("nan"), device="cuda")
+    spl.forward(g, torch.tensor(c, device="cuda"), y, spl.basis(degree))
+    g.status()
+    ref = orc.forward(degree, dims, origin, c.astype(np.float64), geom_of(orc, geo)).reshape(-1)
+    err = np.linalg.norm(y.cpu().numpy() - ref) / np.linalg.norm(ref)
+    assert err <= TOL, err
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+@pytest.mark.parametrize("rays", [700, 12001, 25000, 60000, 110001])
+def test_rays_per_split(env, orc, rays, degree):
+    """Explicit rays from too few to fill the GPU (8 threads a ray) to one
+    thread a ray, with short rays whose parts are empty."""
+    rng = np.random.default_rng(rays + degree)
+    w = I.random_directions(rng, rays)
+    w[::7, rng.integers(3)] = 0.0
+    w /= np.linalg.norm(w, axis=1, keepdims=True)
+    half = 0.5 * (np.asarray(DIMS) - 1.0)
+    s = rng.uniform(-1.15, 1.15, size=(rays, 3)) * half
+    check(env, orc, I.RayGeometry(w, s), degree, 10 + degree)
+
+
+@pytest.mark.parametrize("views", [1, 9, 21, 90])
+@pytest.mark.parametrize("turned", [False, True])
+@pytest.mark.parametrize("kind", ["parallel", "cone"])
+def test_views_per_split_and_lane_axis(env, orc, kind, turned, views):
+    """Views from 8 threads a ray to one, with detector columns along z and
+    (turned) detector rows along z: both lane directions of a warp."""
+    rng = np.random.default_rng(views)
+    nu, nv = 37, 33
+    if kind == "parallel":
+        geo = I.parallel_views(I.random_directions(rng, views), nu, nv, 0.8, center=(0.3, -0.2, 0.1))
+    else:
+        geo = I.helical_cone(views, 50.0, 80.0, nu, nv, 0.9, turns=1.3, table_feed=6.0)
+    if turned:
+        geo = I.ViewGeometry(geo.kind, geo.src, geo.det_center, geo.det_v, -geo.det_u, nu, nv)
+    check(env, orc, geo, 3, 20 + views)
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (2, 40, 3), (33, 2, 65)])
+def test_thin_grids(env, orc, dims):
+    """Grids thinner than a window and around the resampling's chunks."""
+    rng = np.random.default_rng(5)
+    w = I.random_directions(rng, 400)
+    s = rng.uniform(-0.6, 0.6, size=(400, 3)) * np.asarray(dims)
+    for degree in (1, 2, 3):
+        check(env, orc, I.RayGeometry(w, s), degree, 30 + degree, dims)
+
+
+def test_streams_take_turns(env):
+    """Forwards of one geometry on two streams share the resampled arrays:
+    each waits for the one before, and the results are those of calls in
+    line, bit for bit (the sums have a fixed order)."""
+    torch, spl = env
+    rng = np.random.default_rng(6)
+    g = spl.Geometry((64, 60, 56), I.centred_origin((64, 60, 56)),
+                     I.circular_cone(40, 200.0, 300.0, 96, 88, 1.2))
+    bas = spl.basis(3)
+    cs = [torch.tensor(rng.normal(size=(56, 60, 64)).astype(np.float32), device="cuda") for _ in range(2)]
+    ref = [torch.empty(g.n_rays, device="cuda") for _ in range(2)]
+    for c, y in zip(cs, ref):
+        spl.forward(g, c, y, bas)
+    torch.cuda.synchronize()
+    got = [[torch.empty(g.n_rays, device="cuda") for _ in range(4)] for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    for k in range(4):
+        for i in range(2):
+            spl.forward(g, cs[i], got[i][k], bas, stream=streams[i])
+    torch.cuda.synchronize()
+    g.status()
+    for i in range(2):
+        for y in got[i]:
+            assert torch.equal(y, ref[i])
+
+
+def test_captured_forward_matches(env):
+    """A captured forward keeps the footprint form (no scratch to share);
+    its replay agrees with the eager call to rounding."""
+    torch, spl = env
+    rng = np.random.default_rng(7)
+    dims = (30, 28, 26)
+    g = spl.Geometry(dims, I.centred_origin(dims), I.circular_cone(6, 100.0, 150.0, 40, 36, 1.2))
+    bas = spl.basis(3)
+    c = torch.tensor(rng.normal(size=dims[::-1]).astype(np.float32), device="cuda")
+    eager, replayed = (torch.full((g.n_rays,), float("nan"), device="cuda") for _ in range(2))
+    spl.forward(g, c, eager, bas)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        spl.forward(g, c, replayed, bas)
+    graph.replay()
+    torch.cuda.synchronize()
+    g.status()
+    assert float((eager - replayed).norm() / eager.norm()) <= TOL
