@@ -150,7 +150,8 @@ struct __align__(16) LineRay {
     float ea, eb;             // the fraction at which the ray leaves its cell: 1 (r > 0), 0 (r < 0)
     float ra, rb;             // steps per cell
     float scale, scale_lo;    // 1 / |w_d| as a sum of two floats
-    int d, c, cl, pad;        // dominant axis, first and last cell (none: c > cl)
+    int d, c, cl;             // dominant axis, first and last cell (none: c > cl)
+    float h4;                 // longest piece that four Gauss nodes integrate (cubic, line_short)
 };
 
 // The FP32 constants 2/3 and 1/6 of the cubic weights (bweights<3>) are
@@ -159,6 +160,27 @@ struct __align__(16) LineRay {
 // integral over two axes comes out 8.44e-8 too large.  The ray's scale takes
 // that out (it was most of the error against FP64).
 template <int N> __device__ __forceinline__ constexpr float line_excess() { return N == 3 ? 8.44e-8f : 0.0f; }
+
+// The longest piece (in cells) of a cubic ray that the 4-node Gauss rule
+// integrates to FP32 accuracy.  The 4-node rule is exact to degree 7; of the
+// degree-9 product of a piece of length h it misses only the coefficient C8
+// of the 8th power about the piece's middle (the 9th is odd there), by
+//   e8 (h/2)^9 C8,  e8 = 2^9 (4!)^4 / (9 (8!)^2) = 0.01161,
+// and C8 = D2 A3 B3 + D3 A2 B3 + D3 A3 B2 with |D3| <= 1/2, |A3| <= ra^3 / 2,
+// |B3| <= rb^3 / 2 the third- and |D2| <= 1, |A2| <= ra^2, |B2| <= rb^2 the
+// second-order coefficients of the three weights, so a footprint's error is at
+// most 5.67e-6 h^9 (ra rb + ra + rb) ra^2 rb^2.  The rule is taken where that
+// is below 2^-28, an eighth of an ulp of the footprint's peak (0.44): the
+// difference drowns in the FP32 rounding of the sums.  Rays with a small
+// component (most of a cone's) qualify at every length; a warp takes the
+// 5-node rule when one of its lanes has to.
+__device__ __forceinline__ float line_short(float ra, float rb)
+{
+    ra = fabsf(ra);
+    rb = fabsf(rb);
+    const float c = 5.67e-6f * 0x1p28f * (fmaf(ra, rb, ra) + rb) * (ra * ra) * (rb * rb);
+    return exp2f(-0.11111111f * log2f(c));
+}
 
 // The line {s + t w} (w of any length).  The two orientations of a line are
 // the same line: w_d > 0 is implied by dividing by w_d, and the transverse
@@ -194,6 +216,7 @@ __device__ __forceinline__ void line_setup(const DevGeom &g, const double (&s)[3
     const double a0 = fma(-(W + sd), ra, sp) + W, b0 = fma(-(W + sd), rb, sq) + W;
     L.ra = (float)ra;
     L.rb = (float)rb;
+    if (N == 3) L.h4 = line_short(L.ra, L.rb);
     // an axis that the ray does not move along: crossing at 3 - fraction, never inside a cell
     L.ia = ra != 0.0 ? 1.0f / L.ra : 1.0f;
     L.ib = rb != 0.0 ? 1.0f / L.rb : 1.0f;
@@ -302,9 +325,8 @@ __device__ __forceinline__ bool line_march(const LineRay &L, int seg, int ls, co
 #pragma unroll
                 for (int k = 0; k <= N; ++k) col[i][k] = __ldg(r + (size_t)i * D.nq + k);
             float2 S = make_float2(0.0f, 0.0f);
-#pragma unroll
-            for (int q = 0; q < M; ++q) {
-                const float tau = fmaf(half, qr.x[q], mid);
+            auto node = [&](float x, float wt) {
+                const float tau = fmaf(half, x, mid);
                 float wa[N + 1], wb[N + 1];
                 bweights<N>(fmaf(ra, tau, ga), wa);
                 bweights<N>(fmaf(rb, tau, gb), wb);
@@ -327,8 +349,23 @@ __device__ __forceinline__ bool line_march(const LineRay &L, int seg, int ls, co
                     }
                     h = i == 0 ? __fmul2_rn(dup(wa[0]), gk) : __ffma2_rn(dup(wa[i]), gk, h);
                 }
-                if constexpr (N == 1) S = __ffma2_rn(make_float2(qr.w[q] * (0.5f - tau), qr.w[q] * (0.5f + tau)), h, S);
-                else S = __ffma2_rn(make_float2(qr.w[q], qr.w[q] * tau), h, S);
+                if constexpr (N == 1) S = __ffma2_rn(make_float2(wt * (0.5f - tau), wt * (0.5f + tau)), h, S);
+                else S = __ffma2_rn(make_float2(wt, wt * tau), h, S);
+            };
+            if constexpr (N == 3) {
+                // four nodes where they are exact to FP32 (line_short) for
+                // every lane that is here, five otherwise
+                const bool five = t1 - t0 > __uint_as_float(lds128(&L.d).w);
+                if (__any_sync(__activemask(), five)) {
+#pragma unroll
+                    for (int q = 0; q < M; ++q) node(qr.x[q], qr.w[q]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < M - 1; ++q) node(qr.x1[q], qr.w1[q]);
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < M; ++q) node(qr.x[q], qr.w[q]);
             }
             const float v = half * (S.x + S.y);
             if (kahan) kahan_add(sum, comp, v);

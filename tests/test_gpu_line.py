@@ -137,3 +137,26 @@ def test_captured_forward_matches(env):
     torch.cuda.synchronize()
     g.status()
     assert float((eager - replayed).norm() / eager.norm()) <= TOL
+
+
+@pytest.mark.parametrize("ra,rb", [(0.9, 0.04), (0.6, 0.066), (0.3, 0.11), (0.29, 0.29), (0.95, 0.2), (1.0, 1.0)])
+def test_four_node_pieces_single_footprint(env, orc, ra, rb):
+    """One coefficient, so a ray's value is one footprint, for ray slopes on
+    both sides of the 4-node rule's bound (line_short: 5.67e-6 (ra rb + ra +
+    rb) ra^2 rb^2 against 2^-28).  Allowed: at most 12 pieces of 2^-28 each
+    and 20 roundings of 2^-25 at the peak (about 0.45 |w| / |w_d|)."""
+    torch, spl = env
+    rng = np.random.default_rng(8)
+    dims = (9, 9, 9)
+    w = np.tile([ra, 1.0, rb], (2000, 1))
+    s = rng.uniform(-1.5, 1.5, size=w.shape)
+    geo = I.RayGeometry(w / np.linalg.norm(w, axis=1, keepdims=True), s)
+    c = np.zeros(dims, dtype=np.float32)
+    c[4, 4, 4] = 1.0
+    g = spl.Geometry(dims, I.centred_origin(dims), geo)
+    y = torch.empty(g.n_rays, device="cuda")
+    spl.forward(g, torch.tensor(c, device="cuda"), y, spl.basis(3))
+    g.status()
+    ref = orc.forward(3, dims, I.centred_origin(dims), c.astype(np.float64), geom_of(orc, geo)).reshape(-1)
+    scale = np.sqrt(1.0 + ra * ra + rb * rb)
+    assert np.max(np.abs(y.cpu().numpy() - ref)) <= scale * (12 * 2.0 ** -28 + 20 * 2.0 ** -25)
