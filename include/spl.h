@@ -161,8 +161,9 @@ typedef struct {
  * the plane path beside the march of the other views (the caller's stream
  * waits for it, so each call stays one ordered operation on that stream).
  * Scratch of the scatter adjoint, allocated here: the coefficient array in
- * three layouts (x, y and z fast) of four shifted copies each (about
- * 48 nx ny nz bytes; not for a parallel geometry whose views are all in the
+ * up to three layouts (x, y and z fast, those that some ray needs) of four
+ * shifted copies each, on a grid padded by 3 (16 bytes per coefficient and
+ * layout; not for a parallel geometry whose views are all in the
  * flat class) and, for more than 48 views or 2^22 explicit rays, an FP64
  * accumulator (8 nx ny nz bytes).  Scratch of the forward, for geometries
  * with rays outside the flat class: the coefficients resampled along each

@@ -29,6 +29,7 @@
 #include <new>
 
 #include "spl_host.h"
+#include "spl_line.cuh"
 
 namespace spl {
 
@@ -38,12 +39,6 @@ namespace spl {
 // run of columns (see line_lanes_along_v).
 __host__ __device__ constexpr int line_p(int d) { return d == 1 ? 0 : 1; }
 __host__ __device__ constexpr int line_q(int d) { return d == 2 ? 0 : 2; }
-
-// (selects: a run-time index would put the array into local memory)
-template <class T> __host__ __device__ inline T sel3(int i, const T &a, const T &b, const T &c)
-{
-    return i == 0 ? a : (i == 1 ? b : c);
-}
 
 // Resampled array of axis d at degree n: cells c = 0 .. n_d + n - 1, columns
 // padded by n zeros on every side (a piece's window then never leaves the
@@ -135,12 +130,6 @@ __global__ void __launch_bounds__(256) k_line_resample(DevGeom g, const float *_
 }
 
 // ---------------------------------------------------------------- ray set-up
-// Transverse coordinates are carried as 64-bit fixed point with kLineFrac
-// fraction bits: the start is exact to 2^-41 and the step is off by at most
-// 2^-41 per cell, 2^-30 over the longest ray, so a cell's fraction is its
-// FP32 rounding everywhere on the ray, for one 64-bit add per cell.
-constexpr int kLineFrac = 40;
-
 // A ray, in shared memory: set up by one thread, read by the 2^ls threads
 // that share it.
 struct __align__(16) LineRay {
@@ -153,34 +142,6 @@ struct __align__(16) LineRay {
     int d, c, cl;             // dominant axis, first and last cell (none: c > cl)
     float h4;                 // longest piece that four Gauss nodes integrate (cubic, line_short)
 };
-
-// The FP32 constants 2/3 and 1/6 of the cubic weights (bweights<3>) are
-// 1.987e-8 and 4.97e-9 too large, so the four weights of an axis sum to
-// 1 + 2 (1.987e-8) + 4.97e-9 (g^3 + t^3), on average 1 + 4.22e-8, and every
-// integral over two axes comes out 8.44e-8 too large.  The ray's scale takes
-// that out (it was most of the error against FP64).
-template <int N> __device__ __forceinline__ constexpr float line_excess() { return N == 3 ? 8.44e-8f : 0.0f; }
-
-// The longest piece (in cells) of a cubic ray that the 4-node Gauss rule
-// integrates to FP32 accuracy.  The 4-node rule is exact to degree 7; of the
-// degree-9 product of a piece of length h it misses only the coefficient C8
-// of the 8th power about the piece's middle (the 9th is odd there), by
-//   e8 (h/2)^9 C8,  e8 = 2^9 (4!)^4 / (9 (8!)^2) = 0.01161,
-// and C8 = D2 A3 B3 + D3 A2 B3 + D3 A3 B2 with |D3| <= 1/2, |A3| <= ra^3 / 2,
-// |B3| <= rb^3 / 2 the third- and |D2| <= 1, |A2| <= ra^2, |B2| <= rb^2 the
-// second-order coefficients of the three weights, so a footprint's error is at
-// most 5.67e-6 h^9 (ra rb + ra + rb) ra^2 rb^2.  The rule is taken where that
-// is below 2^-28, an eighth of an ulp of the footprint's peak (0.44): the
-// difference drowns in the FP32 rounding of the sums.  Rays with a small
-// component (most of a cone's) qualify at every length; a warp takes the
-// 5-node rule when one of its lanes has to.
-__device__ __forceinline__ float line_short(float ra, float rb)
-{
-    ra = fabsf(ra);
-    rb = fabsf(rb);
-    const float c = 5.67e-6f * 0x1p28f * (fmaf(ra, rb, ra) + rb) * (ra * ra) * (rb * rb);
-    return exp2f(-0.11111111f * log2f(c));
-}
 
 // The line {s + t w} (w of any length).  The two orientations of a line are
 // the same line: w_d > 0 is implied by dividing by w_d, and the transverse
@@ -211,7 +172,7 @@ __device__ __forceinline__ void line_setup(const DevGeom &g, const double (&s)[3
     // from the FP64 residual
     const double q2 = fma(ra, ra, fma(rb, rb, 1.0));
     L.scale = sqrtf((float)q2);
-    L.scale_lo = fmaf(-line_excess<N>(), L.scale, (float)fma(-(double)L.scale, (double)L.scale, q2) * (0.5f / L.scale));
+    L.scale_lo = fmaf(-weight_excess<N>(2), L.scale, (float)fma(-(double)L.scale, (double)L.scale, q2) * (0.5f / L.scale));
     // transverse coordinates at v_d = 0
     const double a0 = fma(-(W + sd), ra, sp) + W, b0 = fma(-(W + sd), rb, sq) + W;
     L.ra = (float)ra;
@@ -248,19 +209,6 @@ __device__ __forceinline__ void line_setup(const DevGeom &g, const double (&s)[3
     L.RB = __double2ll_rn(rb * kOne);
     L.A = __double2ll_rn(fma((double)c, ra, a0) * kOne);
     L.B = __double2ll_rn(fma((double)c, rb, b0) * kOne);
-}
-
-// 16 bytes of a ray, not to be kept in registers: next to 64 column values
-// the cubic march has none for the constants that only its events need (with
-// them in registers it spills: 8 helical views 51.9 ms, 49.5 without), so
-// the load is volatile and stays in the loop.
-__device__ __forceinline__ uint4 lds128(const void *p)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"((unsigned)__cvta_generic_to_shared(p)));
-    return v;
 }
 
 // ---------------------------------------------------------------- the march
@@ -436,56 +384,32 @@ __device__ __forceinline__ bool line_lanes_along_v(const DevGeom &g, const ViewP
     return fabs(q == 2 ? P.dv[2] : P.dv[0]) >= fabs(q == 2 ? P.du[2] : P.du[0]);
 }
 
-// view geometries: view blockIdx.z (of order[], when given); the block's 128
-// >> ls pixels form a tile of 16 x 8, 8 x 8, 8 x 4 or 4 x 4
+// view geometries: view blockIdx.z (of order[], when given)
 template <int N>
 __global__ void __launch_bounds__(128, LineBlocks<N>::value)
     k_line_views(DevGeom g, LineArrays arr, float *__restrict__ y, QuadRule qr, int kahan, const int *order, int ls)
 {
     const int seg = threadIdx.x & ((1 << ls) - 1), p = threadIdx.x >> ls;
-    const int lane = p & 31, wid = p >> 5;
     const int k = order ? order[blockIdx.z] : (int)blockIdx.z;
-    int iu, iv;
-    if (ls == 0) {
-        if (line_lanes_along_v(g, g.views[k])) {
-            iu = blockIdx.x * 16 + wid * 4 + (lane >> 3);
-            iv = blockIdx.y * 8 + (lane & 7);
-        } else {
-            iu = blockIdx.x * 16 + (wid & 1) * 8 + (lane & 7);
-            iv = blockIdx.y * 8 + (wid >> 1) * 4 + (lane >> 3);
-        }
-    } else {
-        // tile of 8 x 8, 8 x 4, 4 x 4
-        const int lw = ls == 3 ? 2 : 3;
-        iu = (blockIdx.x << lw) + (p & ((1 << lw) - 1));
-        iv = blockIdx.y * (ls == 1 ? 8 : 4) + (p >> lw);
-    }
+    const bool along_v = line_lanes_along_v(g, g.views[k]);
     __shared__ LineRay rays[128];
-    auto setup = [&](LineRay &L, int u, int v) {
-        L.c = 0;
-        L.cl = -1;
-        if (u >= g.nu || v >= g.nv) return;  // beyond the detector
-        const ViewPose &P = g.views[k];
-        const double a = u - 0.5 * (g.nu - 1), b = v - 0.5 * (g.nv - 1);
-        double s[3], w[3];
-#pragma unroll
-        for (int e = 0; e < 3; ++e) {
-            const double q = fma(b, P.dv[e], fma(a, P.du[e], P.dc[e])), src = P.src[e];
-            s[e] = q;
-            w[e] = g.kind == SPL_PARALLEL ? src : q - src;
+    // thread t sets up ray t of the block
+    const int t = threadIdx.x;
+    if (t < (128 >> ls)) {
+        int u, v;
+        line_tile(t, ls, along_v, u, v);
+        rays[t].c = 0;
+        rays[t].cl = -1;
+        if (u < g.nu && v < g.nv) {
+            double s[3], w[3];
+            line_pixel(g, k, u, v, s, w);
+            line_setup<N>(g, s, w, rays[t]);
         }
-        line_setup<N>(g, s, w, L);
-    };
-    if (ls == 0) {
-        setup(rays[p], iu, iv);
-        __syncwarp();
-    } else {
-        // thread t sets up ray t of the block
-        const int t = threadIdx.x, lw = ls == 3 ? 2 : 3;
-        if (t < (128 >> ls))
-            setup(rays[t], (blockIdx.x << lw) + (t & ((1 << lw) - 1)), blockIdx.y * (ls == 1 ? 8 : 4) + (t >> lw));
-        __syncthreads();
     }
+    if (ls == 0) __syncwarp();
+    else __syncthreads();
+    int iu, iv;
+    line_tile(p, ls, along_v, iu, iv);
     const bool in = iu < g.nu && iv < g.nv;
     const float v = line_value<N>(g, rays[p], arr, qr, kahan, seg, ls);
     if (seg == 0 && in) y[((long long)k * g.nv + iv) * g.nu + iu] = v;
@@ -539,44 +463,18 @@ struct LineScratch {
 constexpr size_t kLineMaxBytes = (size_t)24 << 30;
 constexpr size_t kLineMaxBytesRays = (size_t)320 << 20;
 
-// Axes that can be the dominant one of a line of the geometry (a superset):
-// |w_e| over a view's pixels lies between bounds taken at its corners, since
-// a pixel's direction is affine in (u, v).
-static unsigned line_axes(const spl_geometry *g, const double *raw_rays)
+// Axes that can be the dominant one of a line of the geometry (a superset).
+static unsigned line_axes(const spl_geometry *g, const double *ray_dirs)
 {
-    const DevGeom &dg = g->dev;
     unsigned mask = 0;
-    auto add = [&](const double (&lo)[3], const double (&hi)[3]) {
+    line_bounds(g, ray_dirs, [&](const double (&lo)[3], const double (&hi)[3]) {
         for (int e = 0; e < 3; ++e) {
             bool can = true;
             for (int f = 0; f < 3; ++f) can = can && hi[e] * (1.0 + 1e-9) >= lo[f];
             if (can) mask |= 1u << e;
         }
-    };
-    if (dg.kind == SPL_RAYS) {
-        for (long long r = 0; r < dg.n_rays && mask != 7u; ++r) {
-            double m[3];
-            for (int e = 0; e < 3; ++e) m[e] = fabs(raw_rays[3 * r + e]);
-            add(m, m);
-        }
-        return mask;
-    }
-    for (int k = 0; k < dg.n_views && mask != 7u; ++k) {
-        const ViewPose &P = g->views_host[k];
-        double lo[3], hi[3];
-        for (int e = 0; e < 3; ++e) {
-            double mn = INFINITY, mx = -INFINITY;
-            for (int corner = 0; corner < 4; ++corner) {
-                const double a = ((corner & 1) ? 0.5 : -0.5) * (dg.nu - 1), b = ((corner & 2) ? 0.5 : -0.5) * (dg.nv - 1);
-                const double v = dg.kind == SPL_PARALLEL ? P.src[e] : P.dc[e] + a * P.du[e] + b * P.dv[e] - P.src[e];
-                mn = fmin(mn, v);
-                mx = fmax(mx, v);
-            }
-            lo[e] = mn <= 0.0 && mx >= 0.0 ? 0.0 : fmin(fabs(mn), fabs(mx)) * (1.0 - 1e-9);
-            hi[e] = fmax(fabs(mn), fabs(mx));
-        }
-        add(lo, hi);
-    }
+        return mask != 7u;
+    });
     return mask;
 }
 
@@ -638,16 +536,6 @@ bool line_usable(const spl_geometry *g, int degree, cudaStream_t st)
     return cap == cudaStreamCaptureStatusNone;
 }
 
-// Threads per ray, 2^ls: the fewest that give every SM its resident threads,
-// at most 8 (a thread keeps at least a few cells of the ray).
-static int line_split(long long rays, int blocks_per_sm)
-{
-    const long long fill = (long long)sm_count() * blocks_per_sm * 128;
-    int ls = 0;
-    while (ls < 3 && (rays << ls) < fill) ++ls;
-    return ls;
-}
-
 template <int N>
 static spl_status line_forward_n(const spl_geometry *g, int kahan, const float *c, float *y, cudaStream_t st)
 {
@@ -676,9 +564,7 @@ static spl_status line_forward_n(const spl_geometry *g, int kahan, const float *
         const int v0 = dg.kind == SPL_PARALLEL ? dg.n_flat : 0, nview = dg.n_views - v0;
         const int *order = dg.kind == SPL_PARALLEL ? dg.view_order + v0 : nullptr;
         const int ls = line_split((long long)nview * dg.nu * dg.nv, LineBlocks<N>::value);
-        const int tw = ls == 0 ? 16 : (ls == 3 ? 4 : 8), th = ls < 2 ? 8 : 4;
-        const dim3 grid((dg.nu + tw - 1) / tw, (dg.nv + th - 1) / th, nview);
-        k_line_views<N><<<grid, 128, 0, st>>>(dg, S.arr, y, qr, kahan, order, ls);
+        k_line_views<N><<<line_grid(dg, nview, ls), 128, 0, st>>>(dg, S.arr, y, qr, kahan, order, ls);
     }
     s = cuda_check(cudaGetLastError(), "line forward launch");
     // recorded also after a failed launch: what did start still uses the scratch

@@ -10,17 +10,15 @@
 // are added along the ray with Kahan compensation.
 //
 // Adjoint, view geometries, two forms that visit the same pairs with the
-// same footprint values:
-//  * scatter (default): the forward's thread mapping; each flushed
-//    contribution y_r * P is added to c with a float atomic (a
-//    fire-and-forget reduction in L2), which overlaps with the FP32 work --
-//    on GB300 A^T then costs about as much as A;
+// same footprints:
+//  * scatter (default, scatter.cu): the forward's thread mapping, vector
+//    reductions into layouts of c; flat parallel views reduce into c here;
 //  * gather: one block per 16^3 coefficient brick; for every batch of 8
 //    views the block projects the brick's support box onto the detectors,
 //    walks the rays of those pixel windows through the brick's cells with
-//    the same set-up and cell march, accumulates y_r * P in shared memory
-//    and folds the batch into FP64 totals; no global atomics, each
-//    coefficient written once.
+//    the piece march, accumulates y_r * P in shared memory and folds the
+//    batch into FP64 totals; no global atomics, each coefficient written
+//    once.
 // Adjoint, explicit rays: no view structure to gather over: scatter.
 #include <stdio.h>
 #include <string.h>
@@ -37,7 +35,6 @@ namespace spl {
 // piece march).
 struct FwdSink {
     static constexpr bool plane = false;
-    static constexpr bool face = false;
     const float *__restrict__ c;
     int S0, S1, S2;
     unsigned off;
@@ -57,7 +54,6 @@ struct FwdSink {
     {
         if (bx.holds(ld, la, lb)) acc[0] = fmaf(__ldg(c + (ld * S0 + la * S1 + lb * S2)), v, acc[0]);
     }
-    __device__ __forceinline__ float wscale() const { return 1.0f; }
     __device__ __forceinline__ void put(unsigned o, bool in, float v, int slot)
     {
         if (in) acc[slot & 3] = fmaf(__ldg(c + o), v, acc[slot & 3]);
@@ -73,7 +69,6 @@ struct FwdSink {
 
 struct CountSink {
     static constexpr bool plane = false;
-    static constexpr bool face = false;
     int S0, S1, S2;
     unsigned off;
     SinkBox bx;
@@ -88,64 +83,18 @@ struct CountSink {
     {
         n += (bx.holds(ld, la, lb) && v > 0.0f) ? 1u : 0u;
     }
-    __device__ __forceinline__ float wscale() const { return 1.0f; }
     __device__ __forceinline__ void put(unsigned, bool in, float v, int) { n += (in && v > 0.0f) ? 1u : 0u; }
     __device__ __forceinline__ void cell_end() {}
 };
 
-// adjoint, scatter: y_r / |w_d| * F_l added to c_l with a float atomic.
-// The target of a piece-marched ray is a set of four shifted copies of a
-// layout of c (copy j holds coefficient i at position j * cs + i + j, cs a
-// multiple of 4): a face row of N+1 = 4 consecutive floats starting at
-// index lo goes, as one 16-byte vector atomic, to the copy j = -lo mod 4 in
-// which it starts a 16-byte group.  Faces without such a row, the cell
-// march's flushes and the last window take scalar atomics into copy 0.
-// The copies are summed into c afterwards (k_fold_copies*).
+// adjoint, flat parallel views: y_r / |w_d| * F_l added to c_l with a float
+// atomic
 struct AtomicSink {
     static constexpr bool plane = false;
-    static constexpr bool face = true;
-    float *__restrict__ c;  // copy 0 (or c itself where no vector row is written)
-    size_t cs;              // copy stride in floats
+    float *__restrict__ c;
     int S0, S1, S2;
-    unsigned off;
     SinkBox bx;
     float yv;
-    // w0..w3 (already scaled) at p, p + s, p + 2 s, p + 3 s with s = +1 (UP)
-    // or -1: one aligned 16-byte atomic into the copy where the run starts
-    // a group
-    template <bool UP>
-    __device__ __forceinline__ void row4(unsigned p, float w0, float w1, float w2, float w3)
-    {
-        const unsigned lo = UP ? p : p - 3u;
-        const unsigned j = (0u - lo) & 3u;
-        const float4 f = UP ? make_float4(w0, w1, w2, w3) : make_float4(w3, w2, w1, w0);
-        atomicAdd(reinterpret_cast<float4 *>(c + ((size_t)j * cs + (size_t)(lo + j))), f);
-    }
-    // the face's (N+1)^2 values at base + x SX + y SY.  In the layout of a
-    // piece-marched ray the b axis is contiguous (S2 = +-1), so the faces of
-    // d and a events (SY = S2) have rows along y; the faces of b events
-    // (SY = S1) take scalar atomics.  The sign of S2 is the ray's and
-    // mostly the warp's, so the two row directions are branches.
-    template <int N>
-    __device__ __forceinline__ void put_face(unsigned base, unsigned SX, unsigned SY, const float (&v)[N + 1][N + 1])
-    {
-        if constexpr (N == 3) {
-            if (SY == 1u) {
-#pragma unroll
-                for (int x = 0; x <= N; ++x) row4<true>(base + (unsigned)x * SX, v[x][0], v[x][1], v[x][2], v[x][3]);
-                return;
-            }
-            if (SY == 0xffffffffu) {
-#pragma unroll
-                for (int x = 0; x <= N; ++x) row4<false>(base + (unsigned)x * SX, v[x][0], v[x][1], v[x][2], v[x][3]);
-                return;
-            }
-        }
-#pragma unroll
-        for (int x = 0; x <= N; ++x)
-#pragma unroll
-            for (int y = 0; y <= N; ++y) atomicAdd(c + (base + (unsigned)x * SX + (unsigned)y * SY), v[x][y]);
-    }
     __device__ __forceinline__ void piece() {}
     __device__ __forceinline__ bool relevant(int d0, int d1, int a0, int a1, int b0, int b1) const
     {
@@ -155,13 +104,6 @@ struct AtomicSink {
     {
         if (bx.holds(ld, la, lb)) atomicAdd(c + (ld * S0 + la * S1 + lb * S2), yv * v);
     }
-    // the piece march scales its Gauss weights by y_r (wscale), so the
-    // window values that reach put and put_face already carry the factor
-    __device__ __forceinline__ float wscale() const { return yv; }
-    __device__ __forceinline__ void put(unsigned o, bool in, float v, int)
-    {
-        if (in) atomicAdd(c + o, v);
-    }
     __device__ __forceinline__ void cell_end() {}
 };
 
@@ -169,7 +111,6 @@ struct AtomicSink {
 // shared-memory brick array (mirrored strides S0..S2, offset off)
 struct BrickSink {
     static constexpr bool plane = false;
-    static constexpr bool face = false;
     float *part;
     int S0, S1, S2;
     unsigned off;
@@ -184,7 +125,6 @@ struct BrickSink {
     {
         if (bx.holds(ld, la, lb)) atomicAdd(part + (unsigned)(ld * S0 + la * S1 + lb * S2 + (int)off), yv * v);
     }
-    __device__ __forceinline__ float wscale() const { return 1.0f; }
     __device__ __forceinline__ void put(unsigned o, bool in, float v, int)
     {
         if (in) atomicAdd(part + o, yv * v);
@@ -365,137 +305,14 @@ __global__ void __launch_bounds__(128) k_count_rays(DevGeom g, unsigned long lon
     add_count(count + 2, pf);
 }
 
-// ---------------------------------------------------------------- adjoint: ray-driven scatter
-
-template <int N, int VM>
-__device__ __forceinline__ void scatter_ray(const RaySetup &rs, float yr, float *__restrict__ c, size_t cs,
-                                            const QuadRule &qr, int *err)
-{
-    AtomicSink sk;
-    sk.c = c;
-    sk.cs = cs;
-    sk.S0 = rs.S[0];
-    sk.S1 = rs.S[1];
-    sk.S2 = rs.S[2];
-    sk.off = 0u;
-    sk.bx = make_box(rs.lo, rs.hi);
-    sk.yv = yr * rs.inv_wd;
-    if (!march_vm<N, VM>(rs, rs.c0, rs.c1, qr, sk)) atomicOr(err, 1);
-}
-
-// The layout a piece-marched scatter ray reduces into: the one whose
-// contiguous axis is the ray's b axis (its smallest direction component),
-// l0 = [z][y][x] (x fast), l1 = [z][x][y] (y fast) or l2 = [y][x][z] (z
-// fast), each as four shifted copies (AtomicSink); rs.S is re-pointed at
-// that layout.  The faces that leave the window on d and a events (all but
-// the rare b events) then contain rows along b and go out as one 16-byte
-// vector atomic per row, and the lanes of a warp, whose rays lie side by
-// side, reduce into neighbouring addresses.  The copies are folded into c
-// after the launch.
-__device__ __forceinline__ float *b_fast_target(const DevGeom &g, RaySetup &rs, float *l0, float *l1, float *l2)
-{
-    if (rs.ax[2] == 0) return l0;
-    int st[3];
-    float *t;
-    if (rs.ax[2] == 1) {
-        st[0] = g.n[1];
-        st[1] = 1;
-        st[2] = g.n[0] * g.n[1];
-        t = l1;
-    } else {
-        st[0] = g.n[2];
-        st[1] = g.n[0] * g.n[2];
-        st[2] = 1;
-        t = l2;
-    }
-#pragma unroll
-    for (int q = 0; q < 3; ++q) rs.S[q] = rs.sg[q] * st[rs.ax[q]];
-    return t;
-}
-
-// rays r0 .. r1-1
+// ---------------------------------------------------------------- adjoint: flat parallel views
+// The flat views outside the plane group: the forward's thread mapping, the
+// flat cell march, scalar atomics into c.  Every other ray scatters through
+// scatter.cu.
 template <int N>
-__global__ void __launch_bounds__(128) k_adjoint_rays(DevGeom g, const float *__restrict__ y, float *__restrict__ l0,
-                                                      float *__restrict__ l1, float *__restrict__ l2, QuadRule qr,
-                                                      long long r0, long long r1)
-{
-    const long long r = r0 + (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= r1) return;
-    const float yr = y[r];
-    if (yr == 0.0f) return;
-    double s[3], w[3];
-    explicit_ray(g, r, s, w);
-    RaySetup rs;
-    if (!ray_setup<N>(grid_of(g), s, w, rs)) return;
-    float *t = b_fast_target(g, rs, l0, l1, l2);
-    scatter_ray<N, VM_RAYS>(rs, yr, t, g.lay_cs, qr, g.err);
-}
-
-// view geometries, scatter form: the forward's thread mapping; views
-// v0 + blockIdx.z
-template <int N>
-__global__ void __launch_bounds__(128, 3)
-    k_adjoint_views_scatter(DevGeom g, const float *__restrict__ y, float *__restrict__ l0, float *__restrict__ l1,
-                            float *__restrict__ l2, QuadRule qr, int v0)
-{
-    int iu, iv;
-    tile_pixel(iu, iv);
-    const int k = v0 + blockIdx.z;
-    if (iu >= g.nu || iv >= g.nv) return;
-    const float yr = __ldg(y + ((long long)k * g.nv + iv) * g.nu + iu);
-    if (yr == 0.0f) return;
-    RaySetup rs;
-    if (!view_setup<N>(g, grid_of(g), k, iu, iv, rs)) return;
-    float *t = b_fast_target(g, rs, l0, l1, l2);
-    scatter_ray<N, VM_CONE>(rs, yr, t, g.lay_cs, qr, g.err);
-}
-
-// c[i] += sum_j l0[j cs + i + j]: the fold of the x-fast copies into c
-__global__ void k_fold_copies(float *__restrict__ c, const float *__restrict__ in, long long n, long long cs)
-{
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        c[i] += (in[i] + in[cs + i + 1]) + (in[2 * cs + i + 2] + in[3 * cs + i + 3]);
-}
-
-// out[s][r][q] += sum_j in[j cs + (s Q + q) R + r + j]: the fold of the
-// shifted copies of a Q x R row-major layout into c, slab by slab.  y fast:
-// slabs z, Q = nx, R = ny; z fast: one slab, Q = nx ny, R = nz.  32 x 32
-// tiles through shared memory, both sides coalesced.
-__global__ void __launch_bounds__(256) k_fold_copies_transpose(float *__restrict__ out, const float *__restrict__ in,
-                                                               long long Q, long long R, long long slabs, long long cs)
-{
-    __shared__ float t[32][33];
-    const long long q0 = (long long)blockIdx.x * 32, r0 = (long long)blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (long long sl = blockIdx.z; sl < slabs; sl += gridDim.z) {
-        const long long base = sl * Q * R;
-        for (int j = ty; j < 32; j += 8) {
-            const long long q = q0 + j, r = r0 + tx;
-            float v = 0.0f;
-            if (q < Q && r < R) {
-                const long long i = base + q * R + r;
-                v = (in[i] + in[cs + i + 1]) + (in[2 * cs + i + 2] + in[3 * cs + i + 3]);
-            }
-            t[j][tx] = v;
-        }
-        __syncthreads();
-        for (int j = ty; j < 32; j += 8) {
-            const long long r = r0 + j, q = q0 + tx;
-            if (q < Q && r < R) out[base + r * Q + q] += t[tx][j];
-        }
-        __syncthreads();
-    }
-}
-
-// parallel views of one class; the general class (piece march) reduces
-// into the view's b-fast layout (ViewConst::lay, Sb), the flat class (cell
-// march, scalar atomics) into c
-template <int N, int VM>
-__global__ void __launch_bounds__(128, ViewBlocks<VM>::value)
-    k_adjoint_pviews_scatter(DevGeom g, const float *__restrict__ y, float *__restrict__ c, float *__restrict__ l0,
-                             float *__restrict__ l1, float *__restrict__ l2, QuadRule qr,
-                             const __grid_constant__ ViewChunk vc)
+__global__ void __launch_bounds__(128, ViewBlocks<VM_FLAT>::value)
+    k_adjoint_flat_scatter(DevGeom g, const float *__restrict__ y, float *__restrict__ c, QuadRule qr,
+                           const __grid_constant__ ViewChunk vc)
 {
     int iu, iv;
     tile_pixel(iu, iv);
@@ -505,17 +322,16 @@ __global__ void __launch_bounds__(128, ViewBlocks<VM>::value)
     const float yr = __ldg(y + ((long long)k * g.nv + iv) * g.nu + iu);
     if (yr == 0.0f) return;
     RaySetup rs;
-    if (view_setup<N>(g, grid_of(g), k, iu, iv, rs)) {
-        use_view_const(V, rs);
-        if constexpr (VM == VM_GENERAL) {
-            float *t = V.lay == 0 ? l0 : (V.lay == 1 ? l1 : l2);
-#pragma unroll
-            for (int q = 0; q < 3; ++q) rs.S[q] = V.Sb[q];
-            scatter_ray<N, VM>(rs, yr, t, g.lay_cs, qr, g.err);
-        } else {
-            scatter_ray<N, VM>(rs, yr, c, 0, qr, g.err);
-        }
-    }
+    if (!view_setup<N>(g, grid_of(g), k, iu, iv, rs)) return;
+    use_view_const(V, rs);
+    AtomicSink sk;
+    sk.c = c;
+    sk.S0 = rs.S[0];
+    sk.S1 = rs.S[1];
+    sk.S2 = rs.S[2];
+    sk.bx = make_box(rs.lo, rs.hi);
+    sk.yv = yr * rs.inv_wd;
+    if (!cell_march<N, AtomicSink, true>(rs, rs.c0, rs.c1, qr, sk)) atomicOr(g.err, 1);
 }
 
 // ---------------------------------------------------------------- adjoint: brick gather (view geometries)
@@ -837,6 +653,64 @@ static spl_status forward_quad(const spl_geometry *g, const spl_basis_desc *b, c
     return b->mode == SPL_FP_DIRECT ? forward_quad_t<N, true>(g, b, c, y, st) : forward_quad_t<N, false>(g, b, c, y, st);
 }
 
+// The scatter form over the views from v0 of the view order (or all rays):
+// the flat class into c, the rest into the layout copies (scatter.cu).
+// has_c: c already holds a part of the result.
+//
+// Both add y_r * F_l with FP32 atomics.  A coefficient of a large geometry
+// receives tens of thousands of them (512^3 helical: ~4e4), and an FP32
+// running sum of that many terms loses ~1e-5 of its value; so a geometry with
+// more than one batch of views (rays) adds each batch to an FP64 total (its
+// scratch, acc64, is allocated with the geometry), which is rounded to c with
+// the last batch.  Each batch's FP32 sum has ~1/B of the terms and of the
+// magnitude, so its rounding error is ~1/B of the whole.
+template <int N>
+static spl_status adjoint_scatter(const spl_geometry *g, const float *y, float *c, int v0, bool has_c, const QuadRule &qr,
+                                  cudaStream_t st)
+{
+    const DevGeom &dg = g->dev;
+    const long long nc = (long long)dg.n[0] * dg.n[1] * dg.n[2];
+    const bool batched = g->acc64 != nullptr, par = dg.kind == SPL_PARALLEL;
+    const long long i0 = par ? dg.n_flat : 0, i1 = dg.kind == SPL_RAYS ? dg.n_rays : dg.n_views;
+    const bool flat = par && v0 < dg.n_flat, rest = dg.n_rays > 0 && i0 < i1;
+    spl_status s = SPL_OK;
+    bool has_total = false;  // the FP64 total holds a part of the result
+    auto clear_c = [&]() {
+        if (s == SPL_OK) s = cuda_check(cudaMemsetAsync(c, 0, nc * sizeof(float), st), "adjoint clear");
+    };
+    auto add_c = [&]() {  // total += c
+        if (s == SPL_OK && !has_total)
+            s = cuda_check(cudaMemsetAsync(g->acc64, 0, nc * sizeof(double), st), "adjoint accumulator clear");
+        if (s != SPL_OK) return;
+        has_total = true;
+        k_acc_add<<<stream_grid(nc), 256, 0, st>>>(nc, g->acc64, c);
+    };
+    if (batched && has_c) add_c();
+    if (flat) {
+        const unsigned gx = (dg.nu + 15) / 16, gy = (dg.nv + 7) / 8;
+        if (!batched && !has_c) clear_c();
+        for_view_chunks(g, v0, dg.n_flat - v0, [&](const ViewChunk &ch, int n) {
+            if (batched) clear_c();
+            if (s != SPL_OK) return;
+            k_adjoint_flat_scatter<N><<<dim3(gx, gy, n), 128, 0, st>>>(dg, y, c, qr, ch);
+            if (batched) add_c();
+        }, batched ? kAdjBatchViews : kViewChunk);
+        has_c = true;
+    }
+    const long long per = !batched ? i1 : (dg.kind == SPL_RAYS ? kAdjBatchRays : kAdjBatchViews);
+    for (long long i = i0; rest && i < i1 && s == SPL_OK; i += per) {
+        const bool last = i + per >= i1;
+        s = scatter_rays(g, N, y, i, last ? i1 : i + per, st);
+        if (s != SPL_OK) break;
+        s = scatter_fold(g, N, has_total ? 2 : (has_c && !batched ? 1 : 0), batched && !last, c, st);
+        has_total = has_total || (batched && !last);
+    }
+    if (s != SPL_OK) return s;
+    if (!rest && has_total) k_acc_store<<<stream_grid(nc), 256, 0, st>>>(nc, g->acc64, c);
+    else if (!rest && !has_c) clear_c();
+    return s == SPL_OK ? launch_status("adjoint launch") : s;
+}
+
 template <int N>
 static spl_status adjoint_quad(const spl_geometry *g, const spl_basis_desc *b, const float *y, float *c, cudaStream_t st)
 {
@@ -850,126 +724,32 @@ static spl_status adjoint_quad(const spl_geometry *g, const spl_basis_desc *b, c
         v0 = plane_views(g, b, &s);
         if (s != SPL_OK) return s;
     }
+    const bool scatter = dg.kind == SPL_RAYS || form != SPL_ADJ_GATHER;
     // With the scatter form the plane path's gather (T, memory-latency
-    // bound) runs on the geometry's side stream beside the march's scatter
-    // into the cleared c (arithmetic bound); after the join, T's
-    // contribution is added to c.  Otherwise the plane path writes every
-    // coefficient first and the other views add.
-    const bool overlap = dg.kind == SPL_PARALLEL && dg.n_rays > 0 && v0 > 0 && v0 < dg.n_views && form != SPL_ADJ_GATHER &&
-                         g->plane->side;
+    // bound) runs on the geometry's side stream beside the scatter of the
+    // other views (arithmetic bound); after the join, T's contribution is
+    // added to c.  Otherwise the plane path writes every coefficient first
+    // and the other views add.
+    const bool overlap = dg.n_rays > 0 && v0 > 0 && v0 < dg.n_views && scatter && g->plane->side;
     if (overlap) {
         s = cuda_check(cudaEventRecord(g->plane->fork, st), "fork record");
         if (s == SPL_OK) s = cuda_check(cudaStreamWaitEvent(g->plane->side, g->plane->fork, 0), "fork wait");
         if (s != SPL_OK) return s;
         s = plane_adjoint_t(g, N, y, g->plane->side);
-        spl_status sj = cuda_check(cudaEventRecord(g->plane->join, g->plane->side), "join record");
-        if (s == SPL_OK) s = sj;
-        if (s == SPL_OK) s = cuda_check(cudaMemsetAsync(c, 0, nc * sizeof(float), st), "adjoint clear");
-        if (s != SPL_OK) {
-            // join the side stream before returning the error
-            if (sj == SPL_OK) cudaStreamWaitEvent(st, g->plane->join, 0);
-            return s;
-        }
-    } else if (v0 > 0) {
+        const spl_status sj = cuda_check(cudaEventRecord(g->plane->join, g->plane->side), "join record");
+        if (s == SPL_OK && sj == SPL_OK) s = adjoint_scatter<N>(g, y, c, v0, false, qr, st);
+        // join the side stream also on an error
+        const spl_status sw =
+            sj == SPL_OK ? cuda_check(cudaStreamWaitEvent(st, g->plane->join, 0), "join wait") : sj;
+        if (s == SPL_OK) s = sw;
+        return s == SPL_OK ? plane_adjoint_add(g, N, c, st) : s;
+    }
+    if (v0 > 0) {
         s = plane_adjoint(g, N, y, c, st);
         if (s != SPL_OK) return s;
-    } else if (dg.kind == SPL_RAYS || form != SPL_ADJ_GATHER) {
-        s = cuda_check(cudaMemsetAsync(c, 0, nc * sizeof(float), st), "adjoint clear");
-        if (s != SPL_OK) return s;
     }
-    if (dg.n_rays == 0) return SPL_OK;
-    // The scatter adds y_r * F_l with FP32 atomics.  A coefficient of a
-    // large geometry receives tens of thousands of them (512^3 helical:
-    // ~4e4), and an FP32 running sum of that many terms loses ~1e-5 of its
-    // value; so a geometry with more than one batch of views (rays) scatters
-    // each batch into the cleared c and adds the batch to an FP64 total
-    // (its scratch, acc64, is allocated with the geometry), which is
-    // rounded to c at the end.  Each batch's FP32 sum has ~1/B of the terms
-    // and of the magnitude, so its rounding error is ~1/B of the whole.
-    const bool batched = g->acc64 != nullptr;
-    auto begin_batch = [&]() -> spl_status {
-        if (!batched) return SPL_OK;
-        return cuda_check(cudaMemsetAsync(c, 0, nc * sizeof(float), st), "adjoint batch clear");
-    };
-    auto end_batch = [&]() {
-        if (batched) k_acc_add<<<stream_grid(nc), 256, 0, st>>>(nc, g->acc64, c);
-    };
-    if (batched && form != SPL_ADJ_GATHER) {
-        s = cuda_check(cudaMemsetAsync(g->acc64, 0, nc * sizeof(double), st), "adjoint accumulator clear");
-        if (s != SPL_OK) return s;
-        // the plane path already wrote its part into c (no side stream):
-        // it enters the total first
-        if (v0 > 0 && !overlap) end_batch();
-    }
-    // the b-fast layouts (see b_fast_target), four shifted copies each:
-    // cleared before and folded into c after each launch that reduces into
-    // them
-    const long long nx = dg.n[0], ny = dg.n[1], nz = dg.n[2], cs = (long long)dg.lay_cs;
-    auto lay_clear = [&]() -> spl_status {
-        spl_status e = SPL_OK;
-        for (int L = 0; L < 3 && e == SPL_OK; ++L)
-            e = cuda_check(cudaMemsetAsync(g->lay[L], 0, 4 * dg.lay_cs * sizeof(float), st), "adjoint layout clear");
-        return e;
-    };
-    auto lay_fold = [&]() {
-        k_fold_copies<<<stream_grid(nc), 256, 0, st>>>(c, g->lay[0], nc, cs);
-        k_fold_copies_transpose<<<dim3((unsigned)((nx + 31) / 32), (unsigned)((ny + 31) / 32),
-                                       (unsigned)(nz < 65535 ? nz : 65535)),
-                                  256, 0, st>>>(c, g->lay[1], nx, ny, nz, cs);
-        k_fold_copies_transpose<<<dim3((unsigned)((nx * ny + 31) / 32), (unsigned)((nz + 31) / 32), 1), 256, 0, st>>>(
-            c, g->lay[2], nx * ny, nz, 1, cs);
-    };
-    if (dg.kind == SPL_RAYS) {
-        for (long long r0 = 0; r0 < dg.n_rays; r0 += kAdjBatchRays) {
-            const long long r1 = r0 + kAdjBatchRays < dg.n_rays ? r0 + kAdjBatchRays : dg.n_rays;
-            if ((s = begin_batch()) != SPL_OK || (s = lay_clear()) != SPL_OK) return s;
-            k_adjoint_rays<N><<<(unsigned)((r1 - r0 + 127) / 128), 128, 0, st>>>(dg, y, g->lay[0], g->lay[1],
-                                                                                  g->lay[2], qr, r0, r1);
-            lay_fold();
-            end_batch();
-        }
-        if (batched) k_acc_store<<<stream_grid(nc), 256, 0, st>>>(nc, g->acc64, c);
-        return launch_status("adjoint launch");
-    }
-    if (form != SPL_ADJ_GATHER) {
-        const unsigned gx = (dg.nu + 15) / 16, gy = (dg.nv + 7) / 8;
-        const int per = batched ? kAdjBatchViews : kViewChunk;
-        if (dg.kind == SPL_PARALLEL) {
-            for_view_chunks(g, v0, dg.n_flat - v0, [&](const ViewChunk &ch, int n) {
-                if (s == SPL_OK) s = begin_batch();
-                k_adjoint_pviews_scatter<N, VM_FLAT><<<dim3(gx, gy, n), 128, 0, st>>>(dg, y, c, nullptr, nullptr,
-                                                                                    nullptr, qr, ch);
-                end_batch();
-            }, per);
-            for_view_chunks(g, dg.n_flat, dg.n_views - dg.n_flat, [&](const ViewChunk &ch, int n) {
-                if (s == SPL_OK) s = begin_batch();
-                if (s == SPL_OK) s = lay_clear();
-                k_adjoint_pviews_scatter<N, VM_GENERAL><<<dim3(gx, gy, n), 128, 0, st>>>(dg, y, c, g->lay[0], g->lay[1],
-                                                                                       g->lay[2], qr, ch);
-                lay_fold();
-                end_batch();
-            }, per);
-            if (batched) k_acc_store<<<stream_grid(nc), 256, 0, st>>>(nc, g->acc64, c);
-            if (overlap) {
-                const spl_status sj = cuda_check(cudaStreamWaitEvent(st, g->plane->join, 0), "join wait");
-                if (s == SPL_OK) s = sj;
-                if (s == SPL_OK) s = plane_adjoint_add(g, N, c, st);
-            }
-            if (s != SPL_OK) return s;
-        } else {
-            const int per_launch = batched ? kAdjBatchViews : dg.n_views;
-            for (int k0 = 0; k0 < dg.n_views; k0 += per_launch) {
-                const int nview = dg.n_views - k0 < per_launch ? dg.n_views - k0 : per_launch;
-                if ((s = begin_batch()) != SPL_OK || (s = lay_clear()) != SPL_OK) return s;
-                k_adjoint_views_scatter<N><<<dim3(gx, gy, nview), 128, 0, st>>>(dg, y, g->lay[0], g->lay[1], g->lay[2],
-                                                                                 qr, k0);
-                lay_fold();
-                end_batch();
-            }
-            if (batched) k_acc_store<<<stream_grid(nc), 256, 0, st>>>(nc, g->acc64, c);
-        }
-        return launch_status("adjoint launch");
-    }
+    if (scatter) return adjoint_scatter<N>(g, y, c, v0, v0 > 0, qr, st);
+    if (dg.n_rays == 0) return cuda_check(cudaMemsetAsync(c, 0, nc * sizeof(float), st), "adjoint clear");
     s = smem_attr_once((const void *)k_adjoint_bricks<N>, (int)kAdjSmem, "adjoint smem attribute");
     if (s != SPL_OK) return s;
     const int bx = (dg.n[0] + kBrick - 1) / kBrick, by = (dg.n[1] + kBrick - 1) / kBrick,

@@ -11,6 +11,7 @@ namespace spl {
 struct PlaneGroup;
 struct TableSet;
 struct LineScratch;
+struct ScatterScratch;
 }
 
 struct spl_geometry {
@@ -23,9 +24,8 @@ struct spl_geometry {
     spl::ViewConst *vconst;       // parallel geometries: per-view constants in view_order order (host)
     spl::TableSet *table;         // footprint tables (SPL_FP_TABLE), built by spl_prepare, or NULL
     double *acc64;                // FP64 accumulator of the scatter adjoint's batches (nx*ny*nz), or NULL
-    float *lay[3];                // the scatter adjoint's targets: c in the x-fast [0], y-fast [1] and z-fast [2]
-                                  // layouts, four copies each shifted by 0..3 floats (4 * dev.lay_cs floats),
-                                  // or NULL (no rays; parallel geometries whose views are all flat)
+    spl::ScatterScratch *scatter; // the scatter adjoint's layout copies of c (scatter.cu), or NULL (no rays;
+                                  // parallel geometries whose views are all flat)
     spl::LineScratch *line;       // the forward's resampled coefficients (line.cu), or NULL (not needed or too large)
 };
 
@@ -137,5 +137,15 @@ void line_create(spl_geometry *g, const double *ray_dirs);
 void line_free(LineScratch *ls);
 bool line_usable(const spl_geometry *g, int degree, cudaStream_t st);
 spl_status line_forward(const spl_geometry *g, int degree, int kahan, const float *c, float *y, cudaStream_t st);
+
+// The scatter adjoint of the same rays (scatter.cu).  scatter_rays reduces
+// the rays (views, in view order) i0 .. i1-1 into the layout copies, which are
+// clear between calls; scatter_fold moves their sum out and clears them: to
+// c, or to the FP64 total acc64 (to64), on top of nothing (src 0), what c
+// holds (1) or the FP64 total (2).
+spl_status scatter_create(spl_geometry *g, const double *ray_dirs);
+void scatter_free(ScatterScratch *S);
+spl_status scatter_rays(const spl_geometry *g, int degree, const float *y, long long i0, long long i1, cudaStream_t st);
+spl_status scatter_fold(const spl_geometry *g, int degree, int src, bool to64, float *c, cudaStream_t st);
 
 }  // namespace spl

@@ -120,12 +120,8 @@ struct ViewConst {
     // footprint-table frame (e1, e2) of H_w in the mirrored (d, a, b) frame,
     // as double-float pairs: E1[q] = sg_q e1[ax_q]
     float E1h[3], E1l[3], E2h[3], E2l[3];
-    // the scatter adjoint's copy of c: the layout whose contiguous axis is
-    // b (0 x, 1 y, 2 z fast) and the strides of (d, a, b) in it
-    int lay;
-    int Sb[3];
 };
-constexpr int kViewChunk = 192;  // views per launch (26.25 KB of parameters)
+constexpr int kViewChunk = 192;  // views per launch (23.25 KB of parameters)
 struct ViewChunk {
     ViewConst v[kViewChunk];
 };
@@ -143,13 +139,9 @@ __host__ __device__ inline void view_const(const DirSetup &ds, int view, const i
     vc.rbh = ds.rbh;
     vc.rbl = ds.rbl;
     vc.view = view;
-    // b-fast layouts: x fast [z][y][x], y fast [z][x][y], z fast [y][x][z]
-    const int sb[3][3] = {{1, n[0], n[0] * n[1]}, {n[1], 1, n[0] * n[1]}, {n[2], n[0] * n[2], 1}};
-    vc.lay = ds.ax[2];
     for (int q = 0; q < 3; ++q) {
         const int e = ds.ax[q];
         vc.S[q] = ds.sg[q] * stride[e];
-        vc.Sb[q] = ds.sg[q] * sb[vc.lay][e];
         vc.lo[q] = ds.sg[q] > 0 ? 0 : -(n[e] - 1);
         vc.hi[q] = ds.sg[q] > 0 ? n[e] - 1 : 0;
     }
@@ -196,7 +188,6 @@ struct DevGeom {
     // pair count rebuilds each ray from them
     const double *raw;
     int *err;            // device error flag (bit 0: a loop bound was reached)
-    size_t lay_cs;       // copy stride (floats) of the scatter adjoint's shifted layout copies
 };
 
 // ------------------------------------------------------------------ B-splines
@@ -851,12 +842,8 @@ __device__ __forceinline__ bool cell_march(const RaySetup &rs, int cf, int cl, c
 // flushed through sink.put(offset, in_region, F, slot) at offsets in the
 // sink's layout (sink.S0..S2, sink.off, region sink.bx; slot in 0..N is the
 // face entry's second index, so a sink may spread the face over N+1
-// independent partial sums) -- or, when the whole window lies in the region
-// and the sink has Sink::face, through one sink.put_face(base, SX, SY, F)
-// of the face's (N+1)^2 values at base + x SX + y SY -- and the window shifted
-// with selects along the event's axis.  Only the set-up of the next cell
-// is a branch.  The Gauss weights carry the factor sink.wscale() (1, or the
-// adjoint's y_r), so the values the sink receives already include it.
+// independent partial sums), and the window shifted with selects along the
+// event's axis.  Only the set-up of the next cell is a branch.
 template <int N, class Sink>
 __device__ __forceinline__ bool piece_march(const RaySetup &rs, int cf, int cl, const QuadRule &qr, Sink &sink)
 {
@@ -889,7 +876,7 @@ __device__ __forceinline__ bool piece_march(const RaySetup &rs, int cf, int cl, 
     while (true) {
         const float t1 = fminf(fminf(ta, tb), 1.0f);
         if (t1 > t0 && sink.relevant(c - N, c, QA - N, QA, QB - N, QB)) {
-            const float half = 0.5f * (t1 - t0), mid = 0.5f * (t0 + t1), hs = half * sink.wscale();
+            const float half = 0.5f * (t1 - t0), mid = 0.5f * (t0 + t1);
 #pragma unroll
             for (int q = 0; q < M; ++q) {
                 const float t = fmaf(half, qr.x[q], mid);
@@ -897,7 +884,7 @@ __device__ __forceinline__ bool piece_march(const RaySetup &rs, int cf, int cl, 
                 bweights<N>(t, wd);
                 bweights<N>(fmaf(rs.ra, t, ga), wa);
                 bweights<N>(fmaf(rs.rb, t, gb), wb);
-                const float cw = hs * qr.w[q];
+                const float cw = half * qr.w[q];
 #pragma unroll
                 for (int d = 0; d <= N; ++d) wd[d] *= cw;
                 window_update<N>(acc, wd, wa, wb);
@@ -918,23 +905,13 @@ __device__ __forceinline__ bool piece_march(const RaySetup &rs, int cf, int cl, 
             if (sink.bx.cube_in(bd, ba, bb, N)) {
                 // the whole window lies in the region (most pieces): every
                 // face entry is in, no per-entry tests
-                if constexpr (Sink::face) {
-                    float fv[N + 1][N + 1];
 #pragma unroll
-                    for (int x = 0; x <= N; ++x)
+                for (int x = 0; x <= N; ++x)
 #pragma unroll
-                        for (int y = 0; y <= N; ++y)
-                            fv[x][y] = evA ? acc[x][0][y] : (evB ? acc[x][y][0] : acc[0][x][y]);
-                    sink.template put_face<N>(base, SX, SY, fv);
-                } else {
-#pragma unroll
-                    for (int x = 0; x <= N; ++x)
-#pragma unroll
-                        for (int y = 0; y <= N; ++y) {
-                            const float v = evA ? acc[x][0][y] : (evB ? acc[x][y][0] : acc[0][x][y]);
-                            sink.put(base + (unsigned)x * SX + (unsigned)y * SY, true, v, y);
-                        }
-                }
+                    for (int y = 0; y <= N; ++y) {
+                        const float v = evA ? acc[x][0][y] : (evB ? acc[x][y][0] : acc[0][x][y]);
+                        sink.put(base + (unsigned)x * SX + (unsigned)y * SY, true, v, y);
+                    }
             } else {
                 const bool vf = evA ? sink.bx.in1(ba) : (evB ? sink.bx.in2(bb) : sink.bx.in0(bd));
                 bool vx[N + 1], vy[N + 1];

@@ -1,0 +1,117 @@
+"""The scatter adjoint (csrc/scatter.cu): the shapes at which its dispatch
+changes, against the FP64 oracle.
+
+Tolerance: a coefficient is an FP32 sum of up to a few thousand terms in
+arbitrary order; with random signs the running sum's rounding is about
+sqrt(terms) * 2^-24 of a term's size against sqrt(terms) of the sum's, plus
+about 20 roundings of a footprint: below 2e-6 in relative L2.
+"""
+import numpy as np
+import pytest
+
+from paper_2511_11078_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+TOL = 2e-6
+DIMS = (13, 21, 18)
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+
+    from paper_2511_11078_gb300 import build as B
+    from paper_2511_11078_gb300 import spl
+
+    B.build()
+    spl.lib()
+    return torch, spl
+
+
+def geom_of(orc, geo):
+    if geo.kind == "rays":
+        return orc.Geometry("rays", omega=geo.omega, s=geo.s)
+    key = "direction" if geo.kind == "parallel" else "source"
+    return orc.Geometry(geo.kind, det_center=geo.det_center, det_u=geo.det_u, det_v=geo.det_v, nu=geo.nu, nv=geo.nv,
+                        **{key: geo.src})
+
+
+def check(env, orc, geo, degrees, seed, dims=DIMS):
+    """The degrees in turn on one geometry (they share the layouts), each
+    twice: the layouts must be clear again after a call."""
+    torch, spl = env
+    rng = np.random.default_rng(seed)
+    origin = I.centred_origin(dims)
+    g = spl.Geometry(dims, origin, geo)
+    y = rng.normal(size=geo.n_rays).astype(np.float32)
+    yt = torch.tensor(y, device="cuda")
+    for degree in degrees:
+        ref = orc.adjoint(degree, dims, origin, y.astype(np.float64), geom_of(orc, geo))
+        for _ in range(2):
+            c = torch.full(g.coeff_shape, float("nan"), device="cuda")
+            spl.adjoint(g, yt, c, spl.basis(degree))
+            g.status()
+            err = np.linalg.norm(c.cpu().numpy() - ref) / np.linalg.norm(ref)
+            assert err <= TOL, (degree, err)
+
+
+@pytest.mark.parametrize("rays", [700, 25000, 90001])
+def test_rays_per_split(env, orc, rays):
+    """From too few rays to fill the GPU (8 threads a ray) to one thread a
+    ray, with flat rays and short rays whose parts are empty."""
+    rng = np.random.default_rng(rays)
+    w = I.random_directions(rng, rays)
+    w[::7, rng.integers(3)] = 0.0
+    w /= np.linalg.norm(w, axis=1, keepdims=True)
+    s = rng.uniform(-1.15, 1.15, size=(rays, 3)) * 0.5 * (np.asarray(DIMS) - 1.0)
+    check(env, orc, I.RayGeometry(w, s), (3, 0, 2, 1, 3) if rays < 10000 else (3, 1), 10)
+
+
+@pytest.mark.parametrize("views", [1, 21, 60])
+@pytest.mark.parametrize("turned", [False, True])
+@pytest.mark.parametrize("kind", ["parallel", "cone"])
+def test_views_per_split_lane_axis_and_batches(env, orc, kind, turned, views):
+    """8 threads a ray to one, both lane directions of a warp, and (60 views)
+    two batches through the FP64 total."""
+    rng = np.random.default_rng(views)
+    nu, nv = 37, 33
+    if kind == "parallel":
+        geo = I.parallel_views(I.random_directions(rng, views), nu, nv, 0.8, center=(0.3, -0.2, 0.1))
+    else:
+        geo = I.helical_cone(views, 50.0, 80.0, nu, nv, 0.9, turns=1.3, table_feed=6.0)
+    if turned:
+        geo = I.ViewGeometry(geo.kind, geo.src, geo.det_center, geo.det_v, -geo.det_u, nu, nv)
+    check(env, orc, geo, (3, 1), 20 + views)
+
+
+@pytest.mark.parametrize("dims", [(1, 1, 1), (2, 40, 3), (70, 61, 65)])
+def test_thin_and_tiled_folds(env, orc, dims):
+    """Grids thinner than a window, and one above the single-launch fold's
+    size with partial tiles."""
+    rng = np.random.default_rng(5)
+    w = I.random_directions(rng, 3000)
+    s = rng.uniform(-0.6, 0.6, size=w.shape) * np.asarray(dims)
+    check(env, orc, I.RayGeometry(w, s), (3, 2, 1, 0), 30, dims)
+
+
+def test_flat_and_general_views_in_batches(env, orc):
+    """Parallel views of all three classes (plane group, other flat views,
+    general views), in and out of the plane path, with more than one batch."""
+    torch, spl = env
+    rng = np.random.default_rng(9)
+    a = I.tilt_series(20, 25, 23, 0.9)
+    b = I.parallel_views(np.array([[0.0, np.cos(t), np.sin(t)] for t in 0.2 + 0.1 * np.arange(15)]), 25, 23, 0.9)
+    c = I.parallel_views(I.random_directions(rng, 70), 25, 23, 0.9)
+    geo = I.ViewGeometry("parallel", *[np.concatenate([getattr(p, f) for p in (a, b, c)])
+                                       for f in ("src", "det_center", "det_u", "det_v")], 25, 23)
+    origin = I.centred_origin(DIMS)
+    g = spl.Geometry(DIMS, origin, geo)
+    y = rng.normal(size=geo.n_rays).astype(np.float32)
+    ref = orc.adjoint(3, DIMS, origin, y.astype(np.float64), geom_of(orc, geo))
+    for separable in (spl.SPL_SEP_AUTO, spl.SPL_SEP_OFF):
+        out = torch.full(g.coeff_shape, float("nan"), device="cuda")
+        spl.adjoint(g, torch.tensor(y, device="cuda"), out, spl.basis(3, separable=separable))
+        g.status()
+        err = np.linalg.norm(out.cpu().numpy() - ref) / np.linalg.norm(ref)
+        assert err <= TOL, err
