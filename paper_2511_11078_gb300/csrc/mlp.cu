@@ -111,13 +111,15 @@ __global__ void __launch_bounds__(2 * kTcRows, 2) k_mlp_rows(MlpDev w, int degre
                                                       float *__restrict__ out)
 {
     extern __shared__ __align__(1024) unsigned char tc_smem[];
-    TcMlpSmem &S = *reinterpret_cast<TcMlpSmem *>(tc_smem);
+    TcMlpSmem<1> &S = *reinterpret_cast<TcMlpSmem<1> *>(tc_smem);
+    TcTile &T = S.tile[0];
+    const int tid = threadIdx.x;
     __shared__ float part[2 * kTcRows];
     tc_mlp_setup(w, S);
     unsigned phase = 0;
     const long long tiles = (count + kTcRows - 1) / kTcRows;
     for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const long long r = tile * kTcRows + tc_rowid<2>();
+        const long long r = tile * kTcRows + (tid & (kTcRows - 1));
         float x[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
         float mask = 0.0f;
         if (r < count) {
@@ -156,18 +158,18 @@ __global__ void __launch_bounds__(2 * kTcRows, 2) k_mlp_rows(MlpDev w, int degre
             }
         }
         float o;
-        const bool ok = tc_mlp_tile<2>(S, x, o, phase, part);
+        const bool ok = tc_mlp_tile<2>(S.img, T, tid, 0, true, x, o, phase, part);
         // a tensor-core wait that gave up (not expected) leaves NaN in the
         // rows of the tile, sets the network's error flag and stops the CTA
         const bool bad = __syncthreads_or(!ok);
-        if (r < count && tc_half<2>() == 0) out[r] = bad ? __int_as_float(0x7FC00000) : o * mask;
+        if (r < count && tid < kTcRows) out[r] = bad ? __int_as_float(0x7FC00000) : o * mask;
         if (bad) {
             if (threadIdx.x == 0) atomicOr(w.err, kErrTimeout);
-            tc_mlp_teardown(S, phase, true);
+            tc_mlp_teardown(S, T, phase, true);
             return;
         }
     }
-    tc_mlp_teardown(S);
+    tc_mlp_teardown(S, T);
 }
 
 static unsigned eval_blocks(long long count)
@@ -180,7 +182,7 @@ static unsigned eval_blocks(long long count)
 // dynamic shared memory of the tcgen05 row kernels (set once per process)
 template <bool FROM_WP> static spl_status rows_smem_attr()
 {
-    return smem_attr_once((const void *)k_mlp_rows<FROM_WP>, (int)sizeof(TcMlpSmem), "mlp rows smem attribute");
+    return smem_attr_once((const void *)k_mlp_rows<FROM_WP>, (int)sizeof(TcMlpSmem<1>), "mlp rows smem attribute");
 }
 
 spl_status footprint_mlp(const spl_basis_desc *b, long long count, const float *w, const float *p, float *out,
@@ -188,7 +190,7 @@ spl_status footprint_mlp(const spl_basis_desc *b, long long count, const float *
 {
     spl_status s = rows_smem_attr<true>();
     if (s != SPL_OK) return s;
-    k_mlp_rows<true><<<eval_blocks(count), 2 * kTcRows, sizeof(TcMlpSmem), st>>>(mlp_dev(b->mlp), b->degree, count, w, p,
+    k_mlp_rows<true><<<eval_blocks(count), 2 * kTcRows, sizeof(TcMlpSmem<1>), st>>>(mlp_dev(b->mlp), b->degree, count, w, p,
                                                                              out);
     return cuda_check(cudaGetLastError(), "mlp footprint launch");
 }
@@ -198,32 +200,34 @@ __global__ void __launch_bounds__(2 * kTcRows, 2) k_train_forward(MlpDev w, int 
                                                                float *act, float *out, int max_batch)
 {
     extern __shared__ __align__(1024) unsigned char tc_smem[];
-    TcMlpSmem &S = *reinterpret_cast<TcMlpSmem *>(tc_smem);
+    TcMlpSmem<1> &S = *reinterpret_cast<TcMlpSmem<1> *>(tc_smem);
+    TcTile &T = S.tile[0];
+    const int tid = threadIdx.x;
     __shared__ float part[2 * kTcRows];
     tc_mlp_setup(w, S);
     unsigned phase = 0;
     const size_t L = (size_t)max_batch * 64;
     const int tiles = (B + kTcRows - 1) / kTcRows;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const int r = tile * kTcRows + tc_rowid<2>();
+        const int r = tile * kTcRows + (tid & (kTcRows - 1));
         float x[5];
 #pragma unroll
         for (int e = 0; e < 5; ++e) x[e] = r < B ? X[5 * r + e] : 0.0f;
         const TcSave sv{act, act + L, act + 2 * L, act + 3 * L, act + 4 * L, act + 5 * L, r < B ? r : -1};
         float o;
-        const bool ok = tc_mlp_tile<2, true>(S, x, o, phase, part, &sv);
+        const bool ok = tc_mlp_tile<2, true>(S.img, T, tid, 0, true, x, o, phase, part, &sv);
         // a tensor-core wait that gave up (not expected) leaves NaN outputs,
         // so the loss and the gradient come out NaN, and sets the network's
         // error flag
         const bool bad = __syncthreads_or(!ok);
-        if (r < B && tc_half<2>() == 0) out[r] = bad ? __int_as_float(0x7FC00000) : o;
+        if (r < B && tid < kTcRows) out[r] = bad ? __int_as_float(0x7FC00000) : o;
         if (bad) {
             if (threadIdx.x == 0) atomicOr(w.err, kErrTimeout);
-            tc_mlp_teardown(S, phase, true);
+            tc_mlp_teardown(S, T, phase, true);
             return;
         }
     }
-    tc_mlp_teardown(S);
+    tc_mlp_teardown(S, T);
 }
 
 __device__ __forceinline__ float silu_grad(float z)
@@ -459,11 +463,11 @@ static spl_status grad_impl(spl_mlp *m, int B, const float *X, const float *Y, f
 {
     const MlpDev w = mlp_dev(m);
     {
-        spl_status s = smem_attr_once((const void *)k_train_forward, (int)sizeof(TcMlpSmem),
+        spl_status s = smem_attr_once((const void *)k_train_forward, (int)sizeof(TcMlpSmem<1>),
                                       "train forward smem attribute");
         if (s != SPL_OK) return s;
     }
-    k_train_forward<<<eval_blocks(B), 2 * kTcRows, sizeof(TcMlpSmem), st>>>(w, B, X, m->act, m->out, m->max_batch);
+    k_train_forward<<<eval_blocks(B), 2 * kTcRows, sizeof(TcMlpSmem<1>), st>>>(w, B, X, m->act, m->out, m->max_batch);
     const int bblocks = (B + kBwdRows - 1) / kBwdRows;
     k_train_backward<<<bblocks, kBwdThreads, 0, st>>>(m->master, B, Y, m->act, m->out, m->dz, m->dz4, m->loss_part,
                                                       m->max_batch);
@@ -753,7 +757,7 @@ extern "C" spl_status spl_mlp_eval(const spl_mlp *m, long long count, const floa
     if (!feat_dev || !out_dev) return fail(SPL_ERR_ARG, "NULL array");
     spl_status s = rows_smem_attr<false>();
     if (s != SPL_OK) return s;
-    k_mlp_rows<false><<<eval_blocks(count), 2 * kTcRows, sizeof(TcMlpSmem), (cudaStream_t)stream>>>(
+    k_mlp_rows<false><<<eval_blocks(count), 2 * kTcRows, sizeof(TcMlpSmem<1>), (cudaStream_t)stream>>>(
         mlp_dev(m), m->degree, count, feat_dev, nullptr, out_dev);
     return cuda_check(cudaGetLastError(), "mlp eval launch");
 }

@@ -1,12 +1,14 @@
 // mlp_project.cu -- forward projection and adjoint with the learned
 // footprint f_theta in place of the exact one (Algorithm 2 with f_theta*).
 //
-// A CTA owns 128 rays (an 8 x 16 detector tile).  It walks the rays' slabs
+// A group of 128 threads owns 128 rays (an 8 x 16 detector tile); a CTA is two
+// groups that share the network's operands and nothing else, two CTAs per SM.
+// A group walks its rays' slabs
 // in lock-step rounds: in each round every thread sweeps one slab of its ray
 // in pair-enumeration mode (the same dominant-axis slab march and window as
 // the exact path, so the pair set is the exact support of every basis --
 // f_theta is kept only where the ray meets the basis) and appends one 16-bit
-// row per pair to the CTA's queue in shared memory.  The CTA then drains the
+// row per pair to the group's queue in shared memory.  The group then drains the
 // queue in tiles of 128 rows through the tcgen05 network (one row per
 // thread, accumulator in TMEM) and accumulates c * f_theta per ray (forward,
 // shared-memory atomics) or y_r * f_theta per coefficient (adjoint, float
@@ -15,7 +17,8 @@
 
 namespace spl {
 
-constexpr int kMlpThreads = kTcRows;
+constexpr int kMlpThreads = kTcRows;  // threads (rays) of a group
+constexpr int kMlpGroups = 2;
 
 // most pairs one slab can produce: the initial (N+1)^2 window plus N+1 per
 // window shift; a transverse axis crosses at most N+2 knot planes in a slab
@@ -105,30 +108,43 @@ __device__ __forceinline__ void decode_row(const MlpRayTab &T, unsigned e, int &
     x[4] = fmaf(B.y, Pa, B.z * Pb);
 }
 
-template <int N> constexpr int mlp_queue_bytes() { return (kMlpThreads * PairCap<N>::value * 2 + 15) / 16 * 16; }
-template <int N> constexpr size_t mlp_views_smem()
-{
-    return sizeof(TcMlpSmem) + sizeof(MlpRayTab) + (size_t)mlp_queue_bytes<N>();
-}
+template <int N> struct __align__(16) MlpGroup {
+    MlpRayTab tab;
+    uint16_t q[(kMlpThreads * PairCap<N>::value + 7) / 8 * 8];
+};
+template <int N> struct MlpSmem {
+    TcMlpSmem<kMlpGroups> tc;
+    MlpGroup<N> group[kMlpGroups];
+};
 
+// Bound by issue latency at 16 warps per SM: 54 % issue, MUFU 38 %, FMA pipe
+// 45 %, tensor pipe 15 % (one view of the 256^3 cone).  6 such views: 282 ms
+// (A), 274 (A^T) with one group of 168 registers per CTA, three CTAs per SM,
+// and a reciprocal per SiLU; 239 with the shared reciprocal (silu4), 228 and
+// 225 with two groups sharing the operands at 128 registers, 16 warps per SM.
+// Measured and not kept: both halves of a row loaded before either is
+// evaluated, with the ray's enumeration state parked in TMEM (228).
+//
 // ADJ = false: y = A_theta c ; ADJ = true: c += A_theta^T y (c zeroed by the host)
 template <int N, bool ADJ>
-__global__ void __launch_bounds__(kMlpThreads, 3) k_mlp_views(DevGeom g, MlpDev wts, const float *__restrict__ cin,
-                                                           float *__restrict__ yout, const float *__restrict__ yin,
-                                                           float *__restrict__ cout, QuadRule qr)
+__global__ void __launch_bounds__(kMlpThreads *kMlpGroups, 2)
+    k_mlp_views(DevGeom g, MlpDev wts, const float *__restrict__ cin, float *__restrict__ yout, const float *__restrict__ yin,
+                float *__restrict__ cout, QuadRule qr)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    TcMlpSmem &S = *reinterpret_cast<TcMlpSmem *>(smem);
-    MlpRayTab &T = *reinterpret_cast<MlpRayTab *>(smem + sizeof(TcMlpSmem));
-    uint16_t *q = reinterpret_cast<uint16_t *>(smem + sizeof(TcMlpSmem) + sizeof(MlpRayTab));
+    MlpSmem<N> &M = *reinterpret_cast<MlpSmem<N> *>(smem);
+    const int grp = threadIdx.x / kMlpThreads, tid = threadIdx.x % kMlpThreads, lane = tid & 31, wid = tid >> 5;
+    const int bar = 1 + grp;
+    TcTile &tile = M.tc.tile[grp];
+    MlpRayTab &T = M.group[grp].tab;
+    uint16_t *q = M.group[grp].q;
     constexpr int cap = kMlpThreads * PairCap<N>::value;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid == 0) {
         T.count = 0;
         T.rounds = 0;
     }
-    tc_mlp_setup(wts, S);  // ends with a CTA barrier
-    const int iu = blockIdx.x * 8 + (lane & 7), iv = blockIdx.y * 16 + wid * 4 + (lane >> 3);
+    tc_mlp_setup(wts, M.tc);  // ends with a CTA barrier
+    const int iu = (blockIdx.x * kMlpGroups + grp) * 8 + (lane & 7), iv = blockIdx.y * 16 + wid * 4 + (lane >> 3);
     const int k = blockIdx.z;
     const bool valid = iu < g.nu && iv < g.nv;
     const long long ray = ((long long)k * g.nv + (valid ? iv : 0)) * g.nu + (valid ? iu : 0);
@@ -160,11 +176,14 @@ __global__ void __launch_bounds__(kMlpThreads, 3) k_mlp_views(DevGeom g, MlpDev 
     T.yv[tid] = yr;
     const int nslab = rs.j1 - rs.j0 + 1;
     if (nslab > 0) atomicMax(&T.rounds, nslab);
-    __syncthreads();
+    tc::bar_sync(bar, kMlpThreads);
     const int rounds = T.rounds;
     unsigned phase = 0;
-    bool ok = true, stop = false, timeout = false;
-    for (int round = 0; round < rounds && !stop; ++round) {
+    // tok: this thread's tensor-core waits; one that gives up (not expected)
+    // raises the group's stop flag, which every thread reads after the same
+    // barrier
+    bool ok = true, tok = true, timeout = false;
+    for (int round = 0; round < rounds; ++round) {
         if (round < nslab) {
             MlpSinkN<N> sk;
             sk.q = q;
@@ -184,7 +203,7 @@ __global__ void __launch_bounds__(kMlpThreads, 3) k_mlp_views(DevGeom g, MlpDev 
             ok &= slab_pairs<N, MlpSinkN<N>>(rs, sk.j, qr, sk);
             ok &= !sk.bad;
         }
-        __syncthreads();
+        tc::bar_sync(bar, kMlpThreads);
         int n = T.count;
         if (n > cap) {
             ok = false;
@@ -200,25 +219,23 @@ __global__ void __launch_bounds__(kMlpThreads, 3) k_mlp_views(DevGeom g, MlpDev 
                 if (!ADJ) cv = __ldg(cin + addr);
             }
             float o;
-            const bool tok = tc_mlp_tile<1>(S, x, o, phase);
-            if (__syncthreads_or(!tok)) {  // a tensor-core wait gave up (not expected)
-                timeout = true;
-                stop = true;
-                break;
-            }
-            if (r < n) {
+            tok = tc_mlp_tile<1>(M.tc.img, tile, tid, bar, tok, x, o, phase);
+            if (r < n && tok) {
                 if (ADJ) atomicAdd(cout + addr, T.yv[l] * o);
                 else atomicAdd(&T.acc[l], cv * o);
             }
         }
-        __syncthreads();  // queue drained
+        if (!tok) tile.stop = 1;
+        tc::bar_sync(bar, kMlpThreads);  // queue drained
+        timeout = tile.stop != 0;
         if (tid == 0) T.count = 0;
-        __syncthreads();
+        if (timeout) break;
+        tc::bar_sync(bar, kMlpThreads);
     }
     if (!ok) atomicOr(g.err, kErrStepCap);
     if (timeout && tid == 0) atomicOr(g.err, kErrTimeout);
     if (!ADJ && valid) yout[ray] = timeout ? __int_as_float(0x7FC00000) : T.acc[tid];
-    tc_mlp_teardown(S, phase, timeout);
+    tc_mlp_teardown(M.tc, tile, phase, timeout);
 }
 
 template <int N, bool ADJ>
@@ -227,13 +244,13 @@ static spl_status launch_mlp_views(const spl_geometry *g, const spl_mlp *m, cons
 {
     const DevGeom &dg = g->dev;
     if (dg.n_rays == 0) return SPL_OK;
-    const size_t sm = mlp_views_smem<N>();
+    constexpr size_t sm = sizeof(MlpSmem<N>);
     {
         spl_status s = smem_attr_once((const void *)k_mlp_views<N, ADJ>, (int)sm, "mlp smem attribute");
         if (s != SPL_OK) return s;
     }
-    dim3 grid((dg.nu + 7) / 8, (dg.nv + 15) / 16, dg.n_views);
-    k_mlp_views<N, ADJ><<<grid, kMlpThreads, sm, st>>>(dg, mlp_dev(m), cin, yout, yin, cout, quad_rule(N));
+    dim3 grid((dg.nu + 8 * kMlpGroups - 1) / (8 * kMlpGroups), (dg.nv + 15) / 16, dg.n_views);
+    k_mlp_views<N, ADJ><<<grid, kMlpThreads * kMlpGroups, sm, st>>>(dg, mlp_dev(m), cin, yout, yin, cout, quad_rule(N));
     return cuda_check(cudaGetLastError(), "mlp projector launch");
 }
 

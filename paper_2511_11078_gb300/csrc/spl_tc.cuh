@@ -2,15 +2,16 @@
 // tensor cores: tcgen05.mma with operands in shared memory and the FP32
 // accumulator in tensor memory (TMEM).
 //
-// A CTA evaluates tiles of 128 rows, with one thread per row (128 threads)
-// or two (256 threads, each taking half of the row's 64 columns).  Each
-// layer is one M=128 x N=64 product: the threads write their parts of the A
-// operand (BF16) to shared memory, one thread issues the MMAs, the tensor
-// core accumulates the 128 x 64 FP32 result in 64 TMEM columns, and every
-// thread reads its part back with tcgen05.ld (TMEM lane = row), applies
-// SiLU and writes the next layer's A operand.  The MMAs take no issue slots
-// of the other threads and no registers: what is left to the threads is
-// SiLU, the BF16 packing and the 64 -> 1 output layer.
+// A group of 128 or 256 threads (a CTA, or a part of one) evaluates tiles of
+// 128 rows, with one thread per row or two (each taking half of the row's 64
+// columns).  Each layer is one M=128 x N=64 product: the threads write their
+// parts of the A operand (BF16) to shared memory, one thread issues the MMAs,
+// the tensor core accumulates the 128 x 64 FP32 result in 64 TMEM columns,
+// and every thread reads its part back with tcgen05.ld (TMEM lane = row),
+// applies SiLU and writes the next layer's A operand.  The MMAs take no issue
+// slots of the other threads and no registers: what is left to the threads is
+// SiLU, the BF16 packing and the 64 -> 1 output layer.  A layer's barrier,
+// MMA and TMEM round trip are hidden by the other groups of the SM.
 //
 // Precision contract (the one the oracle emulates): layers 2 and 3 multiply
 // BF16 weights with the BF16-rounded activations, accumulating in FP32;
@@ -81,10 +82,10 @@ __device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count)
 // Wait for the phase with the given parity to complete; gives up (false)
 // after a bounded number of polls.
 constexpr unsigned kWaitPolls = 1u << 20;
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity)
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, unsigned polls = kWaitPolls)
 {
     const uint32_t a = saddr(bar);
-    for (unsigned it = 0; it < kWaitPolls; ++it) {
+    for (unsigned it = 0; it < polls; ++it) {
         uint32_t done;
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -95,6 +96,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity)
         if (done) return true;
     }
     return false;
+}
+
+// barrier over `threads` threads (a group of the CTA's warps), reached by
+// each thread on its own (not .aligned)
+__device__ __forceinline__ void bar_sync(int id, int threads)
+{
+    asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -137,11 +145,8 @@ __device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.
 
 }  // namespace tc
 
-constexpr int kTcRows = 128;  // rows of a tile (threads of a CTA: 128 or 256)
+constexpr int kTcRows = 128;  // rows of a tile
 constexpr int kTcCols = 64;   // TMEM columns of the accumulator (N = 64, FP32)
-// TMEM allocation never waits: every CTA that allocates holds at least
-// sizeof(TcMlpSmem) (49 KB) of shared memory, so at most 4 of them are
-// resident on an SM (228 KB), and 4 x 64 columns stay below the SM's 512.
 
 // The network in the tile's operand layout (built once per parameter
 // update in global memory, copied into every CTA's shared memory).
@@ -156,19 +161,31 @@ struct __align__(16) TcMlpImage {
     float pad[3];
 };
 
-// Shared memory of a CTA: the network image and the operands of one tile.
-struct __align__(1024) TcMlpSmem {
-    TcMlpImage img;
-    uint8_t a2[kTcRows * 64 * 2];  // A of layers 2 and 3: 128 x 64
-    uint8_t a1[kTcRows * 16 * 2];  // A of layer 1: 128 x 16
-    uint32_t tmem;
+// A group's operands: A of layers 2 and 3 (128 x 64), whose first 4 KB also
+// hold A of layer 1 (128 x 16; read before layer 2's is written).
+struct __align__(128) TcTile {
+    uint8_t a2[kTcRows * 64 * 2];
+    uint32_t tmem;   // the group's 64 accumulator columns
+    int stop;        // a completion wait of the group gave up
     uint64_t mbar;
+};
+// Shared memory of a CTA: the network image and one tile per group.
+template <int GROUPS> struct __align__(1024) TcMlpSmem {
+    TcMlpImage img;
+    TcTile tile[GROUPS];
 };
 
 static_assert(sizeof(TcMlpImage) % 16 == 0, "the image is copied in 16-byte units");
-static_assert(offsetof(TcMlpSmem, a2) % 16 == 0 && offsetof(TcMlpSmem, a1) % 16 == 0,
+static_assert(offsetof(TcMlpSmem<2>, tile) % 16 == 0 && sizeof(TcTile) % 16 == 0,
               "operands start on 16-byte boundaries (shared-memory descriptors)");
-static_assert(5 * (sizeof(TcMlpSmem) + 1024) > 228 * 1024, "at most 4 allocating CTAs per SM");
+// TMEM allocation never waits: a CTA holds at least sizeof(TcMlpSmem<GROUPS>)
+// of shared memory for 64 GROUPS columns, so the CTAs of an SM (228 KB) stay
+// below its 512 columns.
+template <int GROUPS> constexpr size_t tc_max_cols()
+{
+    return 228 * 1024 / (sizeof(TcMlpSmem<GROUPS>) + 1024) * (kTcCols * GROUPS);
+}
+static_assert(tc_max_cols<1>() <= 512 && tc_max_cols<2>() <= 512, "TMEM columns of the CTAs an SM can hold");
 
 // byte offset of element (row, k) in an operand of R rows (K-major, no swizzle)
 __host__ __device__ constexpr uint32_t kmaj_off(int R, int row, int k)
@@ -230,62 +247,77 @@ __device__ __forceinline__ void tc_mlp_image(const float *__restrict__ P, TcMlpI
     }
 }
 
-// The network image into shared memory (16-byte copies), the completion
-// barrier and the TMEM accumulator.  Called by all threads of the CTA; ends
-// with a CTA barrier.
-__device__ __forceinline__ void tc_mlp_setup(const MlpDev &w, TcMlpSmem &S)
+// The network image into shared memory (16-byte copies), the groups'
+// completion barriers and TMEM accumulators.  Called by all threads of the
+// CTA; ends with a CTA barrier.
+template <int GROUPS>
+__device__ __forceinline__ void tc_mlp_setup(const MlpDev &w, TcMlpSmem<GROUPS> &S)
 {
     const int tid = threadIdx.x;
     const uint4 *src = reinterpret_cast<const uint4 *>(w.tc_img);
     uint4 *dst = reinterpret_cast<uint4 *>(&S.img);
     for (int i = tid; i < (int)(sizeof(TcMlpImage) / 16); i += blockDim.x) dst[i] = __ldg(src + i);
     if (tid == 0) {
-        tc::mbar_init(&S.mbar, 1);
+#pragma unroll
+        for (int g = 0; g < GROUPS; ++g) {
+            tc::mbar_init(&S.tile[g].mbar, 1);
+            S.tile[g].stop = 0;
+        }
         tc::fence_mbar_init();
     }
-    if (tid < 32) tc::alloc(&S.tmem, kTcCols);
+    if (tid < 32) tc::alloc(&S.tile[0].tmem, kTcCols * GROUPS);
     tc::fence_proxy_async();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
+    if (GROUPS > 1) {
+        if (tid == 0)
+#pragma unroll
+            for (int g = 1; g < GROUPS; ++g) S.tile[g].tmem = S.tile[0].tmem + (uint32_t)(g * kTcCols);
+        __syncthreads();
+    }
 }
 
-// Release the TMEM accumulator (after a CTA barrier).  When a completion
-// wait gave up (`pending`), the last committed MMAs may still be running:
-// wait once more, bounded, for the phase of the last commit (`phase` is the
-// parity the next wait would use) before the columns are freed.
-__device__ __forceinline__ void tc_mlp_teardown(TcMlpSmem &S, unsigned phase = 0u, bool pending = false)
+// Release the TMEM accumulators.  Called by all threads of the CTA.  When a
+// completion wait gave up (`pending`), the group's last committed MMAs may
+// still be running: wait once more, bounded, for the phase of the last commit
+// (`phase` is the parity the next wait would use) before the columns are
+// freed.
+template <int GROUPS>
+__device__ __forceinline__ void tc_mlp_teardown(TcMlpSmem<GROUPS> &S, TcTile &T, unsigned phase = 0u, bool pending = false)
 {
-    if (pending) tc::mbar_wait(&S.mbar, phase ^ 1u);
+    if (pending) tc::mbar_wait(&T.mbar, phase ^ 1u);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    if (threadIdx.x < 32) tc::dealloc(S.tmem, kTcCols);
+    if (threadIdx.x < 32) tc::dealloc(S.tile[0].tmem, kTcCols * GROUPS);
 }
 
-// One MMA layer: D = sum over k-steps of A * B, plus the bias step; thread 0
-// issues, everyone waits for completion.  nk: K=16 steps of the A operand
+// One MMA layer: D = sum over k-steps of A * B, plus the bias step; the
+// group's thread `tid` 0 issues, everyone waits for completion (a group that
+// has given up before does not wait again).  nk: K=16 steps of the A operand
 // (A columns 16 s .. 16 s + 15 at a + s * (rows / 8) * 256 bytes, B at
-// b + s * 8 * 256).
-__device__ __forceinline__ bool tc_layer(TcMlpSmem &S, const uint8_t *a, const uint8_t *b, int nk, int layer,
-                                         unsigned &phase)
+// b + s * 8 * 256).  bar: the group's barrier, of `threads` threads.
+__device__ __forceinline__ bool tc_layer(const TcMlpImage &img, TcTile &T, int tid, int bar, int threads, const uint8_t *b,
+                                         int nk, int layer, unsigned &phase, bool ok)
 {
     constexpr uint32_t idesc = tc::idesc_bf16(kTcRows, 64);
     tc::fence_proxy_async();
     tc::fence_before();
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    tc::bar_sync(bar, threads);
+    if (tid == 0) {
         tc::fence_after();
-        const uint32_t sa = tc::saddr(a), sb = tc::saddr(b);
+        const uint32_t sa = tc::saddr(T.a2), sb = tc::saddr(b);
         for (int s = 0; s < nk; ++s)
-            tc::mma(S.tmem, tc::desc(sa + s * (kTcRows / 8) * 256, (kTcRows / 8) * 128, 128),
+            tc::mma(T.tmem, tc::desc(sa + s * (kTcRows / 8) * 256, (kTcRows / 8) * 128, 128),
                     tc::desc(sb + s * 8 * 256, 8 * 128, 128), idesc, s > 0);
-        tc::mma(S.tmem, tc::desc(tc::saddr(S.img.one), (kTcRows / 8) * 128, 128),
-                tc::desc(tc::saddr(S.img.bias[layer]), 8 * 128, 128), idesc, 1);
-        tc::commit(&S.mbar);
+        tc::mma(T.tmem, tc::desc(tc::saddr(img.one), (kTcRows / 8) * 128, 128),
+                tc::desc(tc::saddr(img.bias[layer]), 8 * 128, 128), idesc, 1);
+        tc::commit(&T.mbar);
     }
-    const bool ok = tc::mbar_wait(&S.mbar, phase);
+    ok = tc::mbar_wait(&T.mbar, phase, ok ? tc::kWaitPolls : 1u) && ok;
     phase ^= 1u;
+    __syncwarp();  // tcgen05.ld is warp-wide
     tc::fence_after();
     return ok;
 }
@@ -295,83 +327,91 @@ __device__ __forceinline__ bool tc_layer(TcMlpSmem &S, const uint8_t *a, const u
 // w % 4, and take columns 0..31 and 32..63 of its rows): half the serial
 // work per thread, for batches too small to fill the GPU with 128-row tiles.
 // (threadIdx.x & 96 is the warp's TMEM lane quarter, 32 * (warp % 4).)
-template <int TPR> __device__ __forceinline__ int tc_rowid() { return threadIdx.x & (kTcRows - 1); }
-template <int TPR> __device__ __forceinline__ int tc_half() { return TPR == 1 ? 0 : (int)(threadIdx.x >> 7); }
 
-// This thread's columns of its row of the accumulator after a layer:
-// 64 / TPR FP32 values, from column 64 / TPR * half.
-template <int TPR>
-__device__ __forceinline__ void tc_row(const TcMlpSmem &S, float (&z)[64 / TPR])
+// Columns C0 .. C0 + 31 of this thread's row of the accumulator.
+template <int C0>
+__device__ __forceinline__ void tc_cols(uint32_t tmem, float (&z)[32])
 {
-    const uint32_t t = S.tmem + ((uint32_t)(threadIdx.x & 96) << 16) + (uint32_t)(tc_half<TPR>() * 32);
-    tc::ld32<0>(t, z);
-    if (TPR == 1) tc::ld32<(TPR == 1 ? 32 : 0)>(t + 32, z);
+    tc::ld32<0>(tmem + ((uint32_t)(threadIdx.x & 96) << 16) + (uint32_t)C0, z);
     tc::wait_ld();
 }
 
-// SiLU of two values with the reciprocal 1 / d, d = 1 + 2^(-z log2 e), by
-// Newton-Raphson steps r <- r + r (1 - d r) on the FMA pipe instead of the
-// MUFU.  The seed negates the IEEE-754 exponent by an integer subtraction
-// from the bit pattern of 2^127 (bits(2^127) - bits(d) ~ bits(1/d) for
-// d >= 1) and lies within 12.5 % above 1/d; each step squares the relative
-// error, so three take it to 0.125^8 ~ 6e-8.  d is capped at 2^126
-// (z < -87, where SiLU is below 1e-36 either way) so the seed stays normal.
-__device__ __forceinline__ float2 silu2_nr(float2 z)
+// SiLU of four values, z / d with d = 1 + 2^(-z log2 e), through one MUFU
+// reciprocal of the four denominators' product instead of one each: with
+// P = (d0 d2, d1 d3) and r = 1 / (P.x P.y), 1 / d0 = (r P.y) d2 and so on.
+// GB300's MUFU takes base-2 exponentials at twice the rate of reciprocals, so
+// a reciprocal per value was two thirds of its work (a quarter of them by
+// Newton steps on the FMA pipe); now it is a fifth.  Each reciprocal carries
+// four more roundings of 2^-24 than rcp(d) itself, far below the BF16 rounding
+// that follows.  Values below -87 can take the product out of range (`over`
+// collects the largest; the caller then repeats its values with silu_safe).
+__device__ __forceinline__ void silu4(const float (&z)[4], float (&h)[4], float &over)
 {
     constexpr float kNegLog2e = -1.4426950408889634f;
-    const float2 m = __fmul2_rn(z, make_float2(kNegLog2e, kNegLog2e));
-    float2 d = __fadd2_rn(make_float2(ex2_approx(m.x), ex2_approx(m.y)), make_float2(1.0f, 1.0f));
-    d.x = fminf(d.x, 0x1p126f);
-    d.y = fminf(d.y, 0x1p126f);
-    float2 r = make_float2(__int_as_float(0x7F000000 - __float_as_int(d.x)),
-                           __int_as_float(0x7F000000 - __float_as_int(d.y)));
-    const float2 nd = __fmul2_rn(d, make_float2(-1.0f, -1.0f));
-#pragma unroll
-    for (int it = 0; it < 3; ++it) r = __ffma2_rn(r, __ffma2_rn(nd, r, make_float2(1.0f, 1.0f)), r);
-    return __fmul2_rn(z, r);
+    const float2 one = make_float2(1.0f, 1.0f), k = make_float2(kNegLog2e, kNegLog2e);
+    const float2 za = make_float2(z[0], z[1]), zb = make_float2(z[2], z[3]);
+    const float2 ma = __fmul2_rn(za, k), mb = __fmul2_rn(zb, k);
+    const float2 da = __fadd2_rn(make_float2(ex2_approx(ma.x), ex2_approx(ma.y)), one);
+    const float2 db = __fadd2_rn(make_float2(ex2_approx(mb.x), ex2_approx(mb.y)), one);
+    const float2 P = __fmul2_rn(da, db);
+    const float q = P.x * P.y, r = rcp_approx(q);
+    over = fmaxf(over, q);
+    const float2 R = make_float2(r * P.y, r * P.x);
+    const float2 ha = __fmul2_rn(za, __fmul2_rn(R, db)), hb = __fmul2_rn(zb, __fmul2_rn(R, da));
+    h[0] = ha.x;
+    h[1] = ha.y;
+    h[2] = hb.x;
+    h[3] = hb.y;
 }
-
-// The SiLU pairs of a row (p = 0..31 per layer) are split between the MUFU
-// reciprocal and the Newton form so that the MUFU queue and the FMA pipe
-// share the work: pair p takes the Newton form when bit (p mod 8) of
-// kTcNrMask is set.
-#ifndef SPL_TC_NR_MASK
-#define SPL_TC_NR_MASK 0x11
-#endif
-constexpr unsigned kTcNrMask = SPL_TC_NR_MASK;
-__device__ __forceinline__ float2 tc_silu2(int p, float2 z)
+constexpr float kSiluOver = 0x1p125f;  // above it the reciprocal is not a normal number
+// one value at a time; d is capped where SiLU is below 1e-36 either way
+__device__ __forceinline__ float silu_safe(float z)
 {
-    return ((kTcNrMask >> (p & 7)) & 1u) ? silu2_nr(z) : silu2(z);
+    return z * rcp_approx(fminf(1.0f + ex2_approx(-1.4426950408889634f * z), 0x1p126f));
 }
 
-// SiLU of this thread's columns, rounded to BF16 into its part of the row
-// of the A operand of the next layer (and, with SAVE, z and the rounded
+// SiLU of 32 columns of a row from column c0, rounded to BF16 into the row of
+// the A operand of the next layer (and, with SAVE, z and the rounded
 // activations to zb / hb, which point at the row).
-template <int TPR, bool SAVE>
-__device__ __forceinline__ void tc_silu_store(TcMlpSmem &S, const float (&z)[64 / TPR], float *zb, float *hb)
+template <bool SAVE>
+__device__ __forceinline__ void tc_silu_store(TcTile &T, int m, int c0, const float (&z)[32], float *zb, float *hb)
 {
-    constexpr int NC = 64 / TPR;  // columns of this thread
-    const int m = tc_rowid<TPR>(), c0 = NC * tc_half<TPR>();
     if (SAVE) {
 #pragma unroll
-        for (int k = 0; k < NC; k += 4)
+        for (int k = 0; k < 32; k += 4)
             *reinterpret_cast<float4 *>(zb + c0 + k) = make_float4(z[k], z[k + 1], z[k + 2], z[k + 3]);
     }
+    float over = 0.0f;
 #pragma unroll
-    for (int j = 0; j < NC / 8; ++j) {
+    for (int j = 0; j < 4; ++j) {
         uint32_t w[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float2 h = tc_silu2(4 * j + q, make_float2(z[8 * j + 2 * q], z[8 * j + 2 * q + 1]));
-            w[q] = pack_bf16(h.x, h.y);
+        for (int q = 0; q < 2; ++q) {
+            const float zz[4] = {z[8 * j + 4 * q], z[8 * j + 4 * q + 1], z[8 * j + 4 * q + 2], z[8 * j + 4 * q + 3]};
+            float h[4];
+            silu4(zz, h, over);
+            w[2 * q] = pack_bf16(h[0], h[1]);
+            w[2 * q + 1] = pack_bf16(h[2], h[3]);
         }
-        *reinterpret_cast<uint4 *>(S.a2 + kmaj_off(kTcRows, m, c0 + 8 * j)) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4 *>(T.a2 + kmaj_off(kTcRows, m, c0 + 8 * j)) = make_uint4(w[0], w[1], w[2], w[3]);
         if (SAVE) {
             float4 *d = reinterpret_cast<float4 *>(hb + c0 + 8 * j);
             d[0] = make_float4(__uint_as_float(w[0] << 16), __uint_as_float(w[0] & 0xFFFF0000u),
                                __uint_as_float(w[1] << 16), __uint_as_float(w[1] & 0xFFFF0000u));
             d[1] = make_float4(__uint_as_float(w[2] << 16), __uint_as_float(w[2] & 0xFFFF0000u),
                                __uint_as_float(w[3] << 16), __uint_as_float(w[3] & 0xFFFF0000u));
+        }
+    }
+    if (over > kSiluOver) {
+        // a value far below zero (not met in practice): again, one by one
+#pragma unroll 1
+        for (int c = 0; c < 32; ++c) {
+            float v = z[0];
+#pragma unroll
+            for (int e = 1; e < 32; ++e) v = e == c ? z[e] : v;
+            const uint16_t b = bf16_bits_rn(silu_safe(v));
+            *reinterpret_cast<uint16_t *>(T.a2 + kmaj_off(kTcRows, m, c0 + c)) = b;
+            if (SAVE) hb[c0 + c] = __uint_as_float((uint32_t)b << 16);
         }
     }
 }
@@ -385,19 +425,53 @@ struct TcSave {
     int row;
 };
 
+// Output layer over 32 columns of a row from column c0: o += w4 . SiLU(z).
+template <bool SAVE>
+__device__ __forceinline__ float tc_output(const TcMlpImage &img, int c0, const float (&z)[32], bool save, float *zb, float *hb)
+{
+    float2 acc = make_float2(0.0f, 0.0f);
+    float over = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 32; k += 4) {
+        if (SAVE && save) *reinterpret_cast<float4 *>(zb + c0 + k) = make_float4(z[k], z[k + 1], z[k + 2], z[k + 3]);
+        const float zz[4] = {z[k], z[k + 1], z[k + 2], z[k + 3]};
+        float h[4];
+        silu4(zz, h, over);
+        if (SAVE && save) *reinterpret_cast<float4 *>(hb + c0 + k) = make_float4(h[0], h[1], h[2], h[3]);
+        const float4 w = *reinterpret_cast<const float4 *>(img.w4 + c0 + k);
+        acc = __ffma2_rn(make_float2(h[0], h[1]), make_float2(w.x, w.y), acc);
+        acc = __ffma2_rn(make_float2(h[2], h[3]), make_float2(w.z, w.w), acc);
+    }
+    float o = acc.x + acc.y;
+    if (over > kSiluOver) {  // as in tc_silu_store
+        o = 0.0f;
+#pragma unroll 1
+        for (int c = 0; c < 32; ++c) {
+            float v = z[0];
+#pragma unroll
+            for (int e = 1; e < 32; ++e) v = e == c ? z[e] : v;
+            const float h = silu_safe(v);
+            o = fmaf(h, img.w4[c0 + c], o);
+            if (SAVE && save) hb[c0 + c] = h;
+        }
+    }
+    return o;
+}
+
 // f_theta of this thread's row x (5 features) in a tile of 128 rows; every
-// thread of the CTA (128 * TPR) calls it, the TPR threads of a row with the
-// same x.  Returns false if a tensor-core wait gave up (the output is then
-// meaningless).  The output is valid in every thread of the row.  part:
-// 2 x 128 floats of shared memory for combining the halves of the output
+// thread of the group (128 * TPR; `tid` its number in the group, `bar` the
+// group's barrier) calls it, the TPR threads of a row with the same x.
+// Returns false if a tensor-core wait gave up, now or before (`ok`; the output
+// is then meaningless).  The output is valid in every thread of the row.
+// part: 2 x 128 floats of shared memory for combining the halves of the output
 // layer (TPR = 2; rewritten only after the next tile's first barrier).
 // SAVE stores the activations of the row (sv->row >= 0).
 template <int TPR, bool SAVE = false>
-__device__ __forceinline__ bool tc_mlp_tile(TcMlpSmem &S, const float (&x)[5], float &out, unsigned &phase,
-                                            float *part = nullptr, const TcSave *sv = nullptr)
+__device__ __forceinline__ bool tc_mlp_tile(const TcMlpImage &img, TcTile &T, int tid, int bar, bool ok, const float (&x)[5],
+                                            float &out, unsigned &phase, float *part = nullptr, const TcSave *sv = nullptr)
 {
-    constexpr int NC = 64 / TPR;
-    const int m = tc_rowid<TPR>(), half = tc_half<TPR>();
+    constexpr int threads = kTcRows * TPR;
+    const int m = tid & (kTcRows - 1), half = TPR == 1 ? 0 : tid >> 7;
     const bool save = SAVE && sv->row >= 0;
     const size_t ro = SAVE ? (size_t)(sv->row < 0 ? 0 : sv->row) * 64 : 0;
     {
@@ -409,38 +483,52 @@ __device__ __forceinline__ bool tc_mlp_tile(TcMlpSmem &S, const float (&x)[5], f
 #pragma unroll
         for (int q = 0; q < 8; ++q) v[q] = (uint32_t)p[2 * q] | ((uint32_t)p[2 * q + 1] << 16);
         if (TPR == 1 || half == 0)
-            *reinterpret_cast<uint4 *>(S.a1 + kmaj_off(kTcRows, m, 0)) = make_uint4(v[0], v[1], v[2], v[3]);
+            *reinterpret_cast<uint4 *>(T.a2 + kmaj_off(kTcRows, m, 0)) = make_uint4(v[0], v[1], v[2], v[3]);
         if (TPR == 1 || half == 1)
-            *reinterpret_cast<uint4 *>(S.a1 + kmaj_off(kTcRows, m, 8)) = make_uint4(v[4], v[5], v[6], v[7]);
+            *reinterpret_cast<uint4 *>(T.a2 + kmaj_off(kTcRows, m, 8)) = make_uint4(v[4], v[5], v[6], v[7]);
     }
-    bool ok = tc_layer(S, S.a1, S.img.w1, 1, 0, phase);
-    float z[NC];
-    tc_row<TPR>(S, z);
-    if (save) tc_silu_store<TPR, true>(S, z, sv->z1 + ro, sv->h1 + ro);
-    else tc_silu_store<TPR, false>(S, z, nullptr, nullptr);
-    ok &= tc_layer(S, S.a2, S.img.w2, 4, 1, phase);
-    tc_row<TPR>(S, z);
-    if (save) tc_silu_store<TPR, true>(S, z, sv->z2 + ro, sv->h2 + ro);
-    else tc_silu_store<TPR, false>(S, z, nullptr, nullptr);
-    ok &= tc_layer(S, S.a2, S.img.w3, 4, 2, phase);
-    tc_row<TPR>(S, z);
-    const int c0 = NC * half;
-    float2 acc = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int k = 0; k < NC; k += 2) {
-        if (save) *reinterpret_cast<float2 *>(sv->z3 + ro + c0 + k) = make_float2(z[k], z[k + 1]);
-        const float2 h = tc_silu2(k >> 1, make_float2(z[k], z[k + 1]));
-        if (save) *reinterpret_cast<float2 *>(sv->h3 + ro + c0 + k) = h;
-        acc = __ffma2_rn(h, make_float2(S.img.w4[c0 + k], S.img.w4[c0 + k + 1]), acc);
+    const uint32_t tm = T.tmem;
+    // 32 columns at a time: 32 values in registers instead of 64
+    auto hidden = [&](float *zb, float *hb) {
+        float z[32];
+        auto store = [&](int c0) {
+            if (save) tc_silu_store<true>(T, m, c0, z, zb + ro, hb + ro);
+            else tc_silu_store<false>(T, m, c0, z, nullptr, nullptr);
+        };
+        if (TPR == 1 || half == 0) {
+            tc_cols<0>(tm, z);
+            store(0);
+        }
+        if (TPR == 1 || half == 1) {
+            tc_cols<32>(tm, z);
+            store(32);
+        }
+    };
+    ok = tc_layer(img, T, tid, bar, threads, img.w1, 1, 0, phase, ok);
+    hidden(SAVE ? sv->z1 : nullptr, SAVE ? sv->h1 : nullptr);
+    ok = tc_layer(img, T, tid, bar, threads, img.w2, 4, 1, phase, ok);
+    hidden(SAVE ? sv->z2 : nullptr, SAVE ? sv->h2 : nullptr);
+    ok = tc_layer(img, T, tid, bar, threads, img.w3, 4, 2, phase, ok);
+    float o = 0.0f;
+    {
+        float z[32];
+        float *zb = SAVE ? sv->z3 + ro : nullptr, *hb = SAVE ? sv->h3 + ro : nullptr;
+        if (TPR == 1 || half == 0) {
+            tc_cols<0>(tm, z);
+            o = tc_output<SAVE>(img, 0, z, save, zb, hb);
+        }
+        if (TPR == 1 || half == 1) {
+            tc_cols<32>(tm, z);
+            o += tc_output<SAVE>(img, 32, z, save, zb, hb);
+        }
     }
-    float o = acc.x + acc.y;
     if (TPR == 2) {
         // both threads of the row add the two halves in the same order
         part[half * kTcRows + m] = o;
-        __syncthreads();
+        tc::bar_sync(bar, threads);
         o = part[m] + part[kTcRows + m];
     }
-    out = o + S.img.b4;
+    out = o + img.b4;
     return ok;
 }
 

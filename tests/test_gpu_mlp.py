@@ -400,3 +400,40 @@ def test_trained_network_gain(env, orc):
         rates[name] = 5 * data.count / (time.perf_counter() - t0)
     print("trained f_theta: max|err|/peak %.2e (untrained %.2e), rms %.2e; footprints/s exact %.3g, mlp %.3g"
           % (after["max_abs_rel_peak"], before["max_abs_rel_peak"], after["rms"], rates["exact"], rates["mlp"]))
+
+
+@pytest.mark.parametrize("count", [1, 200])
+def test_mlp_far_negative_preactivations(env, orc, count):
+    """SiLU takes one reciprocal for four denominators; pre-activations below
+    about -22 in all four (and far below in one) drive their product out of
+    range, and the values are taken one by one: against the oracle's BF16
+    contract, on every layer and both thread layouts (evaluation and
+    training forward), with the contract's own tolerances."""
+    torch, spl, learn = env
+    rng = np.random.default_rng(5600)
+    prm = np.zeros(spl.MLP_PARAMS, dtype=np.float32)
+    W1, b1 = prm[:320].reshape(64, 5), prm[320:384]
+    W1[:] = rng.integers(-2, 3, size=(64, 5)) * 0.25
+    b1[:16] = -40.0  # whole groups of four far below zero
+    b1[16:20] = (-1.0, 0.5, -3000.0, 1.0)  # one of a group beyond the range by itself
+    b1[20:] = rng.integers(-4, 5, size=44) * 0.25
+    for o in (384, 384 + 4160):
+        prm[o:o + 4096] = (rng.integers(-1, 2, size=4096) * 0.0625).astype(np.float32)
+        prm[o + 4096:o + 4100] = -60.0
+        prm[o + 4100] = -200.0
+    prm[8704:8768] = rng.integers(-4, 5, size=64) * 0.125
+    m = spl.Mlp(3, max_batch=256, seed=1)
+    m.set_params(prm)
+    X = np.round(rng.uniform(-2, 2, size=(count, 5)) * 8).astype(np.float32) / 8
+    out = torch.empty(count, device="cuda")
+    Xt = torch.tensor(X, device="cuda")
+    m.eval(Xt, out)
+    grad, loss = torch.empty(spl.MLP_PARAMS, device="cuda"), torch.empty(1, device="cuda")
+    Y = torch.zeros(count, device="cuda")
+    m.grad(Xt, Y, grad, loss)
+    m.status()
+    assert torch.isfinite(out).all() and torch.isfinite(grad).all()
+    ref = orc.mlp_forward(SIZES, prm.astype(np.float64), X.astype(np.float64), mode=1)
+    got = out.cpu().numpy().astype(np.float64)
+    assert_matches_contract(orc, prm, X, got, ref)
+    assert abs(float(loss) - np.mean(got ** 2)) <= 1e-5 * np.mean(got ** 2) + 1e-12
