@@ -7,10 +7,10 @@
 //   k_train_forward  -- the inference tile (tcgen05 BF16 MMAs) on the batch,
 //                       saving pre-activations and the activations that
 //                       entered each layer;
-//   k_train_backward -- one thread per row: dL/dz of every layer (FP32, the
-//                       BF16 roundings passed straight through);
-//   k_train_wgrad    -- per batch chunk, dL/dW = sum_b dz_b x h_b^T and
-//                       dL/db (FP32), into fixed partial slots;
+//   k_train_backward -- per batch chunk, dL/dz of every layer (FP32, the BF16
+//                       roundings passed straight through) and from it
+//                       dL/dW = sum_b dz_b x h_b^T and dL/db, into fixed
+//                       partial slots;
 //   k_train_reduce   -- adds the chunk partials in a fixed order (deterministic)
 //                       and the loss;
 //   k_adam           -- Adam on the FP32 master copy, then k_prep refreshes
@@ -26,7 +26,6 @@
 namespace spl {
 
 constexpr int kChunkRows = 64;     // rows per weight-gradient partial
-constexpr int kWgThreads = 256;
 
 }  // namespace spl
 
@@ -45,10 +44,8 @@ struct spl_mlp {
     void *tc_img;     // evaluation copy in the tcgen05 tile's operand layout
     float *act;       // [6][max_batch][64] z1 h1 z2 h2 z3 h3
     float *out;       // [max_batch] outputs
-    float *dz;        // [3][max_batch][64] dz1 dz2 dz3
-    float *dz4;       // [max_batch]
-    float *part;      // [chunks][kParams + 1] weight-gradient (and loss) partials
-    double *loss_part;  // [max_batch / 128 + 1] per-block loss partials
+    float *part;      // [chunks][kPartStride] weight-gradient partials
+    double *loss_part;  // [chunks] loss partials
     int *err;         // device error flag (kErrTimeout: a tensor-core wait gave up)
     void *block;      // single device allocation holding all of the above
 };
@@ -236,170 +233,180 @@ __device__ __forceinline__ float silu_grad(float z)
     return s * (1.0f + z * (1.0f - s));
 }
 
-// dL/dz of every layer for L = (1/B) sum (f(x_b) - y_b)^2.  Four threads
-// per row (consecutive lanes), each owning 16 of the 64 units of a layer;
-// a layer's gradient vector passes between them through shared memory
-// (rows padded to 65 floats: the 8 rows of a warp hit distinct banks).
-// Weights as used in the forward (BF16-rounded) come from the FP32 master
-// rounded on the fly; roundings of activations pass straight through.
-constexpr int kBwdThreads = 64;
-constexpr int kBwdSplit = 4;                         // threads per row
-constexpr int kBwdRows = kBwdThreads / kBwdSplit;    // rows per block
-constexpr int kBwdUnits = kHid / kBwdSplit;          // units per thread
+// Gradients of one batch chunk (64 rows) for L = (1/B) sum (f(x_b) - y_b)^2:
+// dL/dz of the three hidden layers, and from each the layer's weight and bias
+// gradients, without leaving the block.  A layer is two 64 x 64 x 64 FP32
+// products on the chunk's dz: dW[o][i] = sum_r dz[r][o] h[r][i] and the layer
+// below's dh[r][i] = sum_o dz[r][o] W[o][i]; dz sits in shared memory in both
+// orders, so that every operand of a thread's 4 x 4 outputs is one 16-byte
+// load per step.  Weights as used in the forward (BF16-rounded) come from the
+// FP32 master rounded on the fly; roundings of activations pass straight
+// through.  Rows are summed in order (deterministic).
+//
+// 8192 rows are 128 blocks, less than one wave: the time is one block's
+// latency.  A gradient of 8192 samples went from 82 to 40 us with this kernel
+// in place of one thread group per row for dz and 512 blocks for the products,
+// which passed dz through memory; 512 threads with 4 x 2 outputs took 41.
+constexpr int kBwdThreads = 256;
+constexpr int kPartStride = (kParams + 1 + 3) & ~3;  // floats per chunk of partials, 16-byte rows
+constexpr int kDzPad = 4;                            // row padding (floats) of the dz arrays
+struct __align__(16) BwdSmem {
+    float W2[kHid * kHid], W3[kHid * kHid];
+    float D[kChunkRows][kHid + kDzPad];   // dz[r][o]
+    float DT[kHid][kChunkRows + kDzPad];  // dz[o][r]
+    float H[kChunkRows][kHid];            // activations that entered the layer
+    float W4[kHid], d4[kChunkRows], X[kChunkRows * kIn];
+    double red[kBwdThreads / 32];
+};
 
-// gout[i] = silu'(z[i]) * sum_c W[c][i] gin[c] for this thread's units
-// i = i0 .. i0 + 15; W as [c][i] (row c = output unit of the layer above)
-__device__ __forceinline__ void back_layer(const float *__restrict__ W, const float *__restrict__ gin, int i0,
-                                           const float *__restrict__ z, float *__restrict__ gout_g,
-                                           float *__restrict__ gout_s)
+// sum_k a[k][i0 + i] b[k][j0 + j] for i, j = 0..3 over 64 k; rows of sa, sb floats
+__device__ __forceinline__ void product4x4(const float *a, int sa, const float *b, int sb, float (&c)[4][4])
 {
-    float acc[kBwdUnits];
+    float2 acc[4][2];
 #pragma unroll
-    for (int q = 0; q < kBwdUnits; ++q) acc[q] = 0.0f;
+    for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = make_float2(0.0f, 0.0f);
 #pragma unroll 8
-    for (int c = 0; c < kHid; ++c) {
-        const float g = gin[c];
-        const float4 *w = reinterpret_cast<const float4 *>(W + c * kHid + i0);
+    for (int k = 0; k < 64; ++k) {
+        const float4 x = *reinterpret_cast<const float4 *>(a + k * sa), y = *reinterpret_cast<const float4 *>(b + k * sb);
+        const float xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-        for (int q4 = 0; q4 < kBwdUnits / 4; ++q4) {
-            const float4 v = w[q4];
-            acc[4 * q4] = fmaf(v.x, g, acc[4 * q4]);
-            acc[4 * q4 + 1] = fmaf(v.y, g, acc[4 * q4 + 1]);
-            acc[4 * q4 + 2] = fmaf(v.z, g, acc[4 * q4 + 2]);
-            acc[4 * q4 + 3] = fmaf(v.w, g, acc[4 * q4 + 3]);
+        for (int i = 0; i < 4; ++i) {
+            acc[i][0] = __ffma2_rn(make_float2(xs[i], xs[i]), make_float2(y.x, y.y), acc[i][0]);
+            acc[i][1] = __ffma2_rn(make_float2(xs[i], xs[i]), make_float2(y.z, y.w), acc[i][1]);
         }
     }
 #pragma unroll
-    for (int q4 = 0; q4 < kBwdUnits / 4; ++q4) {
-        const float4 zz = *reinterpret_cast<const float4 *>(z + i0 + 4 * q4);
-        const float4 g = make_float4(acc[4 * q4] * silu_grad(zz.x), acc[4 * q4 + 1] * silu_grad(zz.y),
-                                     acc[4 * q4 + 2] * silu_grad(zz.z), acc[4 * q4 + 3] * silu_grad(zz.w));
-        *reinterpret_cast<float4 *>(gout_g + i0 + 4 * q4) = g;
-        gout_s[i0 + 4 * q4] = g.x;
-        gout_s[i0 + 4 * q4 + 1] = g.y;
-        gout_s[i0 + 4 * q4 + 2] = g.z;
-        gout_s[i0 + 4 * q4 + 3] = g.w;
+    for (int i = 0; i < 4; ++i) {
+        c[i][0] = acc[i][0].x;
+        c[i][1] = acc[i][0].y;
+        c[i][2] = acc[i][1].x;
+        c[i][3] = acc[i][1].y;
     }
 }
 
-__global__ void __launch_bounds__(kBwdThreads) k_train_backward(const float *__restrict__ P, int B,
-                                                                const float *__restrict__ Y,
-                                                                const float *__restrict__ act,
-                                                                const float *__restrict__ out, float *dz, float *dz4,
-                                                                double *loss_part, int max_batch)
+__global__ void __launch_bounds__(kBwdThreads, 2) k_train_backward(const float *__restrict__ P, int B,
+                                                                   const float *__restrict__ X, const float *__restrict__ Y,
+                                                                   const float *__restrict__ act,
+                                                                   const float *__restrict__ out, float *__restrict__ part,
+                                                                   double *__restrict__ loss_part, int max_batch)
 {
-    // W2, W3 stored as [c][i] = W[c][i] (row c = output unit): reading
-    // W[c][i0..i0+3] for fixed c is a float4
-    __shared__ __align__(16) float W2[kHid * kHid];
-    __shared__ __align__(16) float W3[kHid * kHid];
-    __shared__ float W4[kHid];
-    __shared__ float gbuf[2][kBwdRows][kHid + 1];
-    __shared__ double red[kBwdThreads / 32];
-    for (int i = threadIdx.x; i < kHid * kHid; i += blockDim.x) {
-        W2[i] = bf16r(P[kOffW2 + i]);
-        W3[i] = bf16r(P[kOffW3 + i]);
-    }
-    if (threadIdx.x < kHid) W4[threadIdx.x] = bf16r(P[kOffW4 + threadIdx.x]);
-    __syncthreads();
-    const int lr = threadIdx.x / kBwdSplit, i0 = (threadIdx.x % kBwdSplit) * kBwdUnits;
-    const int r = blockIdx.x * kBwdRows + lr;
+    extern __shared__ __align__(16) unsigned char bwd_smem[];
+    BwdSmem &S = *reinterpret_cast<BwdSmem *>(bwd_smem);
+    const int t = threadIdx.x, r0 = blockIdx.x * kChunkRows, nr = min(kChunkRows, B - r0);
     const size_t L = (size_t)max_batch * 64;
-    double l2 = 0.0;
-    const bool live = r < B;  // the four threads of a row agree
-    if (live) {
-        const float res = out[r] - Y[r];
-        if (i0 == 0) {
-            l2 = (double)res * res;
-            dz4[r] = 2.0f * res / (float)B;
-        }
-        const float d4 = 2.0f * res / (float)B;
-        const float *z3 = act + 4 * L + (size_t)r * 64;
+    float *dst = part + (size_t)blockIdx.x * kPartStride;
+    const int p4 = 4 * (t >> 4), q4 = 4 * (t & 15);  // this thread's 4 x 4 outputs
+    // rows p4 .. p4 + 3, columns q4 .. q4 + 3 of an activation array (0 beyond the batch)
+    auto rows = [&](const float *src, float4 (&v)[4]) {
 #pragma unroll
-        for (int c = i0; c < i0 + kBwdUnits; c += 4) {
-            const float4 zz = *reinterpret_cast<const float4 *>(z3 + c);
-            const float4 g = make_float4(W4[c] * d4 * silu_grad(zz.x), W4[c + 1] * d4 * silu_grad(zz.y),
-                                         W4[c + 2] * d4 * silu_grad(zz.z), W4[c + 3] * d4 * silu_grad(zz.w));
-            *reinterpret_cast<float4 *>(dz + 2 * L + (size_t)r * 64 + c) = g;
-            gbuf[0][lr][c] = g.x;
-            gbuf[0][lr][c + 1] = g.y;
-            gbuf[0][lr][c + 2] = g.z;
-            gbuf[0][lr][c + 3] = g.w;
-        }
+        for (int i = 0; i < 4; ++i)
+            v[i] = p4 + i < nr ? __ldg(reinterpret_cast<const float4 *>(src + (size_t)(r0 + p4 + i) * 64 + q4))
+                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    };
+    // everything the block reads is requested first
+    float4 z3[4], h2[4], z2[4], h1[4], z1[4], h3[4];
+    rows(act + 4 * L, z3);
+    rows(act + 5 * L, h3);
+    rows(act + 3 * L, h2);
+    rows(act + 2 * L, z2);
+    rows(act + L, h1);
+    rows(act, z1);
+    for (int i = t; i < kHid * kHid / 4; i += kBwdThreads) {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(P + kOffW2) + i),
+                     b = __ldg(reinterpret_cast<const float4 *>(P + kOffW3) + i);
+        reinterpret_cast<float4 *>(S.W2)[i] = make_float4(bf16r(a.x), bf16r(a.y), bf16r(a.z), bf16r(a.w));
+        reinterpret_cast<float4 *>(S.W3)[i] = make_float4(bf16r(b.x), bf16r(b.y), bf16r(b.z), bf16r(b.w));
     }
-    __syncwarp();
-    if (live) back_layer(W3, gbuf[0][lr], i0, act + 2 * L + (size_t)r * 64, dz + L + (size_t)r * 64, gbuf[1][lr]);
-    __syncwarp();
-    if (live) back_layer(W2, gbuf[1][lr], i0, act + (size_t)r * 64, dz + (size_t)r * 64, gbuf[0][lr]);
-    // per-block loss partial (fixed order)
+    if (t < kHid) S.W4[t] = bf16r(P[kOffW4 + t]);
+    for (int i = t; i < kChunkRows * kIn; i += kBwdThreads) S.X[i] = i < nr * kIn ? X[(size_t)r0 * kIn + i] : 0.0f;
+    double l2 = 0.0;
+    if (t < kChunkRows) {
+        const float res = t < nr ? out[r0 + t] - Y[r0 + t] : 0.0f;
+        l2 = (double)res * res;
+        S.d4[t] = 2.0f * res / (float)B;
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) l2 += __shfl_down_sync(0xffffffffu, l2, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l2;
+    if ((t & 31) == 0) S.red[t >> 5] = l2;
+    auto put = [&](float (&dst_)[kChunkRows][kHid], const float4 (&v)[4]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) *reinterpret_cast<float4 *>(&dst_[p4 + i][q4]) = v[i];
+    };
+    // dz of a layer in both orders, and the activations that entered it
+    auto put_dz = [&](const float (&d)[4][4]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            *reinterpret_cast<float4 *>(&S.D[p4 + i][q4]) = make_float4(d[i][0], d[i][1], d[i][2], d[i][3]);
+            *reinterpret_cast<float4 *>(&S.DT[q4 + i][p4]) = make_float4(d[0][i], d[1][i], d[2][i], d[3][i]);
+        }
+    };
+    auto grad_of = [&](const float (&g)[4][4], const float4 (&z)[4], float (&d)[4][4]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            d[i][0] = g[i][0] * silu_grad(z[i].x);
+            d[i][1] = g[i][1] * silu_grad(z[i].y);
+            d[i][2] = g[i][2] * silu_grad(z[i].z);
+            d[i][3] = g[i][3] * silu_grad(z[i].w);
+        }
+    };
+    float g[4][4], d[4][4];
+    // output layer: dW4 = sum_r d4 h3, db4 = sum_r d4
+    put(S.H, h3);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kBwdThreads / 32; ++w) t += red[w];
-        loss_part[blockIdx.x] = t;
+    if (t < kHid) {
+        float a = 0.0f;
+        for (int r = 0; r < nr; ++r) a = fmaf(S.d4[r], S.H[r][t], a);
+        dst[kOffW4 + t] = a;
+    } else if (t == kHid) {
+        float a = 0.0f;
+        for (int r = 0; r < nr; ++r) a += S.d4[r];
+        dst[kOffB4] = a;
+    } else if (t == kHid + 1) {
+        double s = 0.0;
+        for (int w = 0; w < kBwdThreads / 32; ++w) s += S.red[w];
+        loss_part[blockIdx.x] = s;
     }
-}
-
-// Weight gradients of one batch chunk: block (chunk, layer).  Rows are
-// staged through shared memory 32 at a time; for the 64x64 layers each
-// thread owns one output unit o and 16 consecutive inputs, and sums the
-// chunk's rows in order (deterministic).
-constexpr int kStageRows = 32;
-
-__global__ void __launch_bounds__(kWgThreads) k_train_wgrad(int B, const float *__restrict__ X,
-                                                            const float *__restrict__ act,
-                                                            const float *__restrict__ dz,
-                                                            const float *__restrict__ dz4, float *part, int max_batch)
-{
-    __shared__ __align__(16) float Gs[kStageRows][kHid];
-    __shared__ __align__(16) float Hs[kStageRows][kHid];
-    const int chunk = blockIdx.x, layer = blockIdx.y;
-    const size_t L = (size_t)max_batch * 64;
-    const int r0 = chunk * kChunkRows, r1 = min(B, r0 + kChunkRows);
-    float *dst = part + (size_t)chunk * (kParams + 1);
-    int nin, nout, offW, offB, hstride, gstride;
-    const float *H, *G;
-    if (layer == 0) { nin = kIn; nout = kHid; H = X; hstride = kIn; G = dz; gstride = 64; offW = kOffW1; offB = kOffB1; }
-    else if (layer == 1) { nin = kHid; nout = kHid; H = act + L; hstride = 64; G = dz + L; gstride = 64; offW = kOffW2; offB = kOffB2; }
-    else if (layer == 2) { nin = kHid; nout = kHid; H = act + 3 * L; hstride = 64; G = dz + 2 * L; gstride = 64; offW = kOffW3; offB = kOffB3; }
-    else { nin = kHid; nout = 1; H = act + 5 * L; hstride = 64; G = dz4; gstride = 1; offW = kOffW4; offB = kOffB4; }
-    // thread -> (o, 16 inputs starting at i0); the thread with i0 = 0 also
-    // sums the bias gradient of o
-    const int nslots = nout * ((nin + 15) / 16);
-    const int slot = threadIdx.x;
-    const bool has_w = slot < nslots;
-    const int o = has_w ? slot / ((nin + 15) / 16) : 0;
-    const int i0 = has_w ? (slot % ((nin + 15) / 16)) * 16 : 0;
-    const bool has_b = has_w && i0 == 0;
-    float acc[16];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) acc[q] = 0.0f;
-    float accb = 0.0f;
-    for (int rs = r0; rs < r1; rs += kStageRows) {
-        const int nr = min(kStageRows, r1 - rs);
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) g[i][j] = S.W4[q4 + j] * S.d4[p4 + i];
+    grad_of(g, z3, d);
+    __syncthreads();
+    // a hidden layer: weight gradient, bias gradient, dz of the layer below
+    auto layer = [&](const float4 (&h)[4], int offW, int offB, const float *W, const float4 (&zb)[4]) {
+        put_dz(d);
+        put(S.H, h);
         __syncthreads();
-        for (int e = threadIdx.x; e < kStageRows * kHid; e += blockDim.x) {
-            const int rr = e / kHid, cc = e % kHid;
-            Gs[rr][cc] = (rr < nr && cc < nout) ? G[(size_t)(rs + rr) * gstride + cc] : 0.0f;
-            Hs[rr][cc] = (rr < nr && cc < nin) ? H[(size_t)(rs + rr) * hstride + cc] : 0.0f;
+        float w[4][4];
+        product4x4(&S.D[0][p4], kHid + kDzPad, &S.H[0][q4], kHid, w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4 *>(dst + offW + (p4 + i) * kHid + q4) = make_float4(w[i][0], w[i][1], w[i][2], w[i][3]);
+        if (t < kHid) {
+            float a = 0.0f;
+            for (int r = 0; r < kChunkRows; ++r) a += S.D[r][t];
+            dst[offB + t] = a;
         }
+        product4x4(&S.DT[0][p4], kChunkRows + kDzPad, W + q4, kHid, g);
+        grad_of(g, zb, d);
         __syncthreads();
-        if (has_w) {
-            for (int rr = 0; rr < nr; ++rr) {
-                const float gv = Gs[rr][o];
-                accb += gv;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) acc[q] = fmaf(gv, Hs[rr][i0 + q], acc[q]);
-            }
+    };
+    layer(h2, kOffW3, kOffB3, S.W3, z2);
+    layer(h1, kOffW2, kOffB2, S.W2, z1);
+    put_dz(d);
+    __syncthreads();
+    // first layer: inputs e = t / 64 and (t / 64 == 0) 4, the bias with e = 1
+    {
+        const int o = t & 63, e = t >> 6;
+        float a = 0.0f, c = 0.0f;
+        for (int r = 0; r < nr; ++r) {
+            const float v = S.D[r][o];
+            a = fmaf(v, S.X[r * kIn + e], a);
+            c = e == 0 ? fmaf(v, S.X[r * kIn + 4], c) : c + v;
         }
-    }
-    if (has_w) {
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-            if (i0 + q < nin) dst[offW + o * nin + i0 + q] = acc[q];
-        if (has_b) dst[offB + o] = accb;
+        dst[kOffW1 + o * kIn + e] = a;
+        if (e == 0) dst[kOffW1 + o * kIn + 4] = c;
+        if (e == 1) dst[kOffB1 + o] = c;
     }
 }
 
@@ -418,7 +425,8 @@ __global__ void __launch_bounds__(kRedThreads) k_train_reduce(const float *__res
     const int i = blockIdx.x * 32 + lane;
     float acc = 0.0f;
     if (i < kParams)
-        for (int c = w; c < chunks; c += kRedThreads / 32) acc += part[(size_t)c * (kParams + 1) + i];
+#pragma unroll 8
+        for (int c = w; c < chunks; c += kRedThreads / 32) acc += __ldg(part + (size_t)c * kPartStride + i);
     ps[w][lane] = acc;
     const bool do_loss = blockIdx.x == 0 && loss_out != nullptr;
     if (do_loss) {
@@ -468,12 +476,12 @@ static spl_status grad_impl(spl_mlp *m, int B, const float *X, const float *Y, f
         if (s != SPL_OK) return s;
     }
     k_train_forward<<<eval_blocks(B), 2 * kTcRows, sizeof(TcMlpSmem<1>), st>>>(w, B, X, m->act, m->out, m->max_batch);
-    const int bblocks = (B + kBwdRows - 1) / kBwdRows;
-    k_train_backward<<<bblocks, kBwdThreads, 0, st>>>(m->master, B, Y, m->act, m->out, m->dz, m->dz4, m->loss_part,
-                                                      m->max_batch);
+    const spl_status sb = smem_attr_once((const void *)k_train_backward, (int)sizeof(BwdSmem), "train backward smem attribute");
+    if (sb != SPL_OK) return sb;
     const int chunks = (B + kChunkRows - 1) / kChunkRows;
-    k_train_wgrad<<<dim3(chunks, 4), kWgThreads, 0, st>>>(B, X, m->act, m->dz, m->dz4, m->part, m->max_batch);
-    k_train_reduce<<<(kParams + 31) / 32, kRedThreads, 0, st>>>(m->part, chunks, m->loss_part, bblocks, B, grad, loss);
+    k_train_backward<<<chunks, kBwdThreads, sizeof(BwdSmem), st>>>(m->master, B, X, Y, m->act, m->out, m->part, m->loss_part,
+                                                                   m->max_batch);
+    k_train_reduce<<<(kParams + 31) / 32, kRedThreads, 0, st>>>(m->part, chunks, m->loss_part, chunks, B, grad, loss);
     return cuda_check(cudaGetLastError(), "mlp gradient launch");
 }
 
@@ -506,7 +514,7 @@ extern "C" spl_status spl_mlp_create(int degree, int max_batch, unsigned long lo
     m->seed = seed;
     cudaGetDevice(&m->device);
     const int chunks = (max_batch + kChunkRows - 1) / kChunkRows;
-    const int nloss = (max_batch + kBwdRows - 1) / kBwdRows;
+    const int nloss = chunks;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -517,8 +525,7 @@ extern "C" spl_status spl_mlp_create(int degree, int max_batch, unsigned long lo
                  o_grad = take(kParams * 4), o_w23 = take(2 * kHid * kRowWords * 4), o_f32 = take(kF32Size * 4),
                  o_img = take(sizeof(TcMlpImage)),
                  o_act = take((size_t)6 * max_batch * 64 * 4), o_out = take((size_t)max_batch * 4),
-                 o_dz = take((size_t)3 * max_batch * 64 * 4), o_dz4 = take((size_t)max_batch * 4),
-                 o_part = take((size_t)chunks * (kParams + 1) * 4), o_loss = take((size_t)nloss * 8),
+                 o_part = take((size_t)chunks * kPartStride * 4), o_loss = take((size_t)nloss * 8),
                  o_err = take(sizeof(int));
     void *blk = nullptr;
     cudaError_t ce = cudaMalloc(&blk, off);
@@ -538,8 +545,6 @@ extern "C" spl_status spl_mlp_create(int degree, int max_batch, unsigned long lo
     m->tc_img = base + o_img;
     m->act = (float *)(base + o_act);
     m->out = (float *)(base + o_out);
-    m->dz = (float *)(base + o_dz);
-    m->dz4 = (float *)(base + o_dz4);
     m->part = (float *)(base + o_part);
     m->loss_part = (double *)(base + o_loss);
     m->err = (int *)(base + o_err);

@@ -59,13 +59,28 @@ def check(env, orc, geo, degrees, seed, dims=DIMS):
 @pytest.mark.parametrize("rays", [700, 25000, 90001])
 def test_rays_per_split(env, orc, rays):
     """From too few rays to fill the GPU (8 threads a ray) to one thread a
-    ray, with flat rays and short rays whose parts are empty."""
+    ray, with flat rays and short rays whose parts are empty.  The most rays
+    at degree 3 (slow in the oracle) against the sum over two geometries with
+    half of them each, which take two threads a ray."""
     rng = np.random.default_rng(rays)
     w = I.random_directions(rng, rays)
     w[::7, rng.integers(3)] = 0.0
     w /= np.linalg.norm(w, axis=1, keepdims=True)
     s = rng.uniform(-1.15, 1.15, size=(rays, 3)) * 0.5 * (np.asarray(DIMS) - 1.0)
-    check(env, orc, I.RayGeometry(w, s), (3, 0, 2, 1, 3) if rays < 10000 else (3, 1), 10)
+    if rays < 10000:
+        check(env, orc, I.RayGeometry(w, s), (3, 0, 2, 1, 3), 10)
+        return
+    check(env, orc, I.RayGeometry(w, s), (1,), 10)
+    torch, spl = env
+    y = torch.randn(rays, device="cuda")
+    parts = []
+    for sl in (slice(None), slice(0, rays // 2), slice(rays // 2, None)):
+        g = spl.Geometry(DIMS, I.centred_origin(DIMS), I.RayGeometry(w[sl], s[sl]))
+        c = torch.empty(g.coeff_shape, device="cuda")
+        spl.adjoint(g, y[sl].contiguous(), c, spl.basis(3))
+        g.status()
+        parts.append(c.double())
+    assert float((parts[0] - parts[1] - parts[2]).norm() / parts[0].norm()) <= 2 * TOL
 
 
 @pytest.mark.parametrize("views", [1, 21, 60])
@@ -82,17 +97,31 @@ def test_views_per_split_lane_axis_and_batches(env, orc, kind, turned, views):
         geo = I.helical_cone(views, 50.0, 80.0, nu, nv, 0.9, turns=1.3, table_feed=6.0)
     if turned:
         geo = I.ViewGeometry(geo.kind, geo.src, geo.det_center, geo.det_v, -geo.det_u, nu, nv)
-    check(env, orc, geo, (3, 1), 20 + views)
+    check(env, orc, geo, (3, 1) if views < 60 else (1,), 20 + views)
 
 
 @pytest.mark.parametrize("dims", [(1, 1, 1), (2, 40, 3), (70, 61, 65)])
 def test_thin_and_tiled_folds(env, orc, dims):
     """Grids thinner than a window, and one above the single-launch fold's
-    size with partial tiles."""
+    size with partial tiles.  The sum of one coefficient's 3000 terms can
+    come out near zero, so the error is taken against the sum of their
+    magnitudes, A^T |y|: a running FP32 sum in any order is within a few
+    roundings of 2^-24 of that."""
     rng = np.random.default_rng(5)
     w = I.random_directions(rng, 3000)
     s = rng.uniform(-0.6, 0.6, size=w.shape) * np.asarray(dims)
-    check(env, orc, I.RayGeometry(w, s), (3, 2, 1, 0), 30, dims)
+    torch, spl = env
+    geo, origin = I.RayGeometry(w, s), I.centred_origin(dims)
+    g = spl.Geometry(dims, origin, geo)
+    y = rng.normal(size=geo.n_rays).astype(np.float32)
+    for degree in (3, 2, 1, 0):
+        ref = orc.adjoint(degree, dims, origin, y.astype(np.float64), geom_of(orc, geo))
+        mag = orc.adjoint(degree, dims, origin, np.abs(y).astype(np.float64), geom_of(orc, geo))
+        for _ in range(2):
+            c = torch.full(g.coeff_shape, float("nan"), device="cuda")
+            spl.adjoint(g, torch.tensor(y, device="cuda"), c, spl.basis(degree))
+            g.status()
+            assert np.linalg.norm(c.cpu().numpy() - ref) <= 8 * 2.0 ** -24 * np.linalg.norm(mag), degree
 
 
 def test_flat_and_general_views_in_batches(env, orc):
