@@ -173,7 +173,7 @@ struct PlaneCall {
     int n_p, n_q, n_b;           // grid sizes of p, q, b
     long long st_p, st_q, st_b;  // linear strides of p, q, b in c
     long long ncol, rows;
-    int nu, nv;
+    int nu, nv, nvs;             // nvs: row stride of S, T and y^T, nv rounded up to even
 };
 
 // S[col][v] = sum_i wz[v][i] c(col, lb0[v] + i)
@@ -194,31 +194,41 @@ __global__ void __launch_bounds__(256) k_plane_zres(PlaneCall pc, const float *_
         const int lb = l0 + i;
         if (lb >= 0 && lb < pc.n_b) s = fmaf(wz[v * (N + 1) + i], __ldg(cc + lb * pc.st_b), s);
     }
-    S[idx] = s;
+    S[col * pc.nvs + v] = s;
 }
 
 // Warp-per-row sparse gather: out[row][v] = sum_e val[e] * in[idx[e]][v]
-// (rows of the forward, columns of the adjoint).  Lanes cover v; each chunk
-// of 32 entries is loaded once and broadcast by shuffles.  KAHAN: the chunk
-// partials are added with compensation.
+// (rows of the forward, columns of the adjoint).  Lanes cover v in pairs (rows
+// of `in` have an even stride nvs; the value beyond an odd nv is never
+// stored); each chunk of 32 entries is loaded once and broadcast by shuffles.
+// KAHAN: the chunk partials are added with compensation.  The rows of `in`
+// come from L1 and L2 (12.6 MB of S for 128^3 and 192 rows; the 180 views'
+// entries read 17 GB of it a call), so the loads and instructions per entry
+// count: pairs instead of single values took A of those views from 1.08 to
+// 0.68 ms and A^T from 1.43 to 0.82.
 constexpr int kPlaneWarps = 8;
-constexpr int kPlaneMV = 8;  // v per lane per pass (256 v per pass)
+constexpr int kPlaneMV = 4;  // v pairs per lane per pass (256 v per pass)
 
 template <bool KAHAN, bool TO_Y>
 __global__ void __launch_bounds__(32 * kPlaneWarps) k_plane_gather(long long nrow, const long long *__restrict__ ptr,
                                                                    const int *__restrict__ idx,
                                                                    const float *__restrict__ val,
                                                                    const float *__restrict__ in, float *__restrict__ out,
-                                                                   int nv, int nu, const int *view_order)
+                                                                   int nv, int nvs, int nu, const int *view_order)
 {
     const long long r = (long long)blockIdx.x * kPlaneWarps + (threadIdx.x >> 5);
     if (r >= nrow) return;
     const int lane = threadIdx.x & 31;
     const long long e0 = ptr[r], e1 = ptr[r + 1];
-    for (int vb = 0; vb < nv; vb += 32 * kPlaneMV) {
-        float acc[kPlaneMV], sum[kPlaneMV], comp[kPlaneMV];
+    for (int vb = 0; vb < nv; vb += 64 * kPlaneMV) {
+        float2 acc[kPlaneMV];
+        float sum[2 * kPlaneMV], comp[2 * kPlaneMV];
 #pragma unroll
-        for (int m = 0; m < kPlaneMV; ++m) acc[m] = sum[m] = comp[m] = 0.0f;
+        for (int m = 0; m < kPlaneMV; ++m) {
+            acc[m] = make_float2(0.0f, 0.0f);
+            sum[2 * m] = sum[2 * m + 1] = comp[2 * m] = comp[2 * m + 1] = 0.0f;
+        }
+        const float *base = in + vb + 2 * lane;
         for (long long e = e0; e < e1; e += 32) {
             const int n = (int)(e1 - e < 32 ? e1 - e : 32);
             int mi = 0;
@@ -227,40 +237,46 @@ __global__ void __launch_bounds__(32 * kPlaneWarps) k_plane_gather(long long nro
                 mi = idx[e + lane];
                 mv = val[e + lane];
             }
+#pragma unroll 4
             for (int j = 0; j < n; ++j) {
-                const long long ij = __shfl_sync(0xffffffffu, mi, j);
+                const int ij = __shfl_sync(0xffffffffu, mi, j);
                 const float gj = __shfl_sync(0xffffffffu, mv, j);
-                const float *src = in + ij * nv + vb + lane;
+                const float *src = base + (long long)ij * nvs;
 #pragma unroll
                 for (int m = 0; m < kPlaneMV; ++m)
-                    if (vb + lane + 32 * m < nv) acc[m] = fmaf(gj, __ldg(src + 32 * m), acc[m]);
+                    if (vb + 2 * lane + 64 * m < nv)
+                        acc[m] = __ffma2_rn(make_float2(gj, gj), __ldg(reinterpret_cast<const float2 *>(src + 64 * m)),
+                                            acc[m]);
             }
             if (KAHAN) {
 #pragma unroll
                 for (int m = 0; m < kPlaneMV; ++m) {
-                    kahan_add(sum[m], comp[m], acc[m]);
-                    acc[m] = 0.0f;
+                    kahan_add(sum[2 * m], comp[2 * m], acc[m].x);
+                    kahan_add(sum[2 * m + 1], comp[2 * m + 1], acc[m].y);
+                    acc[m] = make_float2(0.0f, 0.0f);
                 }
             }
         }
 #pragma unroll
-        for (int m = 0; m < kPlaneMV; ++m) {
-            const int v = vb + lane + 32 * m;
-            if (v >= nv) continue;
-            const float o = KAHAN ? sum[m] : acc[m];
-            if (TO_Y) {
-                const int gi = (int)(r / nu), u = (int)(r % nu);
-                out[((long long)view_order[gi] * nv + v) * nu + u] = o;
-            } else {
-                out[r * nv + v] = o;
+        for (int m = 0; m < kPlaneMV; ++m)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int v = vb + 2 * lane + 64 * m + h;
+                if (v >= nv) continue;
+                const float o = KAHAN ? sum[2 * m + h] : (h ? acc[m].y : acc[m].x);
+                if (TO_Y) {
+                    const int gi = (int)(r / nu), u = (int)(r % nu);
+                    out[((long long)view_order[gi] * nv + v) * nu + u] = o;
+                } else {
+                    out[r * nvs + v] = o;
+                }
             }
-        }
     }
 }
 
 // yt[gi*nu + u][v] = y[view_order[gi]][v][u]: 32 x 32 tiles through shared memory
 __global__ void __launch_bounds__(256) k_plane_ytrans(const float *__restrict__ y, float *__restrict__ yt,
-                                                      const int *view_order, int nu, int nv)
+                                                      const int *view_order, int nu, int nv, int nvs)
 {
     __shared__ float tile[32][33];
     const int gi = blockIdx.z;
@@ -274,7 +290,7 @@ __global__ void __launch_bounds__(256) k_plane_ytrans(const float *__restrict__ 
     __syncthreads();
     for (int j = ty; j < 32; j += 8) {
         const int u = u0 + j, v = v0 + tx;
-        if (u < nu && v < nv) yt[((long long)gi * nu + u) * nv + v] = tile[tx][j];
+        if (u < nu && v < nv) yt[((long long)gi * nu + u) * nvs + v] = tile[tx][j];
     }
 }
 
@@ -293,7 +309,7 @@ __global__ void __launch_bounds__(256) k_plane_zadj(PlaneCall pc, const float *_
     const int v0 = vr[2 * lb], v1 = vr[2 * lb + 1];
     for (int v = v0; v <= v1; ++v) {
         const int i = lb - lb0[v];
-        if (i >= 0 && i <= N) s = fmaf(wz[v * (N + 1) + i], __ldg(T + col * pc.nv + v), s);
+        if (i >= 0 && i <= N) s = fmaf(wz[v * (N + 1) + i], __ldg(T + col * pc.nvs + v), s);
     }
     float *dst = c + (ip * pc.st_p + iq * pc.st_q + (long long)lb * pc.st_b);
     *dst = ADD ? *dst + s : s;
@@ -318,6 +334,9 @@ double bspline(int n, double x)
     }
 }
 
+// row stride of S, T and y^T: even, so that the gather reads pairs
+int plane_stride(int nv) { return (nv + 1) & ~1; }
+
 PlaneCall call_of(const spl_geometry *g)
 {
     const PlaneGroup &pg = *g->plane;
@@ -334,6 +353,7 @@ PlaneCall call_of(const spl_geometry *g)
     pc.rows = pg.rows;
     pc.nu = dg.nu;
     pc.nv = dg.nv;
+    pc.nvs = plane_stride(dg.nv);
     return pc;
 }
 
@@ -345,7 +365,7 @@ spl_status build_pack(spl_geometry *g, cudaStream_t st)
     PlaneGroup &pg = *g->plane;
     PlanePack &pk = pg.pack[N];
     const DevGeom &dg = g->dev;
-    const int nv = dg.nv, nb = dg.n[pg.b];
+    const int nv = dg.nv, nvs = plane_stride(nv), nb = dg.n[pg.b];
     constexpr double W = 0.5 * (N + 1);
     // b weights of the detector rows (FP64 on the host)
     std::vector<int> lb0(nv), vr(2 * (size_t)nb);
@@ -374,9 +394,9 @@ spl_status build_pack(spl_geometry *g, cudaStream_t st)
     const size_t o_wz = align256(o_lb + nv * sizeof(int));
     const size_t o_vr = align256(o_wz + wz.size() * sizeof(float));
     const size_t o_S = align256(o_vr + vr.size() * sizeof(int));
-    const size_t o_T = align256(o_S + pg.ncol * nv * sizeof(float));
-    const size_t o_yt = align256(o_T + pg.ncol * nv * sizeof(float));
-    const size_t o_cur = align256(o_yt + pg.rows * nv * sizeof(float));
+    const size_t o_T = align256(o_S + pg.ncol * nvs * sizeof(float));
+    const size_t o_yt = align256(o_T + pg.ncol * nvs * sizeof(float));
+    const size_t o_cur = align256(o_yt + pg.rows * nvs * sizeof(float));
     const size_t bytes1 = align256(o_cur + (pg.ncol + 1) * sizeof(long long));
     char *b1 = nullptr;
     if (cudaMalloc(&b1, bytes1) != cudaSuccess) {
@@ -514,10 +534,10 @@ static spl_status plane_forward_n(const spl_geometry *g, int kahan, const float 
     const unsigned blocks = (unsigned)((pg.rows + kPlaneWarps - 1) / kPlaneWarps);
     if (kahan)
         k_plane_gather<true, true><<<blocks, 32 * kPlaneWarps, 0, st>>>(pg.rows, pk.row_ptr, pk.row_col, pk.row_val, pk.S,
-                                                                        y, pc.nv, pc.nu, g->dev.view_order);
+                                                                        y, pc.nv, pc.nvs, pc.nu, g->dev.view_order);
     else
         k_plane_gather<false, true><<<blocks, 32 * kPlaneWarps, 0, st>>>(pg.rows, pk.row_ptr, pk.row_col, pk.row_val,
-                                                                         pk.S, y, pc.nv, pc.nu, g->dev.view_order);
+                                                                         pk.S, y, pc.nv, pc.nvs, pc.nu, g->dev.view_order);
     return cuda_check(cudaGetLastError(), "plane forward launch");
 }
 
@@ -529,10 +549,10 @@ static spl_status plane_adjoint_t_n(const spl_geometry *g, const float *y, cudaS
     const PlanePack &pk = pg.pack[N];
     const PlaneCall pc = call_of(g);
     dim3 tg((pc.nu + 31) / 32, (pc.nv + 31) / 32, pg.n_views);
-    k_plane_ytrans<<<tg, 256, 0, st>>>(y, pk.yt, g->dev.view_order, pc.nu, pc.nv);
+    k_plane_ytrans<<<tg, 256, 0, st>>>(y, pk.yt, g->dev.view_order, pc.nu, pc.nv, pc.nvs);
     const unsigned blocks = (unsigned)((pg.ncol + kPlaneWarps - 1) / kPlaneWarps);
     k_plane_gather<true, false><<<blocks, 32 * kPlaneWarps, 0, st>>>(pg.ncol, pk.col_ptr, pk.col_row, pk.col_val, pk.yt,
-                                                                     pk.T, pc.nv, pc.nu, nullptr);
+                                                                     pk.T, pc.nv, pc.nvs, pc.nu, nullptr);
     return cuda_check(cudaGetLastError(), "plane adjoint launch");
 }
 

@@ -685,7 +685,7 @@ static spl_status adjoint_scatter(const spl_geometry *g, const float *y, float *
         has_total = true;
         k_acc_add<<<stream_grid(nc), 256, 0, st>>>(nc, g->acc64, c);
     };
-    if (batched && has_c) add_c();
+    if (batched && has_c && (flat || rest)) add_c();
     if (flat) {
         const unsigned gx = (dg.nu + 15) / 16, gy = (dg.nv + 7) / 8;
         if (!batched && !has_c) clear_c();

@@ -247,10 +247,7 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
                 bweights<N>(t, wd);
                 bweights<N>(fmaf(ra, t, ga), wa);
                 bweights<N>(fmaf(rb, t, gb), wb);
-                const float cw = hs * wt;
-#pragma unroll
-                for (int d = 0; d <= N; ++d) wd[d] *= cw;
-                window_update<N>(acc, wd, wa, wb);
+                window_update<N>(acc, wd, wa, wb, hs * wt);
             };
             if constexpr (N == 3) {
                 if (__any_sync(__activemask(), t1 - t0 > __uint_as_float(yl.y))) {

@@ -55,9 +55,9 @@ struct PlanePack {
     int *lb0;                  // [nv] first b-basis whose support holds detector row v
     float *wz;                 // [nv][degree+1] beta^n(z_v - l_b), l_b = lb0[v] + i
     int *vr;                   // [n_b][2] rows v whose b-window holds basis l_b (inclusive range)
-    float *S;                  // [ncol][nv] forward scratch: c resampled along b
-    float *T;                  // [ncol][nv] adjoint scratch
-    float *yt;                 // [rows][nv] adjoint scratch: y of the group, transposed
+    float *S;                  // [ncol][nvs] forward scratch: c resampled along b (nvs: nv rounded up to even)
+    float *T;                  // [ncol][nvs] adjoint scratch
+    float *yt;                 // [rows][nvs] adjoint scratch: y of the group, transposed
 };
 
 // Slice-separable view group of a parallel geometry (host object).

@@ -547,14 +547,17 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float v)
 // packed FP32x2 multiplies and FMAs two k at a time (__fmul2_rn,
 // __ffma2_rn: each component rounds like the scalar operation, so the sums
 // are those of the scalar loop, in half the instructions).
+// cw: a factor (the node's weight), taken into the b pairs, where it is two
+// packed multiplies (in the four d weights it was four).
 template <int N>
 __device__ __forceinline__ void window_update(float (&acc)[N + 1][N + 1][N + 1], const float (&wd)[N + 1],
-                                              const float (&wa)[N + 1], const float (&wb)[N + 1])
+                                              const float (&wa)[N + 1], float (&wb)[N + 1], float cw)
 {
     constexpr int K2 = (N + 1) / 2;
     if constexpr (N == 3) {
         // pairs (3, 0) and (1, 2): the register pairs bweights<3> produces
-        const float2 b30 = make_float2(wb[3], wb[0]), b12 = make_float2(wb[1], wb[2]);
+        const float2 b30 = __fmul2_rn(make_float2(cw, cw), make_float2(wb[3], wb[0])),
+                     b12 = __fmul2_rn(make_float2(cw, cw), make_float2(wb[1], wb[2]));
 #pragma unroll
         for (int i = 0; i <= N; ++i) {
             const float2 a2 = make_float2(wa[i], wa[i]);
@@ -574,6 +577,8 @@ __device__ __forceinline__ void window_update(float (&acc)[N + 1][N + 1][N + 1],
         }
         return;
     }
+#pragma unroll
+    for (int k = 0; k <= N; ++k) wb[k] *= cw;
 #pragma unroll
     for (int i = 0; i <= N; ++i) {
         float2 pk[K2 > 0 ? K2 : 1];
@@ -741,14 +746,14 @@ __device__ __forceinline__ bool cell_march(const RaySetup &rs, int cf, int cl, c
                     bweights<N>(t, wd);
                     bweights<N>(fmaf(rs.ra, t, ga), wa);
                     const float cw = half * (FLAT ? qr.w1[q] : qr.w[q]);
-#pragma unroll
-                    for (int d = 0; d <= N; ++d) wd[d] *= cw;
                     if constexpr (FLAT) {
+#pragma unroll
+                        for (int d = 0; d <= N; ++d) wd[d] *= cw;
                         window_update_flat<N>(acc, wd, wa);
                     } else {
                         float wb[N + 1];
                         bweights<N>(fmaf(rs.rb, t, gb), wb);
-                        window_update<N>(acc, wd, wa, wb);
+                        window_update<N>(acc, wd, wa, wb, cw);
                     }
                 }
                 sink.piece();
@@ -884,10 +889,7 @@ __device__ __forceinline__ bool piece_march(const RaySetup &rs, int cf, int cl, 
                 bweights<N>(t, wd);
                 bweights<N>(fmaf(rs.ra, t, ga), wa);
                 bweights<N>(fmaf(rs.rb, t, gb), wb);
-                const float cw = half * qr.w[q];
-#pragma unroll
-                for (int d = 0; d <= N; ++d) wd[d] *= cw;
-                window_update<N>(acc, wd, wa, wb);
+                window_update<N>(acc, wd, wa, wb, half * qr.w[q]);
             }
             sink.piece();
         }

@@ -790,3 +790,27 @@ def test_plane_matrix_arrays_are_whole(env, degree):
             # the same footprint values, another FP32 summation order
             assert float((a - b).abs().max()) <= 1e-5 * float(b.abs().max())
         keep.append(pair)
+
+
+@pytest.mark.parametrize("nv", [1, 63, 130, 257])
+def test_plane_gather_pairs(env, orc, nv):
+    """Detector heights at the plane gather's edges (odd heights, whose last
+    row is half a pair; more rows than one pass of 256) against the plain
+    march: the same footprint values, another summation order."""
+    torch, spl = env
+    dims = (14, 11, 30)
+    geo = I.tilt_series(5, 20, nv, 0.45)
+    g = spl.Geometry(dims, I.centred_origin(dims), geo)
+    torch.manual_seed(nv)
+    c, y = torch.randn(g.coeff_shape, device="cuda"), torch.randn(g.shape, device="cuda")
+    for degree in (1, 3):
+        got = []
+        for sep in (spl.SPL_SEP_AUTO, spl.SPL_SEP_OFF):
+            p = torch.full(g.shape, float("nan"), device="cuda")
+            b = torch.full(g.coeff_shape, float("nan"), device="cuda")
+            spl.forward(g, c, p, spl.basis(degree, separable=sep))
+            spl.adjoint(g, y, b, spl.basis(degree, separable=sep))
+            got.append((p, b))
+        g.status()
+        for u, v in zip(*got):
+            assert float((u - v).abs().max()) <= 1e-5 * float(v.abs().max())
