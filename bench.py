@@ -62,17 +62,23 @@ if ROOT not in sys.path:
 METRIC = "A/A^T G-contributions/s (exact quadrature footprint, one CGLS iteration per step)"
 UNIT = "Gcontrib/s"
 
-# FP32 arithmetic per Gauss node of the cell march (node position, two
-# transverse arguments, three sets of n+1 B-spline weights, node weight,
-# d-weight scaling, (n+1)^2 transverse products, (n+1)^3 FMAs) and per flushed
-# contribution (one FMA).
+# FP32 arithmetic per Gauss node of the footprint march (node position, two
+# transverse arguments, three sets of n+1 B-spline weights, node weight, its
+# product with one set, (n+1)^2 transverse products, (n+1)^3 FMAs), and per
+# contribution of a forward with footprints (one FMA).
 FLOP_PER_NODE = {0: 11, 1: 32, 2: 94, 3: 200}
 # flat rays (a zero direction component): n+1 nodes per piece, no b-weights,
 # an (n+1)^2 update per node
 FLOP_PER_FLAT_NODE = {0: 8, 1: 17, 2: 40, 3: 71}
 MLP_FLOP_PER_PAIR = 2 * (5 * 64 + 2 * 64 * 64 + 64)
 FLOP_PER_PAIR = 2
-NODES_PER_PIECE = {0: 1, 1: 2, 2: 4, 3: 5}
+# the fewest nodes a piece is integrated with (cubic pieces take four or five,
+# so the cubic work is counted from below)
+NODES_PER_PIECE = {0: 1, 1: 2, 2: 4, 3: 4}
+# the forward on resampled coefficients contracts (n+1)^2 columns per node:
+# position 2, two arguments 4, tau^2 1, two weight sets, per column the even and
+# odd parts (4) and their weighting (4), per row its weighting (4), node 6
+FLOP_PER_NODE_FORWARD = {0: 11, 1: 43, 2: 113, 3: 187}
 # views per batch of the scatter adjoint (FP32 atomics within a batch, FP64
 # totals across batches when a geometry has more views than this)
 ADJ_BATCH_VIEWS = 48
@@ -80,11 +86,11 @@ ADJ_BATCH_VIEWS = 48
 
 def launches_per_cg_step(n_views: int, scatter: bool = True) -> int:
     """Kernels of the library launched by one CGLS iteration on a cone
-    geometry of n_views views: A (one launch), two FP64 dots (two kernels
-    each), the x/r and p updates, and A^T: per batch of 48 views the scatter
-    and the folds of its two layout copies, plus the batch's FP64 total
-    (and the final rounding) when there is more than one batch; the brick
-    gather is one launch."""
+    geometry of n_views views: two FP64 dots (two kernels each), the x/r and
+    p updates, A (the resampling of the coefficients and the march) and, per
+    batch of 48 views of A^T, the scatter and the folds of three layouts:
+    8 + 4 per batch.  With one batch, or the brick gather (one launch), the
+    returned count is the lower one of a forward without resampling."""
     if not scatter:
         return 1 + 4 + 2 + 1
     batched = n_views > ADJ_BATCH_VIEWS
@@ -719,16 +725,15 @@ def run_ours(args):
     geom.status()
 
     peak = fp32_peak(dev, local)
-    # dominant kernel: the slower of A (k_forward_views) and A^T
-    # (k_adjoint_views_scatter) on the cone views; its algorithmic FP32 work
-    # is the nodes it integrates plus one FMA per contribution (this rank's
-    # share of the work: the launch covers its views)
-    flops = (pieces * NODES_PER_PIECE[n] * FLOP_PER_NODE[n] + flat_pieces * (n + 1) * FLOP_PER_FLAT_NODE[n]
-             + pairs * FLOP_PER_PAIR) / ws
+    # dominant kernel: the slower of A (k_line_views) and A^T
+    # (k_scatter_views) on the cone views; its algorithmic FP32 work is the
+    # nodes it integrates, counted from below (this rank's share of the work:
+    # the launch covers its views)
     if fwd >= adj:
-        kname, dom_ms = "k_forward_views", fwd
+        kname, dom_ms, per_node = "k_line_views", fwd, FLOP_PER_NODE_FORWARD[n]
     else:
-        kname, dom_ms = ("k_adjoint_bricks" if args.adjoint == "gather" else "k_adjoint_views_scatter"), adj
+        kname, dom_ms, per_node = ("k_adjoint_bricks" if args.adjoint == "gather" else "k_scatter_views"), adj, FLOP_PER_NODE[n]
+    flops = (pieces * NODES_PER_PIECE[n] * per_node + flat_pieces * (n + 1) * FLOP_PER_FLAT_NODE[n]) / ws
     achieved = flops / (dom_ms * 1e-3) / 1e12
     workload_tag = wl.name + "-cubic"
     roofline = {"bound": "alu", "kernel": kname, "achieved": achieved, "peak": peak["peak"], "unit": "TFLOP/s",

@@ -129,7 +129,7 @@ template <int N> struct MlpSmem {
 template <int N, bool ADJ>
 __global__ void __launch_bounds__(kMlpThreads *kMlpGroups, 2)
     k_mlp_views(DevGeom g, MlpDev wts, const float *__restrict__ cin, float *__restrict__ yout, const float *__restrict__ yin,
-                float *__restrict__ cout, QuadRule qr)
+                float *__restrict__ cout, QuadRule qr, int split)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     MlpSmem<N> &M = *reinterpret_cast<MlpSmem<N> *>(smem);
@@ -145,7 +145,8 @@ __global__ void __launch_bounds__(kMlpThreads *kMlpGroups, 2)
     }
     tc_mlp_setup(wts, M.tc);  // ends with a CTA barrier
     const int iu = (blockIdx.x * kMlpGroups + grp) * 8 + (lane & 7), iv = blockIdx.y * 16 + wid * 4 + (lane >> 3);
-    const int k = blockIdx.z;
+    // view, and which of the `split` equal parts of every ray's slabs
+    const int k = blockIdx.z / split, part = blockIdx.z % split;
     const bool valid = iu < g.nu && iv < g.nv;
     const long long ray = ((long long)k * g.nv + (valid ? iv : 0)) * g.nu + (valid ? iu : 0);
     RaySetup rs;
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(kMlpThreads *kMlpGroups, 2)
     T.rec[tid].c = make_int4(0, 0, rs.S[1], rs.S[2]);
     T.acc[tid] = 0.0f;
     T.yv[tid] = yr;
-    const int nslab = rs.j1 - rs.j0 + 1;
+    const int slabs = rs.j1 - rs.j0 + 1, first = slabs * part / split, nslab = slabs * (part + 1) / split - first;
     if (nslab > 0) atomicMax(&T.rounds, nslab);
     tc::bar_sync(bar, kMlpThreads);
     const int rounds = T.rounds;
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(kMlpThreads *kMlpGroups, 2)
             sk.q = q;
             sk.tab = &T;
             sk.cap = cap;
-            sk.j = rs.j0 + round;
+            sk.j = rs.j0 + first + round;
             sk.S0 = rs.S[0];
             sk.S1 = rs.S[1];
             sk.S2 = rs.S[2];
@@ -234,8 +235,27 @@ __global__ void __launch_bounds__(kMlpThreads *kMlpGroups, 2)
     }
     if (!ok) atomicOr(g.err, kErrStepCap);
     if (timeout && tid == 0) atomicOr(g.err, kErrTimeout);
-    if (!ADJ && valid) yout[ray] = timeout ? __int_as_float(0x7FC00000) : T.acc[tid];
+    if (!ADJ && valid) {
+        const float v = timeout ? __int_as_float(0x7FC00000) : T.acc[tid];
+        if (split == 1) yout[ray] = v;
+        else atomicAdd(yout + ray, v);  // zeroed by the host
+    }
     tc_mlp_teardown(M.tc, tile, phase, timeout);
+}
+
+// Into how many parts each ray's slabs are divided: a CTA works through a
+// whole detector tile, so few CTAs leave SMs idle (450 tiles on 152 SMs put
+// four groups on some and two on others: 7 % slower than three CTAs a SM had
+// been).  Twice as many until there are 32 CTAs per resident one, while a part
+// keeps 8 slabs.  6 views of the 256^3 cone (11.4 waves, then 45): A 229 ->
+// 217 ms, A^T 226 -> 215; one view of 138 x 92 through 89^3: 5.2 ms before, 1.2;
+// 11 views of 97 x 92 through 71^3: 6.4 and 3.3.
+static int mlp_split(const DevGeom &g, long long ctas)
+{
+    const int n = g.n[0] < g.n[1] ? (g.n[0] < g.n[2] ? g.n[0] : g.n[2]) : (g.n[1] < g.n[2] ? g.n[1] : g.n[2]);
+    int s = 1;
+    while (s < 16 && ctas * s < 32LL * 2 * sm_count() && n / (2 * s) >= 8 && (long long)g.n_views * 2 * s <= 65535) s *= 2;
+    return s;
 }
 
 template <int N, bool ADJ>
@@ -249,8 +269,14 @@ static spl_status launch_mlp_views(const spl_geometry *g, const spl_mlp *m, cons
         spl_status s = smem_attr_once((const void *)k_mlp_views<N, ADJ>, (int)sm, "mlp smem attribute");
         if (s != SPL_OK) return s;
     }
-    dim3 grid((dg.nu + 8 * kMlpGroups - 1) / (8 * kMlpGroups), (dg.nv + 15) / 16, dg.n_views);
-    k_mlp_views<N, ADJ><<<grid, kMlpThreads * kMlpGroups, sm, st>>>(dg, mlp_dev(m), cin, yout, yin, cout, quad_rule(N));
+    const int gx = (dg.nu + 8 * kMlpGroups - 1) / (8 * kMlpGroups), gy = (dg.nv + 15) / 16;
+    const int split = mlp_split(dg, (long long)gx * gy * dg.n_views);
+    if (!ADJ && split > 1) {
+        const spl_status s = cuda_check(cudaMemsetAsync(yout, 0, dg.n_rays * sizeof(float), st), "projection clear");
+        if (s != SPL_OK) return s;
+    }
+    k_mlp_views<N, ADJ><<<dim3(gx, gy, dg.n_views * split), kMlpThreads * kMlpGroups, sm, st>>>(
+        dg, mlp_dev(m), cin, yout, yin, cout, quad_rule(N), split);
     return cuda_check(cudaGetLastError(), "mlp projector launch");
 }
 
