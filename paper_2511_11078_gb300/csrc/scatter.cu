@@ -19,7 +19,8 @@
 // in registers (4 blocks of 128 threads per SM); the ray's constants sit in
 // shared memory.  Positions are 64-bit fixed point (spl_line.cuh), one add per
 // cell and axis.  Bound by issue and the FMA pipe together (60 and 62 % busy
-// on 8 views of the 256^3 cone), with the L2's tag lookups at 66 %.  Against
+// on 8 views of the 256^3 cone, the L2's tag lookups at 66 %) and by those tag
+// lookups on the 512^3 helical views (86 %).  Against
 // the mirrored march with bounds tests and double-float positions at 3 blocks
 // per SM: 8 such views 9.5 -> 7.3 ms, 8 helical views of 512^3 71.2 -> 56.2, 64
 // general parallel views of 128^3 8.4 -> 5.9, quadratic 180 x 180 x 50 8.5 ->
