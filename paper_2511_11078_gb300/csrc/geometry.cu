@@ -507,6 +507,13 @@ extern "C" spl_status spl_make_geometry(const spl_geometry_desc *desc, spl_geome
         return ss;
     }
     line_create(g, d.ray_omega);
+    // The uploads and clears above went to the default stream; a first call on
+    // a stream that does not synchronise with it would run beside them.
+    const spl_status sync = cuda_check(cudaStreamSynchronize(0), "geometry upload");
+    if (sync != SPL_OK) {
+        spl_destroy_geometry(g);
+        return sync;
+    }
     *out = g;
     return SPL_OK;
 }

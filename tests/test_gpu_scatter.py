@@ -144,3 +144,28 @@ def test_flat_and_general_views_in_batches(env, orc):
         g.status()
         err = np.linalg.norm(out.cpu().numpy() - ref) / np.linalg.norm(ref)
         assert err <= TOL, err
+
+
+def test_first_adjoint_on_a_side_stream(env):
+    """The first call of a fresh geometry on a stream that does not wait for
+    the default one: the layouts (1.7 GB, in memory that held NaN) must be
+    clear by then.  Against the same call later on the default stream; two
+    runs differ by the order of the atomics only."""
+    torch, spl = env
+    rng = np.random.default_rng(11)
+    dims = (320, 310, 300)
+    w = I.random_directions(rng, 3000)
+    s = rng.uniform(-0.4, 0.4, size=w.shape) * np.asarray(dims)
+    poison = torch.full((3, 1 << 27), float("nan"), device="cuda")
+    y = torch.randn(len(w), device="cuda")
+    first, later = (torch.empty(dims[::-1], device="cuda") for _ in range(2))
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    del poison
+    torch.cuda.empty_cache()
+    g = spl.Geometry(dims, I.centred_origin(dims), I.RayGeometry(w, s))
+    spl.adjoint(g, y, first, spl.basis(3), stream=side)
+    torch.cuda.synchronize()
+    spl.adjoint(g, y, later, spl.basis(3))
+    g.status()
+    assert float((first - later).norm() / later.norm()) <= TOL
