@@ -265,7 +265,10 @@ __device__ __forceinline__ void tc_mlp_setup(const MlpDev &w, TcMlpSmem<GROUPS> 
         }
         tc::fence_mbar_init();
     }
-    if (tid < 32) tc::alloc(&S.tile[0].tmem, kTcCols * GROUPS);
+    if (tid < 32) {
+        __syncwarp();  // lane 0 comes from a branch of its own, the allocation is warp-wide
+        tc::alloc(&S.tile[0].tmem, kTcCols * GROUPS);
+    }
     tc::fence_proxy_async();
     tc::fence_before();
     __syncthreads();
@@ -317,7 +320,6 @@ __device__ __forceinline__ bool tc_layer(const TcMlpImage &img, TcTile &T, int t
     }
     ok = tc::mbar_wait(&T.mbar, phase, ok ? tc::kWaitPolls : 1u) && ok;
     phase ^= 1u;
-    __syncwarp();  // tcgen05.ld is warp-wide
     tc::fence_after();
     return ok;
 }
@@ -328,10 +330,13 @@ __device__ __forceinline__ bool tc_layer(const TcMlpImage &img, TcTile &T, int t
 // work per thread, for batches too small to fill the GPU with 128-row tiles.
 // (threadIdx.x & 96 is the warp's TMEM lane quarter, 32 * (warp % 4).)
 
-// Columns C0 .. C0 + 31 of this thread's row of the accumulator.
+// Columns C0 .. C0 + 31 of this thread's row of the accumulator.  tcgen05.ld is
+// warp-wide, and the lanes may come apart before it: in the completion wait,
+// and where only some of them repeat their SiLU values (tc_silu_store).
 template <int C0>
 __device__ __forceinline__ void tc_cols(uint32_t tmem, float (&z)[32])
 {
+    __syncwarp();
     tc::ld32<0>(tmem + ((uint32_t)(threadIdx.x & 96) << 16) + (uint32_t)C0, z);
     tc::wait_ld();
 }

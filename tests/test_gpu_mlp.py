@@ -470,3 +470,47 @@ def test_mlp_projector_split_slabs(env, orc, dims):
     lhs = float((y.double() * z.double()).sum())
     rhs = float((torch.tensor(c, device="cuda").double() * b.double()).sum())
     assert abs(lhs - rhs) <= 1e-5 * float(y.double().norm() * z.double().norm())
+
+
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_mlp_projector_far_negative_in_some_rows(env, orc, adjoint):
+    """One thread per row (the projector), with pre-activations whose sign and
+    size follow the row's offset: in each layer some rows of a warp take their
+    SiLU values one by one and the others do not, so the lanes reach the next
+    accumulator load apart.  Against the oracle's projector; the adjoint
+    through <A c, z> = <c, A^T z>."""
+    torch, spl, learn = env
+    rng = np.random.default_rng(5800)
+    prm = random_params(rng, 0.8)
+    W1, W2, W3 = prm[:320].reshape(64, 5), prm[384:4480].reshape(64, 64), prm[4544:8640].reshape(64, 64)
+    # offsets x4 in [-3, 3]: z1 = 32 x4 and -16 x4, z2 = -32 x4 and less (units 8 .. 11) from the first four,
+    # z3 = 16 x4 and less (units 12 .. 15) from the next four; the other units see them weakly
+    W1[:8] = 0.0
+    W1[:4, 3], W1[4:8, 3] = 32.0, -16.0
+    W2[:, :8] *= 2.0 ** -7
+    W2[8:12, :4], W2[12:16, 4:8] = -0.25, 0.25
+    W3[:, 12:16] *= 2.0 ** -7
+    W3[12:16, 12:16] = -0.25
+    m = spl.Mlp(3, max_batch=64, seed=6)
+    m.set_params(prm)
+    dims = (14, 13, 15)
+    origin = I.centred_origin(dims)
+    geo = I.parallel_views(I.random_directions(rng, 3), 19, 17, 0.9, center=(0.13, 0.21, 0.07))
+    g = spl.Geometry(dims, origin, geo)
+    c = rng.uniform(0, 1, size=dims[::-1]).astype(np.float32)
+    ct, y = torch.tensor(c, device="cuda"), torch.full((g.n_rays,), float("nan"), device="cuda")
+    spl.forward(g, ct, y, spl.basis(3, spl.SPL_FP_MLP, m))
+    g.status()
+    if adjoint:
+        z = torch.tensor(rng.normal(size=g.n_rays).astype(np.float32), device="cuda")
+        b = torch.empty(g.coeff_shape, device="cuda")
+        spl.adjoint(g, z, b, spl.basis(3, spl.SPL_FP_MLP, m))
+        g.status()
+        lhs, rhs = float((y.double() * z.double()).sum()), float((ct.double() * b.double()).sum())
+        assert abs(lhs - rhs) <= 1e-5 * float(y.double().norm() * z.double().norm())
+        return
+    og = orc.Geometry("parallel", direction=geo.src, det_center=geo.det_center, det_u=geo.det_u, det_v=geo.det_v,
+                      nu=geo.nu, nv=geo.nv)
+    ref = orc.forward_mlp(3, dims, origin, c.astype(np.float64), og, SIZES, prm.astype(np.float64), mode=1)
+    got = y.cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - ref) <= 2e-3 * np.linalg.norm(ref)
