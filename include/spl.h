@@ -217,8 +217,8 @@ spl_status spl_geometry_status(const spl_geometry *g, void *stream);
  * it has run, spl_forward / spl_adjoint refuse such a basis with
  * SPL_ERR_STATE.  Geometries without separable views,
  * basis->separable == SPL_SEP_OFF and the MLP footprint need nothing.  The
- * plane buffers include the scratch of S and of its adjoint, so calls on
- * one geometry must not overlap on the GPU.
+ * plane buffers include the scratch of S and of its adjoint; which calls on
+ * one geometry may overlap is said at spl_forward.
  * Errors: SPL_ERR_ARG; SPL_ERR_OOM (plane matrices: the path stays off for
  * this geometry and degree, and spl_forward / spl_adjoint then walk those
  * views like the others and succeed; tables: SPL_FP_TABLE stays
@@ -237,9 +237,12 @@ spl_status spl_prepare(spl_geometry *g, const spl_basis_desc *basis, void *strea
  * keep an (n+1)^3 window of the bases whose support contains the current
  * point (Algorithm 3's neighbourhood, de-duplicated by construction), and
  * each basis the ray crosses adds c_k * Pphi(w, s - X(k)) once.  The two are
- * the same matrix and agree to FP32 rounding.  Calls on one geometry from
+ * the same matrix and agree to FP32 rounding.  Forwards on one geometry from
  * several streams or threads may overlap: the library orders their use of
- * the scratch on the GPU.  Slice-separable views of a parallel geometry go through the plane
+ * its scratch (the resampled coefficients, the plane path's S) on the GPU.
+ * That does not hold for adjoints, nor for forwards captured into a CUDA
+ * graph on a geometry with a separable group: these must not overlap with
+ * any call on the geometry.  Slice-separable views of a parallel geometry go through the plane
  * matrices instead (see spl_prepare), with the same footprint values.
  *   Cone views: every ray is walked with the general (three-factor) form
  *   of the march, so a ray's values do not depend on its direction class.

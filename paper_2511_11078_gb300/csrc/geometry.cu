@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <mutex>
+#include <new>
 
 #include "spl_host.h"
 
@@ -75,6 +76,34 @@ spl_status smem_attr_once(const void *func, int bytes, const char *what)
     if (s != SPL_OK) return s;
     if (g_attr_n < (int)(sizeof(g_attr_done) / sizeof(g_attr_done[0]))) g_attr_done[g_attr_n++] = {func, dev};
     return SPL_OK;
+}
+
+spl_status turn_create(spl_geometry *g)
+{
+    ForwardTurn *t = new (std::nothrow) ForwardTurn();
+    if (!t) return fail(SPL_ERR_OOM, "host allocation failed");
+    t->used = false;
+    const spl_status s = cuda_check(cudaEventCreateWithFlags(&t->last, cudaEventDisableTiming), "turn event");
+    if (s == SPL_OK) g->turn = t;
+    else delete t;
+    return s;
+}
+
+void turn_free(ForwardTurn *t)
+{
+    if (!t) return;
+    cudaEventDestroy(t->last);
+    delete t;
+}
+
+bool stream_captures(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;  // (the default stream while another one captures)
+    }
+    return cap != cudaStreamCaptureStatusNone;
 }
 
 // ---------------------------------------------------------------- quadrature
@@ -509,7 +538,8 @@ extern "C" spl_status spl_make_geometry(const spl_geometry_desc *desc, spl_geome
     line_create(g, d.ray_omega);
     // The uploads and clears above went to the default stream; a first call on
     // a stream that does not synchronise with it would run beside them.
-    const spl_status sync = cuda_check(cudaStreamSynchronize(0), "geometry upload");
+    spl_status sync = cuda_check(cudaStreamSynchronize(0), "geometry upload");
+    if (sync == SPL_OK && (g->line || g->plane)) sync = turn_create(g);
     if (sync != SPL_OK) {
         spl_destroy_geometry(g);
         return sync;
@@ -524,6 +554,7 @@ extern "C" void spl_destroy_geometry(spl_geometry *g)
     plane_free(g->plane);
     table_free(g->table);
     line_free(g->line);
+    turn_free(g->turn);
     free(g->vconst);
     if (g->acc64) cudaFree(g->acc64);
     scatter_free(g->scatter);

@@ -32,7 +32,6 @@
 // against FP64 is 2.8e-8 (1.25e-7 cubic, 4.3e-8 linear and quadratic).
 #include <math.h>
 
-#include <mutex>
 #include <new>
 
 #include "spl_host.h"
@@ -444,15 +443,11 @@ __global__ void __launch_bounds__(128, LineBlocks<N>::value)
 }
 
 // ---------------------------------------------------------------- host side
-// The resampled arrays of a geometry.  Calls on one geometry from several
-// streams or threads take turns on them: each call makes its stream wait for
-// the previous one's event, under the mutex.
+// The resampled arrays of a geometry; forwards take turns on them
+// (ForwardTurn).
 struct LineScratch {
     LineArrays arr;
     void *block;
-    cudaEvent_t last;
-    bool used;
-    std::mutex mu;
 };
 
 // Where the resampled form is the faster one (both sides measured on GB300):
@@ -510,13 +505,6 @@ void line_create(spl_geometry *g, const double *ray_dirs)
         delete ls;
         return;
     }
-    if (cudaEventCreateWithFlags(&ls->last, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(ls->block);
-        delete ls;
-        return;
-    }
-    ls->used = false;
     for (int d = 0; d < 3; ++d) ls->arr.a[d] = ((mask >> d) & 1u) ? (char *)ls->block + off[d] : nullptr;
     g->line = ls;
 }
@@ -524,23 +512,15 @@ void line_create(spl_geometry *g, const double *ray_dirs)
 void line_free(LineScratch *ls)
 {
     if (!ls) return;
-    cudaEventDestroy(ls->last);
     cudaFree(ls->block);
     delete ls;
 }
 
-bool line_usable(const spl_geometry *g, int degree, cudaStream_t st)
+bool line_usable(const spl_geometry *g, int degree, bool captured)
 {
-    if (!g->line || degree < 1) return false;
-    // a captured call cannot take its turn against calls outside the graph
-    // (an event of the one cannot be waited for in the other): it keeps the
-    // footprint form, which has no scratch
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return cap == cudaStreamCaptureStatusNone;
+    // a captured call takes no turn against calls outside the graph: it keeps
+    // the footprint form, which has no scratch
+    return g->line && degree >= 1 && !captured;
 }
 
 template <int N>
@@ -549,10 +529,6 @@ static spl_status line_forward_n(const spl_geometry *g, int kahan, const float *
     const DevGeom &dg = g->dev;
     LineScratch &S = *g->line;
     const QuadRule qr = quad_rule(N);
-    std::lock_guard<std::mutex> lock(S.mu);
-    spl_status s = SPL_OK;
-    if (S.used) s = cuda_check(cudaStreamWaitEvent(st, S.last, 0), "line scratch wait");
-    if (s != SPL_OK) return s;
     int gx = 0, gy = 0, zc[3];
     for (int d = 0; d < 3; ++d) {
         zc[d] = 0;
@@ -573,11 +549,7 @@ static spl_status line_forward_n(const spl_geometry *g, int kahan, const float *
         const int ls = line_split((long long)nview * dg.nu * dg.nv, LineBlocks<N>::value);
         k_line_views<N><<<line_grid(dg, nview, ls), 128, 0, st>>>(dg, S.arr, y, qr, kahan, order, ls);
     }
-    s = cuda_check(cudaGetLastError(), "line forward launch");
-    // recorded also after a failed launch: what did start still uses the scratch
-    const spl_status e = cuda_check(cudaEventRecord(S.last, st), "line scratch record");
-    S.used = true;
-    return s != SPL_OK ? s : e;
+    return cuda_check(cudaGetLastError(), "line forward launch");
 }
 
 spl_status line_forward(const spl_geometry *g, int degree, int kahan, const float *c, float *y, cudaStream_t st)

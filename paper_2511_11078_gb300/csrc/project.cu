@@ -587,13 +587,12 @@ static int plane_views(const spl_geometry *g, const spl_basis_desc *b, spl_statu
 
 template <int N, bool DIRECT>
 static spl_status forward_quad_t(const spl_geometry *g, const spl_basis_desc *b, const float *c, float *y,
-                                 cudaStream_t st)
+                                 bool captured, cudaStream_t st)
 {
     const DevGeom &dg = g->dev;
     const QuadRule qr = quad_rule(N);
     const int kahan = b->kahan;
-    if (dg.n_rays == 0) return SPL_OK;
-    const bool line = line_usable(g, N, st);
+    const bool line = line_usable(g, N, captured);
     if (line && dg.kind != SPL_PARALLEL) return line_forward(g, N, kahan, c, y, st);
     if (dg.kind == SPL_RAYS) {
         const long long blocks = (dg.n_rays + 127) / 128;
@@ -650,7 +649,22 @@ static spl_status forward_quad_t(const spl_geometry *g, const spl_basis_desc *b,
 template <int N>
 static spl_status forward_quad(const spl_geometry *g, const spl_basis_desc *b, const float *c, float *y, cudaStream_t st)
 {
-    return b->mode == SPL_FP_DIRECT ? forward_quad_t<N, true>(g, b, c, y, st) : forward_quad_t<N, false>(g, b, c, y, st);
+    if (g->dev.n_rays == 0) return SPL_OK;
+    auto run = [&](bool captured) {
+        return b->mode == SPL_FP_DIRECT ? forward_quad_t<N, true>(g, b, c, y, captured, st)
+                                        : forward_quad_t<N, false>(g, b, c, y, captured, st);
+    };
+    ForwardTurn *t = g->turn;
+    if (!t) return run(false);
+    if (stream_captures(st)) return run(true);
+    std::lock_guard<std::mutex> lock(t->mu);
+    spl_status s = t->used ? cuda_check(cudaStreamWaitEvent(st, t->last, 0), "forward turn wait") : SPL_OK;
+    if (s != SPL_OK) return s;
+    s = run(false);
+    // recorded also after a failure: what did start still uses the scratch
+    const spl_status e = cuda_check(cudaEventRecord(t->last, st), "forward turn record");
+    t->used = true;
+    return s != SPL_OK ? s : e;
 }
 
 // The scatter form over the views from v0 of the view order (or all rays):

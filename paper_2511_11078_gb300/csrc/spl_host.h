@@ -4,6 +4,8 @@
 
 #include <cuda_runtime.h>
 
+#include <mutex>
+
 #include "spl.h"
 #include "spl_march.cuh"
 
@@ -12,6 +14,7 @@ struct PlaneGroup;
 struct TableSet;
 struct LineScratch;
 struct ScatterScratch;
+struct ForwardTurn;
 }
 
 struct spl_geometry {
@@ -26,6 +29,7 @@ struct spl_geometry {
     double *acc64;                // FP64 accumulator of the scatter adjoint's batches (nx*ny*nz), or NULL
     spl::ScatterScratch *scatter; // the scatter adjoint's layout copies of c (scatter.cu), or NULL (no rays;
                                   // parallel geometries whose views are all flat)
+    spl::ForwardTurn *turn;       // order of the forwards that use scratch, or NULL (there is none)
     spl::LineScratch *line;       // the forward's resampled coefficients (line.cu), or NULL (not needed or too large)
 };
 
@@ -128,14 +132,28 @@ spl_status table_forward(const spl_geometry *g, const spl_basis_desc *b, const f
 spl_status table_adjoint(const spl_geometry *g, const spl_basis_desc *b, const float *y, float *c, cudaStream_t st);
 void table_free(TableSet *ts);
 
+// Forwards of one geometry from several streams or threads take turns on its
+// scratch (the resampled coefficients, the plane path's S, side stream and
+// events): each makes its stream wait for the event of the one before, under
+// the mutex.  A captured call cannot (an event of a graph cannot be waited for
+// outside of it) and takes no turn.
+struct ForwardTurn {
+    std::mutex mu;
+    cudaEvent_t last;
+    bool used;
+};
+spl_status turn_create(spl_geometry *g);
+void turn_free(ForwardTurn *t);
+bool stream_captures(cudaStream_t st);
+
 // The forward as line integrals of f on resampled coefficients (line.cu),
 // for explicit rays, cone views and the parallel views outside the flat
 // class.  line_create allocates its arrays with the geometry (leaves
 // g->line NULL when they are not needed, too large or not to be had);
-// line_usable: whether a call of this degree on this stream takes it.
+// line_usable: whether an eager call of this degree takes it.
 void line_create(spl_geometry *g, const double *ray_dirs);
 void line_free(LineScratch *ls);
-bool line_usable(const spl_geometry *g, int degree, cudaStream_t st);
+bool line_usable(const spl_geometry *g, int degree, bool captured);
 spl_status line_forward(const spl_geometry *g, int degree, int kahan, const float *c, float *y, cudaStream_t st);
 
 // The scatter adjoint of the same rays (scatter.cu).  scatter_rays reduces

@@ -160,3 +160,51 @@ def test_four_node_pieces_single_footprint(env, orc, ra, rb):
     ref = orc.forward(3, dims, I.centred_origin(dims), c.astype(np.float64), geom_of(orc, geo)).reshape(-1)
     scale = np.sqrt(1.0 + ra * ra + rb * rb)
     assert np.max(np.abs(y.cpu().numpy() - ref)) <= scale * (12 * 2.0 ** -28 + 20 * 2.0 ** -25)
+
+
+@pytest.mark.parametrize("mixed", [False, True])
+@pytest.mark.parametrize("threads", [False, True])
+def test_streams_take_turns_on_the_plane_path(env, mixed, threads):
+    """Forwards of a tilt series (and of one with other views, whose plane
+    path runs on the geometry's own stream) on two streams, from one thread
+    and from two: the results are those of calls in line, bit for bit."""
+    import threading
+
+    torch, spl = env
+    rng = np.random.default_rng(12)
+    dims = (70, 66, 60)
+    geo = I.tilt_series(60, 96, 88, 1.0)
+    if mixed:
+        other = I.parallel_views(I.random_directions(rng, 30), 96, 88, 1.0)
+        geo = I.ViewGeometry("parallel", *[np.concatenate([getattr(geo, f), getattr(other, f)])
+                                           for f in ("src", "det_center", "det_u", "det_v")], 96, 88)
+    g = spl.Geometry(dims, I.centred_origin(dims), geo)
+    bas = spl.basis(3)
+    spl.prepare(g, bas)
+    cs = [torch.tensor(rng.normal(size=dims[::-1]).astype(np.float32), device="cuda") for _ in range(2)]
+    ref = [torch.empty(g.n_rays, device="cuda") for _ in range(2)]
+    for c, y in zip(cs, ref):
+        spl.forward(g, c, y, bas)
+    torch.cuda.synchronize()
+    got = [[torch.empty(g.n_rays, device="cuda") for _ in range(6)] for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+
+    def calls(i, ks):
+        for k in ks:
+            spl.forward(g, cs[i], got[i][k], bas, stream=streams[i])
+
+    if threads:
+        both = [threading.Thread(target=calls, args=(i, range(6))) for i in range(2)]
+        for t in both:
+            t.start()
+        for t in both:
+            t.join()
+    else:
+        for k in range(6):
+            calls(0, [k])
+            calls(1, [k])
+    torch.cuda.synchronize()
+    g.status()
+    for i in range(2):
+        for y in got[i]:
+            assert torch.equal(y, ref[i])
