@@ -598,7 +598,8 @@ static spl_status scatter_n(const spl_geometry *g, const float *y, long long i0,
     if (S.dirty) {
         const spl_status s = cuda_check(cudaMemsetAsync(S.block, 0, S.bytes, st), "adjoint layout clear");
         if (s != SPL_OK) return s;
-        S.dirty = false;
+        // (a captured clear only runs when its graph does)
+        if (!stream_captures(st)) S.dirty = false;
     }
     if (dg.kind == SPL_RAYS) {
         const int ls = line_split(i1 - i0, ScatterBlocks<N>::value);

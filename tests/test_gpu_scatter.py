@@ -169,3 +169,48 @@ def test_first_adjoint_on_a_side_stream(env):
     spl.adjoint(g, y, later, spl.basis(3))
     g.status()
     assert float((first - later).norm() / later.norm()) <= TOL
+
+
+def test_captured_call_after_a_failed_one(env):
+    """A launch that fails (into a capture that a synchronisation made
+    invalid) leaves the layouts to be cleared before the next use.  A captured
+    call records that clear, which then runs with its graph only: the next
+    capture, and the next eager call, must clear as well."""
+    import ctypes as C
+
+    torch, spl = env
+    cu = C.CDLL("libcuda.so.1")
+    rng = np.random.default_rng(13)
+    w = I.random_directions(rng, 500)
+    s = rng.uniform(-0.6, 0.6, size=w.shape) * np.asarray(DIMS)
+    g = spl.Geometry(DIMS, I.centred_origin(DIMS), I.RayGeometry(w, s))
+    y = torch.randn(500, device="cuda")
+    ref, out = (torch.empty(g.coeff_shape, device="cuda") for _ in range(2))
+    spl.adjoint(g, y, ref, spl.basis(3))
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    raw = C.c_void_p(st.cuda_stream)
+
+    def capture(break_it=False):
+        graph, n = C.c_void_p(), C.c_size_t(0)
+        assert cu.cuStreamBeginCapture_v2(raw, 2) == 0  # relaxed
+        if break_it:
+            assert cu.cuStreamSynchronize(raw) != 0
+            with pytest.raises(spl.SplError):
+                spl.adjoint(g, y, out, spl.basis(3), stream=st)
+            assert cu.cuStreamEndCapture(raw, C.byref(graph)) != 0
+            return None
+        spl.adjoint(g, y, out, spl.basis(3), stream=st)
+        assert cu.cuStreamEndCapture(raw, C.byref(graph)) == 0
+        assert cu.cuGraphGetNodes(graph, None, C.byref(n)) == 0
+        assert cu.cuGraphDestroy(graph) == 0
+        return n.value
+
+    plain = capture()
+    capture(break_it=True)
+    assert [capture(), capture()] == [plain + 1, plain + 1]
+    spl.adjoint(g, y, out, spl.basis(3), stream=st)
+    torch.cuda.synchronize()
+    g.status()
+    assert float((out - ref).norm() / ref.norm()) <= TOL
+    assert capture() == plain
