@@ -164,8 +164,11 @@ typedef struct {
  * up to three layouts (x, y and z fast, those that some ray needs) of four
  * shifted copies each, on a grid padded by 3 (16 bytes per coefficient and
  * layout; not for a parallel geometry whose views are all in the
- * flat class) and, for more than 48 views or 2^22 explicit rays, an FP64
- * accumulator (8 nx ny nz bytes).  Scratch of the forward, for geometries
+ * flat class; explicit rays whose neighbours in the caller's order lie far
+ * apart take fewer copies, or one layout in single values, where four copies
+ * outgrow the L2) and, for more than 48 views, 2^22 explicit rays or such
+ * rays in several batches, an FP64 accumulator (8 nx ny nz bytes).  Scratch of
+ * the forward, for geometries
  * with rays outside the flat class: the coefficients resampled along each
  * axis that is the dominant one of some ray, 16 bytes per coefficient and
  * axis on a grid padded by 3 (left out where few rays cross a large grid,

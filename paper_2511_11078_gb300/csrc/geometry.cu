@@ -36,7 +36,7 @@ spl_status cuda_check(cudaError_t e, const char *what)
 namespace {
 constexpr int kMaxDev = 64;
 std::mutex g_dev_mutex;
-int g_sm_count[kMaxDev];             // 0: not queried yet
+int g_sm_count[kMaxDev], g_l2_bytes[kMaxDev];  // 0: not queried yet
 struct AttrDone {
     const void *func;
     int device;
@@ -45,24 +45,29 @@ AttrDone g_attr_done[256];
 int g_attr_n = 0;
 }  // namespace
 
-int sm_count()
+// a positive device attribute, kept in cache[device]; `fallback` on an error
+static int device_attr(int *cache, cudaDeviceAttr attr, int fallback)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
         cudaGetLastError();
-        return 1;
+        return fallback;
     }
     std::lock_guard<std::mutex> lock(g_dev_mutex);
-    if (g_sm_count[dev] == 0) {
+    if (cache[dev] == 0) {
         int n = 0;
-        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) {
+        if (cudaDeviceGetAttribute(&n, attr, dev) != cudaSuccess || n <= 0) {
             cudaGetLastError();
-            n = 1;
+            n = fallback;
         }
-        g_sm_count[dev] = n;
+        cache[dev] = n;
     }
-    return g_sm_count[dev];
+    return cache[dev];
 }
+
+int sm_count() { return device_attr(g_sm_count, cudaDevAttrMultiProcessorCount, 1); }
+
+size_t l2_bytes() { return (size_t)device_attr(g_l2_bytes, cudaDevAttrL2CacheSize, 1 << 26); }
 
 spl_status smem_attr_once(const void *func, int bytes, const char *what)
 {
@@ -504,11 +509,22 @@ extern "C" spl_status spl_make_geometry(const spl_geometry_desc *desc, spl_geome
     }
     dg.raw = (const double *)((const char *)blk + raw_off);
     dg.err = (int *)((char *)blk + flag_off);
+    // the scatter adjoint's layout copies of c (scratch, folded into c after
+    // each batch)
+    const spl_status ss = scatter_create(g, d.ray_omega, d.ray_s);
+    if (ss != SPL_OK) {
+        cudaFree(blk);
+        plane_free(g->plane);
+        free(g->vconst);
+        free(g->views_host);
+        free(g);
+        return ss;
+    }
     // The scatter adjoint of a geometry with more than one batch of views
     // (rays) adds the batches in an FP64 accumulator of the grid's size
     // (scratch sized here, so the adjoint itself allocates nothing).
     const long long nk = (long long)dg.n[0] * dg.n[1] * dg.n[2];
-    const bool batched = d.kind == SPL_RAYS ? dg.n_rays > kAdjBatchRays : d.n_views > kAdjBatchViews;
+    const bool batched = d.kind == SPL_RAYS ? dg.n_rays > kAdjBatchRays || scatter_in_batches(g) : d.n_views > kAdjBatchViews;
     g->acc64 = nullptr;
     if (batched && dg.n_rays > 0) {
         ce = cudaMalloc((void **)&g->acc64, (size_t)nk * sizeof(double));
@@ -516,24 +532,13 @@ extern "C" spl_status spl_make_geometry(const spl_geometry_desc *desc, spl_geome
             cudaGetLastError();
             g->acc64 = nullptr;
             cudaFree(blk);
+            scatter_free(g->scatter);
             plane_free(g->plane);
             free(g->vconst);
             free(g->views_host);
             free(g);
             return fail(SPL_ERR_OOM, "cudaMalloc of the adjoint accumulator (%lld doubles) failed", nk);
         }
-    }
-    // the scatter adjoint's layout copies of c (scratch, folded into c after
-    // each batch)
-    const spl_status ss = scatter_create(g, d.ray_omega);
-    if (ss != SPL_OK) {
-        if (g->acc64) cudaFree(g->acc64);
-        cudaFree(blk);
-        plane_free(g->plane);
-        free(g->vconst);
-        free(g->views_host);
-        free(g);
-        return ss;
     }
     line_create(g, d.ray_omega);
     // The uploads and clears above went to the default stream; a first call on

@@ -711,7 +711,8 @@ static spl_status adjoint_scatter(const spl_geometry *g, const float *y, float *
         }, batched ? kAdjBatchViews : kViewChunk);
         has_c = true;
     }
-    const long long per = !batched ? i1 : (dg.kind == SPL_RAYS ? kAdjBatchRays : kAdjBatchViews);
+    long long per = !batched ? i1 : (dg.kind == SPL_RAYS ? kAdjBatchRays : kAdjBatchViews);
+    if (batched && dg.kind == SPL_RAYS && scatter_batch(g, N) < per) per = scatter_batch(g, N);
     for (long long i = i0; rest && i < i1 && s == SPL_OK; i += per) {
         const bool last = i + per >= i1;
         s = scatter_rays(g, N, y, i, last ? i1 : i + per, st);

@@ -12,8 +12,11 @@
 // for n = 1) into the copy in which it starts a group.  Every axis is padded
 // on both sides, so no entry of a face needs a bounds test, and rows are
 // a multiple of 4 floats apart, so the copy is chosen once per b crossing and
-// not once per row.  k_scatter_fold adds the layouts into c (or the FP64
-// total of the batches) and leaves them cleared for the next call.
+// not once per row.  The values of a b event are single ones and go to copy 0
+// (8 helical views 56.2 -> 55.6 ms against the ray's current copy).  k_fold_*
+// add the layouts into c (or the FP64 total of the batches) and leave them
+// cleared for the next call.  Explicit rays that do not lie side by side take
+// fewer copies, or single values into one layout (scatter_form).
 //
 // The march keeps, next to its 64 accumulators, only what every piece needs
 // in registers (4 blocks of 128 threads per SM); the ray's constants sit in
@@ -45,6 +48,7 @@ template <int N> constexpr int kCopies = N == 0 ? 1 : (N == 1 ? 2 : 4);
 struct ScatterTarget {
     float *lay[3];  // contiguous axis x, y, z; NULL where no ray has it as b axis
     size_t cs;      // copy stride in floats, a multiple of 4
+    int one;        // the layout of every ray (form 0), or -1: that of its b axis
 };
 
 // Layout with contiguous axis b: rows of `row` floats (room for the shift and
@@ -74,7 +78,7 @@ struct __align__(16) ScatterRay {
     int c, cl;         // first and last cell (none: c > cl)
     int sd, sa;        // signed strides of d and a in the target
     float *base;       // target of window entry (0, 0, 0) at cell c, QA = QB = 0, in copy 0
-    long long pad;
+    int sb, pad;       // stride of b in the target
 };
 
 // The line {s + t w}, oriented so that its b component is >= 0 and mirrored
@@ -147,21 +151,24 @@ __device__ __forceinline__ void scatter_setup(const DevGeom &g, const ScatterTar
     R.B = __double2ll_rn(fma((double)c, rb, b0) * kOne);
     R.lim_a = na + N;
     R.lim_b = nb + N;
-    // strides of the layout whose contiguous axis is b: rows, then slabs
-    const ScatterDims D = scatter_dims(g.n, b);
-    const int st_d = d < a ? D.row : D.slab, st_a = d < a ? D.slab : D.row;
+    // strides of the layout with contiguous axis e: rows, then slabs
+    const int e = T.one >= 0 ? T.one : b;
+    const ScatterDims D = scatter_dims(g.n, e);
+    auto stride = [&](int x) { return x == e ? 1 : (x == (e == 2 ? 1 : 2) ? D.slab : D.row); };
+    const int st_d = stride(d), st_a = stride(a);
     R.sd = nd_ ? -st_d : st_d;
     R.sa = na_ ? -st_a : st_a;
+    R.sb = stride(b);
     // window entry (0, 0, 0) is basis (c - N, QA - N, QB - N); basis l sits at
     // l + kPad, a mirrored one at n - 1 - l + kPad
     const long long od = nd_ ? nd - 1 - (c - N) + kPad : c - N + kPad, oa = na_ ? na - 1 + N + kPad : kPad - N;
-    float *lay = sel3(b, T.lay[0], T.lay[1], T.lay[2]);
+    float *lay = sel3(e, T.lay[0], T.lay[1], T.lay[2]);
     if (!lay) {  // an axis that scatter_axes ruled out (not expected)
         atomicOr(g.err, 1);
         R.cl = c - 1;
         return;
     }
-    R.base = lay + (od * st_d + oa * st_a + (kPad - N));
+    R.base = lay + (od * st_d + oa * st_a + (long long)(kPad - N) * R.sb);
 }
 
 // ---------------------------------------------------------------- the march
@@ -173,27 +180,36 @@ __device__ __forceinline__ void red1(float *p, float v)
 {
     asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "f"(v) : "memory");
 }
-template <int N>
-__device__ __forceinline__ void row_add(float *p, const float (&v)[N + 1])
+__device__ __forceinline__ void red2(float *p, float v0, float v1)
 {
-    if constexpr (N >= 2)
+    asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(__cvta_generic_to_global(p)), "f"(v0), "f"(v1)
+                 : "memory");
+}
+// A row of N + 1 values along b, which starts on a boundary of CP floats;
+// CP = 0: values sb floats apart.
+template <int N, int CP>
+__device__ __forceinline__ void row_add(float *p, const float (&v)[N + 1], int sb)
+{
+    if constexpr (CP == 4)
         asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(__cvta_generic_to_global(p)),
                      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(N == 3 ? v[N] : 0.0f)
                      : "memory");
-    else if constexpr (N == 1)
-        asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(__cvta_generic_to_global(p)), "f"(v[0]),
-                     "f"(v[1])
-                     : "memory");
-    else
-        red1(p, v[0]);
+    else {
+        constexpr int P = CP == 2 ? (N + 1) / 2 : 0;
+#pragma unroll
+        for (int k = 0; k < P; ++k) red2(p + 2 * k, v[2 * k], v[2 * k + 1]);
+#pragma unroll
+        for (int k = 2 * P; k <= N; ++k) red1(p + (CP == 0 ? (long long)k * sb : k), v[k]);
+    }
 }
 
 // March over part `seg` of 2^ls equal parts of the ray's cells.  Returns
 // false if the event bound was reached.
-template <int N>
+template <int N, int CP>
 __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int ls, size_t cs, const QuadRule &qr)
 {
-    constexpr int M = GL<N>::M, CP = kCopies<N>;
+    constexpr int M = GL<N>::M, C1 = CP > 0 ? CP : 1;
+    const int sb = CP > 0 ? 1 : R.sb;
     const int cells = R.cl - R.c + 1, k0 = (int)(((long long)cells * seg) >> ls),
               k1 = (int)(((long long)cells * (seg + 1)) >> ls);
     if (k0 >= k1) return true;
@@ -202,12 +218,12 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
     int QA = (int)(A >> kLineFrac), QB = (int)(B >> kLineFrac);
     const float ra = R.ra, rb = R.rb;
     // target of window entry (0, 0, 0), at float lo = QB + kPad - N of its
-    // row: copy j = -lo mod CP holds it at lo + j, where a group starts
+    // row: copy j = -lo mod C1 holds it at lo + j, where a group starts
     constexpr int kLo = kPad - N;
     float *wp;
     {
-        const int j = -(QB + kLo) & (CP - 1);
-        wp = R.base + (long long)k0 * R.sd + (long long)QA * R.sa + (QB + j) + (long long)((size_t)j * cs);
+        const int j = -(QB + kLo) & (C1 - 1);
+        wp = R.base + (long long)k0 * R.sd + (long long)QA * R.sa + ((long long)QB * sb + j) + (long long)((size_t)j * cs);
     }
     float acc[N + 1][N + 1][N + 1];
 #pragma unroll
@@ -268,13 +284,14 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
         const bool evA = ta <= tb && ta <= 1.0f, evB = !evA && tb <= 1.0f, evD = !evA && !evB;
         const int2 st = make_int2(R.sd, R.sa);
         // the face that leaves: D: (0, x, .), A: (x, 0, .): rows along b;
-        // B: (x, y, 0): single values
+        // B: (x, y, 0): single values, into copy 0
         if (in) {
             if (evB) {
+                float *w0 = wp - (-(QB + kLo) & (C1 - 1)) * (long long)(cs + 1);
 #pragma unroll
                 for (int x = 0; x <= N; ++x)
 #pragma unroll
-                    for (int y = 0; y <= N; ++y) red1(wp + ((long long)x * st.x + (long long)y * st.y), acc[x][y][0]);
+                    for (int y = 0; y <= N; ++y) red1(w0 + ((long long)x * st.x + (long long)y * st.y), acc[x][y][0]);
             } else {
                 const long long sx = evD ? st.y : st.x;
 #pragma unroll
@@ -282,7 +299,7 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
                     float v[N + 1];
 #pragma unroll
                     for (int k = 0; k <= N; ++k) v[k] = evD ? acc[0][x][k] : acc[x][0][k];
-                    row_add<N>(wp + x * sx, v);
+                    row_add<N, CP>(wp + x * sx, v, sb);
                 }
             }
         }
@@ -310,12 +327,12 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
             wp += st.y;
         } else {
             // the row start moves on by one: the copy before holds it at the
-            // same position, copy 0's successor is copy CP - 1, CP further on
-            const bool last = ((QB + kLo) & (CP - 1)) == 0;
+            // same position, copy 0's successor is copy C1 - 1, C1 further on
+            const bool last = ((QB + kLo) & (C1 - 1)) == 0;
             ++QB;
             gb -= 1.0f;
             tb = 2.0f;
-            wp += last ? (long long)((CP - 1) * cs) + CP : -(long long)cs;
+            wp += last ? (long long)((C1 - 1) * cs) + C1 * sb : -(long long)cs;
         }
     }
     // what the window still holds (it is shifted: layers c + 1 - N ..), for a
@@ -326,7 +343,7 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
 #pragma unroll
         for (int d = 0; d < N; ++d)
 #pragma unroll
-            for (int i = 0; i <= N; ++i) row_add<N>(wp + ((long long)d * R.sd + (long long)i * R.sa), acc[d][i]);
+            for (int i = 0; i <= N; ++i) row_add<N, CP>(wp + ((long long)d * R.sd + (long long)i * R.sa), acc[d][i], sb);
     }
     return true;
 }
@@ -335,7 +352,7 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
 template <int N> struct ScatterBlocks { static constexpr int value = N == 3 ? 4 : (N == 2 ? 5 : 8); };
 
 // rays r0 .. r1 - 1, 2^ls threads each
-template <int N>
+template <int N, int CP>
 __global__ void __launch_bounds__(128, ScatterBlocks<N>::value)
     k_scatter_rays(DevGeom g, ScatterTarget T, const float *__restrict__ y, QuadRule qr, long long r0, long long r1, int ls)
 {
@@ -355,7 +372,7 @@ __global__ void __launch_bounds__(128, ScatterBlocks<N>::value)
         }
     }
     __syncthreads();
-    if (!scatter_march<N>(rays[t >> ls], t & ((1 << ls) - 1), ls, T.cs, qr)) atomicOr(g.err, 1);
+    if (!scatter_march<N, CP>(rays[t >> ls], t & ((1 << ls) - 1), ls, T.cs, qr)) atomicOr(g.err, 1);
 }
 
 // Whether a warp's eight consecutive lanes run along detector v: along the
@@ -396,7 +413,7 @@ __global__ void __launch_bounds__(128, ScatterBlocks<N>::value)
         }
     }
     __syncthreads();
-    if (!scatter_march<N>(rays[t >> ls], t & ((1 << ls) - 1), ls, T.cs, qr)) atomicOr(g.err, 1);
+    if (!scatter_march<N, kCopies<N>>(rays[t >> ls], t & ((1 << ls) - 1), ls, T.cs, qr)) atomicOr(g.err, 1);
 }
 
 // ---------------------------------------------------------------- fold
@@ -526,7 +543,9 @@ struct ScatterScratch {
     ScatterTarget T;
     void *block;
     size_t bytes;
-    bool dirty;  // a launch failed between scatter and fold: clear before the next call
+    int form[4];     // per degree (scatter_form)
+    int batches[4];  // per degree (scatter_batches)
+    bool dirty;      // a launch failed between scatter and fold: clear before the next call
 };
 
 // Axes that can be the smallest component of a line of the geometry (a
@@ -545,41 +564,168 @@ static unsigned scatter_axes(const spl_geometry *g, const double *ray_dirs)
     return mask;
 }
 
-spl_status scatter_create(spl_geometry *g, const double *ray_dirs)
+// Whether explicit rays are scattered: of 4096 pairs of neighbours in the
+// caller's order, half or more lie more than a sixteenth of the grid apart
+// (at the points nearest the grid's centre, or by their directions half a
+// grid away from it), so that the rays a GPU works on at a time reach all over
+// the grid.
+static bool scattered_rays(const DevGeom &g, const double *dirs, const double *points)
+{
+    const long long pairs = g.n_rays - 1, step = pairs / 4096 > 1 ? pairs / 4096 : 1;
+    const int n = g.n[0] > g.n[1] ? (g.n[0] > g.n[2] ? g.n[0] : g.n[2]) : (g.n[1] > g.n[2] ? g.n[1] : g.n[2]);
+    long long seen = 0, apart = 0;
+    for (long long r = 0; r < pairs; r += step) {
+        double w[2][3], p[2][3];
+        for (int i = 0; i < 2; ++i) {
+            const double *d = dirs + 3 * (r + i), *s = points + 3 * (r + i);
+            const double l = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+            double t = 0.0;
+            for (int e = 0; e < 3; ++e) {
+                w[i][e] = d[e] / l;
+                p[i][e] = s[e] - (g.org[e] + 0.5 * (g.n[e] - 1));
+                t += p[i][e] * w[i][e];
+            }
+            for (int e = 0; e < 3; ++e) p[i][e] -= t * w[i][e];
+        }
+        // (a line has two directions)
+        const double sg = w[0][0] * w[1][0] + w[0][1] * w[1][1] + w[0][2] * w[1][2] < 0.0 ? -1.0 : 1.0;
+        double dp = 0.0, dw = 0.0;
+        for (int e = 0; e < 3; ++e) {
+            dp += (p[0][e] - p[1][e]) * (p[0][e] - p[1][e]);
+            dw += (w[0][e] - sg * w[1][e]) * (w[0][e] - sg * w[1][e]);
+        }
+        ++seen;
+        apart += sqrt(dp) + 0.5 * n * sqrt(dw) > n / 16.0 ? 1 : 0;
+    }
+    return 2 * apart > seen;
+}
+
+// Form of a degree's reductions: the number of shifted copies, or 0 for single
+// values into one layout.  Rays side by side keep working on one part of the
+// grid, and a row in one reduction (kCopies) is the fewest of them.  Scattered
+// rays reach the whole target all the time, and it has to stay in the L2: the
+// most copies with which the layouts do, and one layout (4 bytes a
+// coefficient, a twelfth of the most) where they do not with two.  300 000
+// random rays, ms with 4 copies, 2 copies, one layout (the L2 holds 135 MB):
+//   cubic      128^3   2.55   2.74     -     115 MB in 4 copies
+//              144^3   5.28   3.16    5.14    81 MB in 2
+//              192^3  12.5    9.38    6.49   183 MB in 2
+//              256^3  22.2   19.6     8.65
+//              400^3  40.9   39.9    30.1
+//   linear     160^3          1.14    1.51   109 MB in 2
+//              192^3          3.28    1.71   183 MB in 2
+//              400^3         15.8     9.13
+// (single values into the three layouts of one copy: cubic 192^3 6.57, 256^3
+// 16.9, 400^3 46.5; four copies of the one layout by ray, cubic 192^3 600 000
+// rays 14.7 against 14.5, linear 3.98 against 3.53).
+static int scatter_form(const DevGeom &g, unsigned mask, bool scattered, int degree)
+{
+    const int most = degree == 0 ? kCopies<0> : (degree == 1 ? kCopies<1> : kCopies<3>);
+    if (!scattered) return most;
+    size_t one = 0;  // bytes of the layouts with one copy
+    for (int b = 0; b < 3; ++b) one += ((mask >> b) & 1u) ? scatter_dims(g.n, b).total * sizeof(float) : 0;
+    for (int cp = most; cp >= (degree == 0 ? 1 : 2); cp /= 2)
+        if (cp * one <= l2_bytes()) return cp;
+    return 0;
+}
+
+// Into how many batches the rays of a call are divided where the form has
+// fewer copies than kCopies.  A running FP32 sum of T terms of random sign
+// rounds T / 2 times the square of one rounding of its size; p partial sums
+// (layouts times copies) round T / (2 p), and `tree` more where they are added
+// up.  With the FP64 total of the batches, (T / p) / (T / p0 + 2 (tree0 -
+// tree)) of them round as much as kCopies copies (p0, tree0).  A^T of random
+// rays, relative error against FP64 with 4 copies, in one batch, and so
+// divided: cubic 192^3, 300 000 rays 1.47e-7, 2.81e-7, 1.46e-7; 60 000 rays
+// 1.29e-7, 1.63e-7, 1.30e-7.
+static double scatter_tree(int copies, int layouts)
+{
+    return (copies >= 4 ? 2.0 : (copies == 2 ? 1.0 : 0.0)) + (layouts == 3 ? 1.7 : (layouts == 2 ? 1.0 : 0.0));
+}
+static int scatter_batches(const DevGeom &g, unsigned mask, int degree, int form)
+{
+    const int most = degree == 0 ? kCopies<0> : (degree == 1 ? kCopies<1> : kCopies<3>);
+    if (form == most) return 1;
+    int layouts = 0;
+    for (int b = 0; b < 3; ++b) layouts += (mask >> b) & 1u;
+    const double n = (g.n[0] + g.n[1] + g.n[2]) / 3.0, nc = (double)g.n[0] * g.n[1] * g.n[2];
+    // a ray crosses about 1.5 n cells with (degree + 1)^2 new bases each
+    const double T = g.n_rays * 1.5 * n * (degree + 1) * (degree + 1) / nc;
+    const double p = form == 0 ? 1 : layouts * form, tree = form == 0 ? 0.0 : scatter_tree(form, layouts);
+    const double k = (T / p) / (T / (layouts * most) + 2.0 * (scatter_tree(most, layouts) - tree));
+    return T > 1.0 && k > 1.0 ? (int)ceil(k) : 1;
+}
+
+spl_status scatter_create(spl_geometry *g, const double *ray_dirs, const double *ray_points)
 {
     const DevGeom &dg = g->dev;
     g->scatter = nullptr;
     if (dg.n_rays == 0 || (dg.kind == SPL_PARALLEL && dg.n_flat == dg.n_views)) return SPL_OK;
     const unsigned mask = scatter_axes(g, ray_dirs);
-    size_t cs = 0, bytes = 0;
-    for (int b = 0; b < 3; ++b) {
-        const size_t t = (size_t)scatter_dims(dg.n, b).total;
-        if (((mask >> b) & 1u) && t > cs) cs = t;
-    }
-    cs = (cs + 63) & ~(size_t)63;
-    for (int b = 0; b < 3; ++b) bytes += ((mask >> b) & 1u) ? 4 * cs * sizeof(float) : 0;
+    const bool scattered = dg.kind == SPL_RAYS && scattered_rays(dg, ray_dirs, ray_points);
     ScatterScratch *S = new (std::nothrow) ScatterScratch();
     if (!S) return fail(SPL_ERR_OOM, "host allocation failed");
-    cudaError_t ce = cudaMalloc(&S->block, bytes);
+    // copies of each layout that some degree takes; the first one also serves form 0
+    const int first = (mask & 1u) ? 0 : ((mask & 2u) ? 1 : 2);
+    int copies = 0;
+    for (int n = 0; n < 4; ++n) {
+        S->form[n] = scatter_form(dg, mask, scattered, n);
+        S->batches[n] = scatter_batches(dg, mask, n, S->form[n]);
+        copies = S->form[n] > copies ? S->form[n] : copies;
+    }
+    size_t cs = 0, floats = 0, off[3];
+    for (int b = 0; b < 3; ++b) {
+        const size_t t = (size_t)scatter_dims(dg.n, b).total;
+        if (((mask >> b) & 1u) && (copies > 0 || b == first) && t > cs) cs = t;
+    }
+    cs = (cs + 63) & ~(size_t)63;
+    for (int b = 0; b < 3; ++b) {
+        off[b] = floats;
+        if ((mask >> b) & 1u) floats += cs * (copies > 0 ? copies : (b == first ? 1 : 0));
+    }
+    S->bytes = floats * sizeof(float);
+    cudaError_t ce = cudaMalloc(&S->block, S->bytes);
     if (ce == cudaSuccess) {
-        ce = cudaMemset(S->block, 0, bytes);
+        ce = cudaMemset(S->block, 0, S->bytes);
         if (ce != cudaSuccess) cudaFree(S->block);
     }
     if (ce != cudaSuccess) {
+        const size_t bytes = S->bytes;
         cudaGetLastError();
         delete S;
         return fail(SPL_ERR_OOM, "cudaMalloc of the adjoint's layout copies (%zu bytes) failed", bytes);
     }
-    S->bytes = bytes;
     S->dirty = false;
     S->T.cs = cs;
-    float *p = (float *)S->block;
-    for (int b = 0; b < 3; ++b) {
-        S->T.lay[b] = ((mask >> b) & 1u) ? p : nullptr;
-        if ((mask >> b) & 1u) p += 4 * cs;
-    }
+    S->T.one = first;
+    for (int b = 0; b < 3; ++b)
+        S->T.lay[b] = ((mask >> b) & 1u) && (copies > 0 || b == first) ? (float *)S->block + off[b] : nullptr;
     g->scatter = S;
     return SPL_OK;
+}
+
+// The layouts that a call of this degree reduces into and folds.
+static ScatterTarget scatter_target(const ScatterScratch &S, int degree)
+{
+    ScatterTarget T = S.T;
+    if (S.form[degree] > 0) T.one = -1;
+    else
+        for (int b = 0; b < 3; ++b) T.lay[b] = b == T.one ? T.lay[b] : nullptr;
+    return T;
+}
+
+long long scatter_batch(const spl_geometry *g, int degree)
+{
+    const long long k = g->scatter->batches[degree];
+    return (g->dev.n_rays + k - 1) / k;
+}
+
+bool scatter_in_batches(const spl_geometry *g)
+{
+    if (!g->scatter) return false;
+    for (int n = 0; n < 4; ++n)
+        if (g->scatter->batches[n] > 1) return true;
+    return false;
 }
 
 void scatter_free(ScatterScratch *S)
@@ -602,12 +748,17 @@ static spl_status scatter_n(const spl_geometry *g, const float *y, long long i0,
         if (!stream_captures(st)) S.dirty = false;
     }
     if (dg.kind == SPL_RAYS) {
-        const int ls = line_split(i1 - i0, ScatterBlocks<N>::value);
-        k_scatter_rays<N><<<(unsigned)((((i1 - i0) << ls) + 127) / 128), 128, 0, st>>>(dg, S.T, y, qr, i0, i1, ls);
+        const int form = S.form[N], ls = line_split(i1 - i0, ScatterBlocks<N>::value);
+        const unsigned blocks = (unsigned)((((i1 - i0) << ls) + 127) / 128);
+        const ScatterTarget T = scatter_target(S, N);
+        auto launch = [&](auto kernel) { kernel<<<blocks, 128, 0, st>>>(dg, T, y, qr, i0, i1, ls); };
+        if (form == 0) launch(k_scatter_rays<N, 0>);
+        else if (N >= 2 && form == 2) launch(k_scatter_rays<N, N >= 2 ? 2 : kCopies<N>>);
+        else launch(k_scatter_rays<N, kCopies<N>>);
     } else {
         const int views = (int)(i1 - i0), ls = line_split((long long)views * dg.nu * dg.nv, ScatterBlocks<N>::value);
         k_scatter_views<N><<<line_grid(dg, views, ls), 128, 0, st>>>(
-            dg, S.T, y, qr, dg.kind == SPL_PARALLEL ? dg.view_order : nullptr, (int)i0, ls);
+            dg, scatter_target(S, N), y, qr, dg.kind == SPL_PARALLEL ? dg.view_order : nullptr, (int)i0, ls);
     }
     const spl_status s = cuda_check(cudaGetLastError(), "adjoint launch");
     if (s != SPL_OK) S.dirty = true;
@@ -630,10 +781,9 @@ spl_status scatter_rays(const spl_geometry *g, int degree, const float *y, long 
 constexpr long long kFoldSmall = 1LL << 18;
 
 template <int CP>
-static void launch_fold(const spl_geometry *g, int base, int fin, float *c, cudaStream_t st)
+static void launch_fold(const spl_geometry *g, const ScatterTarget &T, int base, int fin, float *c, cudaStream_t st)
 {
     const DevGeom &dg = g->dev;
-    const ScatterTarget &T = g->scatter->T;
     const int3 n = make_int3(dg.n[0], dg.n[1], dg.n[2]);
     const long long nc = (long long)n.x * n.y * n.z;
     if (nc <= kFoldSmall) {
@@ -658,9 +808,11 @@ spl_status scatter_fold(const spl_geometry *g, int degree, int src, bool to64, f
 {
     const int base = src == 1 ? FOLD_C : FOLD_ZERO;
     const int fin = to64 ? (src == 2 ? FOLD_ADD_ACC : FOLD_TO_ACC) : (src == 2 ? FOLD_ACC_TO_C : FOLD_TO_C);
-    if (degree == 0) launch_fold<kCopies<0>>(g, base, fin, c, st);
-    else if (degree == 1) launch_fold<kCopies<1>>(g, base, fin, c, st);
-    else launch_fold<kCopies<3>>(g, base, fin, c, st);
+    const ScatterTarget T = scatter_target(*g->scatter, degree);
+    const int form = g->scatter->form[degree];
+    if (form == 4) launch_fold<4>(g, T, base, fin, c, st);
+    else if (form == 2) launch_fold<2>(g, T, base, fin, c, st);
+    else launch_fold<1>(g, T, base, fin, c, st);
     const spl_status s = cuda_check(cudaGetLastError(), "adjoint fold launch");
     if (s != SPL_OK) g->scatter->dirty = true;
     return s;

@@ -87,6 +87,8 @@ spl_status cuda_check(cudaError_t e, const char *what);
 void clear_error();
 // Number of SMs of the current device (queried once per device).
 int sm_count();
+// Bytes of the current device's L2 (queried once per device).
+size_t l2_bytes();
 // Raise a kernel's dynamic shared-memory limit to `bytes` on the current
 // device, once per kernel and device (thread-safe).
 spl_status smem_attr_once(const void *func, int bytes, const char *what);
@@ -161,8 +163,12 @@ spl_status line_forward(const spl_geometry *g, int degree, int kahan, const floa
 // clear between calls; scatter_fold moves their sum out and clears them: to
 // c, or to the FP64 total acc64 (to64), on top of nothing (src 0), what c
 // holds (1) or the FP64 total (2).
-spl_status scatter_create(spl_geometry *g, const double *ray_dirs);
+spl_status scatter_create(spl_geometry *g, const double *ray_dirs, const double *ray_points);
 void scatter_free(ScatterScratch *S);
+// rays of one FP32 sum of an adjoint of explicit rays: all of them, or a part;
+// whether some degree takes a part (the geometry then has the FP64 total)
+long long scatter_batch(const spl_geometry *g, int degree);
+bool scatter_in_batches(const spl_geometry *g);
 spl_status scatter_rays(const spl_geometry *g, int degree, const float *y, long long i0, long long i1, cudaStream_t st);
 spl_status scatter_fold(const spl_geometry *g, int degree, int src, bool to64, float *c, cudaStream_t st);
 

@@ -214,3 +214,43 @@ def test_captured_call_after_a_failed_one(env):
     g.status()
     assert float((out - ref).norm() / ref.norm()) <= TOL
     assert capture() == plain
+
+
+@pytest.mark.parametrize("x_rays", [False, True])
+@pytest.mark.parametrize("dims", [(150, 148, 146), (200, 190, 181), (262, 250, 241)])
+def test_scattered_rays_form_per_target_size(env, orc, dims, x_rays):
+    """Random rays whose target outgrows the L2: fewer shifted copies, then
+    single values into one layout, per degree; and rays near the x direction,
+    for which there is no x-fast layout.  400 rays meet a coefficient once or
+    twice, so the error is the footprints' (about 20 roundings)."""
+    rng = np.random.default_rng(14)
+    w = I.random_directions(rng, 400)
+    if x_rays:
+        w *= (1.0, 0.3, 0.3)
+        w[:, 0] = np.sign(w[:, 0]) * (np.abs(w[:, 0]) + 0.5)
+        w /= np.linalg.norm(w, axis=1, keepdims=True)
+    s = rng.uniform(-0.5, 0.5, size=w.shape) * np.asarray(dims)
+    check(env, orc, I.RayGeometry(w, s), (3, 2, 1, 0), 15, dims)
+
+
+@pytest.mark.parametrize("dims", [(150, 148, 146), (200, 190, 181)])
+def test_scattered_rays_in_batches(env, dims):
+    """More rays, which go in batches through the FP64 total: against the sum
+    over geometries with a part of them each (fewer batches)."""
+    torch, spl = env
+    rng = np.random.default_rng(16)
+    rays = 60001
+    w = I.random_directions(rng, rays)
+    s = rng.uniform(-0.5, 0.5, size=w.shape) * np.asarray(dims)
+    y = torch.randn(rays, device="cuda")
+    for degree in (3, 2, 1):
+        parts = []
+        for sl in (slice(None), slice(0, 20000), slice(20000, 30001), slice(30001, None)):
+            g = spl.Geometry(dims, I.centred_origin(dims), I.RayGeometry(w[sl], s[sl]))
+            c = torch.full(g.coeff_shape, float("nan"), device="cuda")
+            for _ in range(2):
+                spl.adjoint(g, y[sl].contiguous(), c, spl.basis(degree))
+            g.status()
+            parts.append(c.double())
+            g.close()
+        assert float((parts[0] - sum(parts[1:])).norm() / parts[0].norm()) <= TOL
