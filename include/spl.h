@@ -235,7 +235,8 @@ spl_status spl_prepare(spl_geometry *g, const spl_basis_desc *basis, void *strea
  * Rays are marched over the unit cells of their dominant axis (Definition
  * 2.1), cut into the pieces on which every basis is one polynomial.  Degrees
  * 1 to 3 integrate f itself on each piece (Eq. 2) from the coefficients
- * resampled once per call into the power basis of the dominant axis; degree
+ * resampled once per call along the dominant axis (in a basis that keeps
+ * y >= 0 for c >= 0); degree
  * 0, calls captured into a CUDA graph and geometries without the scratch
  * keep an (n+1)^3 window of the bases whose support contains the current
  * point (Algorithm 3's neighbourhood, de-duplicated by construction), and

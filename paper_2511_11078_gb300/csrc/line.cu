@@ -1,20 +1,31 @@
 // line.cu -- forward projection A as line integrals of f itself (Eq. 2), on
-// coefficients resampled once per call into the power basis of the rays'
-// dominant axis.
+// coefficients resampled once per call along the rays' dominant axis.
 //
 // f = sum_k c_k phi(x - k) is, on every cell [c, c+1) of axis d (v = u + W,
-// the cells of the cell march), a polynomial in the position along d for
-// each pair of transverse indices (la, lb):
-//   sum_{l_d} c(l_d, la, lb) beta^n(v_d - W - l_d) = sum_j p_j(c, la, lb) tau^j,
-// tau = v_d - c - 1/2 in [-1/2, 1/2].  k_line_resample writes p_0 .. p_n of
-// every cell and column as one float4 (float2 for n = 1).  A ray is cut into
-// the pieces of the piece march (spl_march.cuh: cells along its dominant
-// axis, split at the knot planes of the other two, r <= 1) and each piece is
-// integrated with the same Gauss-Legendre rule; a node needs two weight sets
-// instead of three and contracts (n+1)^2 columns:
-//   f(tau) = sum_i wa_i sum_k wb_k (p_0 + p_2 tau^2 + tau (p_1 + p_3 tau^2)),
-// the even and the odd part as one packed FP32x2 value (n = 1: the two
-// coefficients with weights 1/2 -+ tau).
+// the cells of the cell march), a polynomial in the position t in [0, 1] along
+// d for each pair of transverse indices (la, lb).  With the cell's coefficients
+// c_0 .. c_n along d and s = 1 - t it is
+//   s (x + z g(s)) + t (y + w g(t)),
+//   cubic:     x = c_1, y = c_2, z = (c_0 - 2 c_1 + c_2) / 6,
+//              w = (c_1 - 2 c_2 + c_3) / 6, g(q) = q^2;
+//   quadratic: x = y = c_1, z = (c_0 - c_1) / 2, w = (c_2 - c_1) / 2, g(q) = q;
+//   linear:    x = c_0, y = c_1, z = w = 0.
+// k_line_resample writes x, y, z, w of every cell and column as one float4
+// (x, y as a float2 for n = 1; no y for n = 2).  A ray is cut into the pieces of the piece march
+// (spl_march.cuh: cells along its dominant axis, split at the knot planes of
+// the other two, r <= 1) and each piece is integrated with the same
+// Gauss-Legendre rule; a node needs two weight sets instead of three and
+// contracts (n+1)^2 columns:
+//   f(t) = (s, t) . sum_i wa_i sum_k wb_k ((x, y) + (g(s), g(t)) (z, w)),
+// the two terms as one packed FP32x2 value.
+//
+// For c >= 0 both terms are >= 0 and as accurate relative to themselves as
+// their coefficients: x + z g >= 2/3 c_1 + (c_0 + c_2) g / 6, and a lone
+// coefficient comes out as its weight, s^3 / 6 at the end of its support.  The
+// transverse weights are >= 0 too (the FMA that computes their argument clamps
+// it to [0, 1]), so A c >= 0.  The powers of t - 1/2, which cost the same,
+// cancel at the ends of a support: an absolute error of 6e-9 of the
+// coefficient there, and negative projections of non-negative coefficients.
 //
 // The footprint form (march in spl_march.cuh) carries an (n+1)^3 register
 // window that an event shifts by selects and flushes face by face; that is
@@ -72,20 +83,28 @@ struct LineArrays {
 };
 
 // ---------------------------------------------------------------- resampling
+// x, y, z, w of a cell's coefficients.  Differences first and halves before
+// their sum: neighbours of any size do not overflow, and a zero neighbour leaves
+// no rounding of the others.  (A division: 1/6 rounded to FP32 would scale
+// every value by 1 + 3e-8.)  A coefficient that is not finite would meet its own
+// negative in z and w: such a cell is the sum of its coefficients.
 template <int N>
-__device__ __forceinline__ typename LineVec<N>::T line_poly(const float (&c)[N + 1])
+__device__ __forceinline__ typename LineVec<N>::T line_cell(const float (&c)[N + 1])
 {
     if constexpr (N == 1) {
-        // the two coefficients themselves: weights 1/2 - tau, 1/2 + tau
         return make_float2(c[0], c[1]);
-    } else if constexpr (N == 2) {
-        return make_float4(0.125f * ((c[0] + c[2]) + 6.0f * c[1]), 0.5f * (c[2] - c[0]),
-                           0.5f * ((c[0] - c[1]) - (c[1] - c[2])), 0.0f);
     } else {
-        const float so = c[0] + c[3], si = c[1] + c[2], dq = c[3] - c[0], di = c[2] - c[1];
-        // (divisions: 1/48 and 1/6 rounded to FP32 would scale every value by 1 + 2e-8, 1 + 3e-8)
-        return make_float4(__fdiv_rn(fmaf(23.0f, si, so), 48.0f), 0.125f * fmaf(5.0f, di, dq), 0.25f * (so - si),
-                           __fdiv_rn(fmaf(-3.0f, di, dq), 6.0f));
+        const float l = 0.5f * (c[0] - c[1]), r = 0.5f * (c[2] - c[1]);
+        float4 v;
+        if constexpr (N == 2)
+            v = make_float4(c[1], 0.0f, l, r);
+        else
+            v = make_float4(c[1], c[2], __fdiv_rn(l + r, 3.0f), __fdiv_rn(0.5f * (c[3] - c[2]) - r, 3.0f));
+        if (!isfinite(v.z) || !isfinite(v.w)) {
+            const float t = N == 2 ? (c[0] + c[1]) + c[2] : (c[0] + c[1]) + (c[2] + c[N]);
+            v = make_float4(t, N == 2 ? 0.0f : t, 0.0f, 0.0f);
+        }
+        return v;
     }
 }
 
@@ -130,7 +149,7 @@ __global__ void __launch_bounds__(256) k_line_resample(DevGeom g, const float *_
 #pragma unroll
         for (int i = 0; i < N; ++i) w[i] = w[i + 1];
         w[N] = in && cc < nd ? __ldg(src + cc * sd) : 0.0f;
-        *o = line_poly<N>(w);
+        *o = line_cell<N>(w);
         o += so;
     }
 }
@@ -252,24 +271,24 @@ __device__ __forceinline__ bool line_march(const LineRay &L, int seg, int ls, co
     }
     int QA, QB;
     float ga, gb, ta, tb, t0;
-    // position in the cell: column (QA, QB) and the fractions at the cell's
-    // middle (tau = 0); ta, tb: tau of the crossings (beyond 1/2: none)
+    // position at the cell's start: column (QA, QB) and the fractions; ta, tb:
+    // the crossings (beyond 1: none)
     auto cell = [&]() {
         constexpr float kUnit = 1.0f / 4294967296.0f;
         QA = (int)(A >> kLineFrac);
         QB = (int)(B >> kLineFrac);
-        ga = fmaf(0.5f, ra, __uint2float_rn((unsigned)(A >> (kLineFrac - 32))) * kUnit);
-        gb = fmaf(0.5f, rb, __uint2float_rn((unsigned)(B >> (kLineFrac - 32))) * kUnit);
+        ga = __uint2float_rn((unsigned)(A >> (kLineFrac - 32))) * kUnit;
+        gb = __uint2float_rn((unsigned)(B >> (kLineFrac - 32))) * kUnit;
         const uint4 e = KEEP ? ke : lds128(&L.ia);
         ta = (__uint_as_float(e.z) - ga) * __uint_as_float(e.x);
         tb = (__uint_as_float(e.w) - gb) * __uint_as_float(e.y);
-        t0 = -0.5f;
+        t0 = 0.0f;
     };
     cell();
     int ev = 0;
 #pragma unroll 1
     while (true) {
-        const float t1 = fminf(fminf(ta, tb), 0.5f);
+        const float t1 = fminf(fminf(ta, tb), 1.0f);
         if (t1 > t0 && (unsigned)QA < lim_p && (unsigned)QB < lim_q) {
             const float half = 0.5f * (t1 - t0), mid = 0.5f * (t0 + t1);
             V col[N + 1][N + 1];
@@ -280,31 +299,24 @@ __device__ __forceinline__ bool line_march(const LineRay &L, int seg, int ls, co
                 for (int k = 0; k <= N; ++k) col[i][k] = __ldg(r + (size_t)i * D.nq + k);
             float2 S = make_float2(0.0f, 0.0f);
             auto node = [&](float x, float wt) {
-                const float tau = fmaf(half, x, mid);
+                const float t = fmaf(half, x, mid);
+                const float2 st = make_float2(1.0f - t, t), gg = N == 3 ? __fmul2_rn(st, st) : st;
                 float wa[N + 1], wb[N + 1];
-                bweights<N>(fmaf(ra, tau, ga), wa);
-                bweights<N>(fmaf(rb, tau, gb), wb);
-                const float2 t2 = dup(tau * tau);
+                bweights<N>(__saturatef(fmaf(ra, t, ga)), wa);
+                bweights<N>(__saturatef(fmaf(rb, t, gb)), wb);
                 float2 h = make_float2(0.0f, 0.0f);
 #pragma unroll
                 for (int i = 0; i <= N; ++i) {
                     float2 gk;
 #pragma unroll
                     for (int k = 0; k <= N; ++k) {
-                        float2 e;
-                        if constexpr (N == 3)
-                            e = __ffma2_rn(make_float2(col[i][k].z, col[i][k].w), t2,
-                                           make_float2(col[i][k].x, col[i][k].y));
-                        else if constexpr (N == 2)
-                            e = make_float2(fmaf(col[i][k].z, t2.x, col[i][k].x), col[i][k].y);
-                        else
-                            e = make_float2(col[i][k].x, col[i][k].y);
+                        float2 e = N == 2 ? dup(col[i][k].x) : make_float2(col[i][k].x, col[i][k].y);
+                        if constexpr (N > 1) e = __ffma2_rn(make_float2(col[i][k].z, col[i][k].w), gg, e);
                         gk = k == 0 ? __fmul2_rn(dup(wb[0]), e) : __ffma2_rn(dup(wb[k]), e, gk);
                     }
                     h = i == 0 ? __fmul2_rn(dup(wa[0]), gk) : __ffma2_rn(dup(wa[i]), gk, h);
                 }
-                if constexpr (N == 1) S = __ffma2_rn(make_float2(wt * (0.5f - tau), wt * (0.5f + tau)), h, S);
-                else S = __ffma2_rn(make_float2(wt, wt * tau), h, S);
+                S = __ffma2_rn(__fmul2_rn(dup(wt), st), h, S);
             };
             if constexpr (N == 3) {
                 // four nodes where they are exact to FP32 (line_short) for
@@ -327,7 +339,7 @@ __device__ __forceinline__ bool line_march(const LineRay &L, int seg, int ls, co
         }
         t0 = fmaxf(t0, t1);
         if (++ev > qr.cap) return false;
-        const bool evA = ta <= tb && ta < 0.5f, evB = !evA && tb < 0.5f;
+        const bool evA = ta <= tb && ta < 1.0f, evB = !evA && tb < 1.0f;
         if (evA || evB) {
             // the column's neighbour along the crossed axis, once per cell
             const int step = (evA ? ra : rb) > 0.0f ? 1 : -1;
@@ -373,6 +385,7 @@ __device__ __forceinline__ float line_value(const DevGeom &g, const LineRay &L, 
         hi = s;
     }
     const float p = __fmul_rn(hi, L.scale);
+    if (!isfinite(p)) return p;  // (its corrections would be inf - inf)
     return p + fmaf(hi, L.scale_lo, fmaf(lo, L.scale, fmaf(hi, L.scale, -p)));
 }
 

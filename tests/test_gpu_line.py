@@ -208,3 +208,73 @@ def test_streams_take_turns_on_the_plane_path(env, mixed, threads):
     for i in range(2):
         for y in got[i]:
             assert torch.equal(y, ref[i])
+
+
+def project(env, dims, geo, c, degree, kahan=True):
+    torch, spl = env
+    g = spl.Geometry(dims, I.centred_origin(dims), geo)
+    y = torch.empty(g.n_rays, device="cuda")
+    spl.forward(g, torch.tensor(c, device="cuda"), y, spl.basis(degree, kahan=kahan))
+    g.status()
+    return y.cpu().numpy()
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+@pytest.mark.parametrize("d,a", [(0, 1), (1, 2), (2, 0), (2, 1)])
+def test_support_corner_is_accurate_by_itself(env, orc, degree, d, a):
+    """One coefficient and rays that clip the corner of its support within
+    t = 1e-3 .. 0.3 cells, where two weights are t^n and (ra (tau - t))^n: the
+    projection is positive, and accurate relative to itself.  Allowed: the
+    clipped argument's rounding at the outermost node (0.047 of the piece),
+    n 2^-25 / 0.047, the 2^-32 of the position, n 2^-32 / (ra t) = 5e-7, and 20
+    roundings of 2^-24: below 6e-6."""
+    rng = np.random.default_rng(20)
+    dims, W = (9, 9, 9), 0.5 * (degree + 1)
+    b = 3 - d - a
+    ra, tau = 0.7, 10.0 ** rng.uniform(-3.0, -0.5, 2000)
+    w, s = np.zeros((2000, 3)), np.zeros((2000, 3))
+    w[:, d], w[:, a], w[:, b] = 1.0, -ra, 0.02
+    # at the low d face of the support, ra tau inside its low a face
+    s[:, d], s[:, a], s[:, b] = -W, -W + ra * tau, rng.uniform(-0.4, 0.4, 2000)
+    s += 3.0 * w  # elsewhere on the line
+    geo = I.RayGeometry(w / np.linalg.norm(w, axis=1, keepdims=True), s)
+    c = np.zeros(dims, dtype=np.float32)
+    c[4, 4, 4] = 1.0
+    y = project(env, dims, geo, c, degree)
+    ref = orc.forward(degree, dims, I.centred_origin(dims), c.astype(np.float64), geom_of(orc, geo)).reshape(-1)
+    assert np.all(ref > 0.0)
+    assert np.all(y > 0.0)
+    assert np.max(np.abs(y - ref) / ref) <= 6e-6
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+def test_nonnegative_coefficients_project_nonnegative(env, degree):
+    """c >= 0 with many zeros: no ray comes out below zero."""
+    rng = np.random.default_rng(21)
+    dims = (13, 12, 11)
+    c = rng.uniform(0.0, 1.0, dims[::-1]) * (rng.uniform(size=dims[::-1]) < 0.02)
+    w = I.random_directions(rng, 200000)
+    s = rng.uniform(-0.75, 0.75, size=w.shape) * np.asarray(dims)
+    y = project(env, dims, I.RayGeometry(w, s), c.astype(np.float32), degree)
+    assert np.all(y >= 0.0) and np.any(y > 0.0)
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+def test_large_and_infinite_coefficients(env, orc, degree):
+    """Neighbours of 2e37 (a ray's integral stays below the largest float) and
+    one infinite coefficient (in plain sums: a compensation of an infinite sum is
+    NaN by itself)."""
+    rng = np.random.default_rng(22)
+    dims = (9, 9, 9)
+    w = I.random_directions(rng, 2000)
+    s = rng.uniform(-0.5, 0.5, size=w.shape) * 9.0
+    geo = I.RayGeometry(w, s)
+    c = rng.uniform(0.9, 1.0, dims).astype(np.float32)
+    one, big = project(env, dims, geo, c, degree), project(env, dims, geo, c * np.float32(2.0 ** 124), degree)
+    assert np.array_equal(big, one * np.float32(2.0 ** 124))
+    hot = np.zeros(dims, dtype=np.float32)
+    hot[4, 4, 4] = 1.0
+    ref = orc.forward(degree, dims, I.centred_origin(dims), hot.astype(np.float64), geom_of(orc, geo)).reshape(-1)
+    c[4, 4, 4] = np.inf
+    y = project(env, dims, geo, c, degree, kahan=False)
+    assert np.all(np.isposinf(y[ref > 1e-3])) and np.all(np.isfinite(y[ref == 0.0]))
