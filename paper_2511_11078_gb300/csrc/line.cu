@@ -165,7 +165,7 @@ struct __align__(16) LineRay {
     float ra, rb;             // steps per cell
     float scale, scale_lo;    // 1 / |w_d| as a sum of two floats
     int d, c, cl;             // dominant axis, first and last cell (none: c > cl)
-    float h4;                 // longest piece that four Gauss nodes integrate (cubic, line_short)
+    int four;                 // cubic: every piece takes four Gauss nodes (line_four)
 };
 
 // The line {s + t w} (w of any length).  The two orientations of a line are
@@ -202,7 +202,7 @@ __device__ __forceinline__ void line_setup(const DevGeom &g, const double (&s)[3
     const double a0 = fma(-(W + sd), ra, sp) + W, b0 = fma(-(W + sd), rb, sq) + W;
     L.ra = (float)ra;
     L.rb = (float)rb;
-    if (N == 3) L.h4 = line_short(L.ra, L.rb);
+    if (N == 3) L.four = line_four(L.ra, L.rb);
     // an axis that the ray does not move along: crossing at 3 - fraction, never inside a cell
     L.ia = ra != 0.0 ? 1.0f / L.ra : 1.0f;
     L.ib = rb != 0.0 ? 1.0f / L.rb : 1.0f;
@@ -253,6 +253,7 @@ __device__ __forceinline__ bool line_march(const LineRay &L, int seg, int ls, co
     sum = comp = 0.0f;
     const int cells = L.cl - L.c + 1, k0 = (int)(((long long)cells * seg) >> ls),
               k1 = (int)(((long long)cells * (seg + 1)) >> ls);
+    const bool four = N == 3 && __all_sync(0xffffffffu, k0 >= k1 || L.four);
     if (k0 >= k1) return true;
     const int d = L.d;
     long long A = L.A + L.RA * k0, B = L.B + L.RB * k0;
@@ -321,15 +322,12 @@ __device__ __forceinline__ bool line_march(const LineRay &L, int seg, int ls, co
                 S = fmaf(wt, fmaf(st.x, h.x, st.y * h.y), S);
             };
             if constexpr (N == 3) {
-                // four nodes where they are exact to FP32 (line_short) for
-                // every lane that is here, five otherwise
-                const bool five = t1 - t0 > __uint_as_float(lds128(&L.d).w);
-                if (__any_sync(__activemask(), five)) {
-#pragma unroll
-                    for (int q = 0; q < M; ++q) node(qr.x[q], qr.w[q]);
-                } else {
+                if (four) {
 #pragma unroll
                     for (int q = 0; q < M - 1; ++q) node(qr.x1[q], qr.w1[q]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < M; ++q) node(qr.x[q], qr.w[q]);
                 }
             } else {
 #pragma unroll

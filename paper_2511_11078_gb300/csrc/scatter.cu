@@ -73,7 +73,8 @@ struct __align__(16) ScatterRay {
     long long RA, RB;  // and their steps, >= 0
     float ia, ib;      // reciprocals of ra, rb
     float ra, rb;      // steps per cell, 0 <= rb <= ra <= 1
-    float yv, h4;      // y / |w_d|; longest piece of four Gauss nodes (line_short)
+    float yv;          // y / |w_d|
+    int four;          // cubic: every piece takes four Gauss nodes (line_four)
     int lim_a, lim_b;  // the window meets the grid while 0 <= Q < lim
     int c, cl;         // first and last cell (none: c > cl)
     int sd, sa;        // signed strides of d and a in the target
@@ -123,7 +124,7 @@ __device__ __forceinline__ void scatter_setup(const DevGeom &g, const ScatterTar
     R.rb = (float)rb;
     R.ia = ra > 0.0 ? 1.0f / R.ra : 1.0f;
     R.ib = rb > 0.0 ? 1.0f / R.rb : 1.0f;
-    if (N == 3) R.h4 = line_short(R.ra, R.rb);
+    if (N == 3) R.four = line_four(R.ra, R.rb);
     const double a0 = fma(-(W + ud), ra, ua) + W, b0 = fma(-(W + ud), rb, ub) + W;
     float vmin = 0.0f, vmax = (float)(nd + N);
     if (ra > 0.0) {
@@ -212,6 +213,7 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
     const int sb = CP > 0 ? 1 : R.sb;
     const int cells = R.cl - R.c + 1, k0 = (int)(((long long)cells * seg) >> ls),
               k1 = (int)(((long long)cells * (seg + 1)) >> ls);
+    const bool four = N == 3 && __all_sync(0xffffffffu, k0 >= k1 || R.four);
     if (k0 >= k1) return true;
     int left = k1 - k0;
     long long A = R.A + R.RA * k0, B = R.B + R.RB * k0;
@@ -267,12 +269,12 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
                 window_update<N>(acc, wd, wa, wb, hs * wt);
             };
             if constexpr (N == 3) {
-                if (__any_sync(__activemask(), t1 - t0 > __uint_as_float(yl.y))) {
-#pragma unroll
-                    for (int q = 0; q < M; ++q) node(qr.x[q], qr.w[q]);
-                } else {
+                if (four) {
 #pragma unroll
                     for (int q = 0; q < M - 1; ++q) node(qr.x1[q], qr.w1[q]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < M; ++q) node(qr.x[q], qr.w[q]);
                 }
             } else {
 #pragma unroll

@@ -26,25 +26,32 @@ constexpr int kLineFrac = 40;
 // scale takes it out (it was most of the forward's error against FP64).
 template <int N> __device__ __forceinline__ constexpr float weight_excess(int axes) { return N == 3 ? 4.22e-8f * axes : 0.0f; }
 
-// The longest piece (in cells) of a cubic ray that the 4-node Gauss rule
-// integrates to FP32 accuracy.  The 4-node rule is exact to degree 7; of the
-// degree-9 product of a piece of length h it misses only the coefficient C8
-// of the 8th power about the piece's middle (the 9th is odd there), by
+// Whether every piece of a cubic ray takes the 4-node Gauss rule.  It is exact
+// to degree 7; of the degree-9 product of a piece of length h <= 1 it misses
+// only the coefficient C8 of the 8th power about the piece's middle (the 9th is
+// odd there), by
 //   e8 (h/2)^9 C8,  e8 = 2^9 (4!)^4 / (9 (8!)^2) = 0.01161,
 // and C8 = D2 A3 B3 + D3 A2 B3 + D3 A3 B2 with |D3| <= 1/2, |A3| <= ra^3 / 2,
 // |B3| <= rb^3 / 2 the third- and |D2| <= 1, |A2| <= ra^2, |B2| <= rb^2 the
-// second-order coefficients of the three weights, so a footprint's error is at
-// most 5.67e-6 h^9 (ra rb + ra + rb) ra^2 rb^2.  The rule is taken where that
-// is below 2^-28, an eighth of an ulp of the footprint's peak (0.44): the
-// difference drowns in the FP32 rounding of the sums.  Rays with a small
-// component (most of a cone's) qualify at every length; a warp takes the
-// 5-node rule when one of its lanes has to.
-__device__ __forceinline__ float line_short(float ra, float rb)
+// second-order coefficients of the three weights, so a piece misses at most
+// 5.67e-6 h^9 (ra rb + ra + rb) ra^2 rb^2 of a footprint.  The rule is taken
+// where that is below 2^-28 at h = 1, an eighth of an ulp of the footprint's
+// peak (0.44) for each of its pieces (up to a dozen, most of them far shorter):
+// the difference drowns in the FP32 rounding of the sums (A^T of a 128^3 cone
+// against FP64: 1.359e-7 with the rule, 1.373e-7 with five nodes for all).  It
+// is an absolute bound: where a ray clips the corner of a support, a footprint
+// of 1e-8 of the peak can miss 1e-4 of itself.
+// A warp takes it when all its rays do, decided once where the warp is whole,
+// so a ray's value depends on the rays that share its warp and on nothing else;
+// half of the warps of a cone or helical orbit do.  Five nodes for all: 8
+// helical views A 44.4 -> 50.9 ms, A^T 54.9 -> 60.3, 8 cone views 6.16 -> 6.45 and
+// 7.35 -> 7.68.  A rule for each piece and lane (selected nodes, the fifth in a
+// branch): 44.5, 55.9, 6.15, 7.50.
+__device__ __forceinline__ bool line_four(float ra, float rb)
 {
     ra = fabsf(ra);
     rb = fabsf(rb);
-    const float c = 5.67e-6f * 0x1p28f * (fmaf(ra, rb, ra) + rb) * (ra * ra) * (rb * rb);
-    return exp2f(-0.11111111f * log2f(c));
+    return 5.67e-6f * 0x1p28f * (fmaf(ra, rb, ra) + rb) * (ra * ra) * (rb * rb) <= 1.0f;
 }
 
 // 16 bytes of a ray, not to be kept in registers: next to 64 column values

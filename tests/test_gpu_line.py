@@ -278,3 +278,21 @@ def test_large_and_infinite_coefficients(env, orc, degree):
     c[4, 4, 4] = np.inf
     y = project(env, dims, geo, c, degree, kahan=False)
     assert np.all(np.isposinf(y[ref > 1e-3])) and np.all(np.isfinite(y[ref == 0.0]))
+
+
+def test_warp_mates_in_any_order(env):
+    """The Gauss rule of a cubic ray depends on which rays share its warp and on
+    nothing else: rays put in another order within each group of 32 keep their
+    values bit for bit."""
+    torch, spl = env
+    rng = np.random.default_rng(23)
+    rays = 90016  # one thread a ray
+    w = I.random_directions(rng, rays)
+    w[::3] = np.array([1.0, 0.3, 0.01]) * rng.uniform(0.5, 1.0, size=(len(w[::3]), 1)) + 0.02 * w[::3]
+    w[rays // 2:] = w[0] + 0.01 * w[rays // 2:]  # whole groups that take four nodes
+    w /= np.linalg.norm(w, axis=1, keepdims=True)
+    s = rng.uniform(-1.15, 1.15, size=(rays, 3)) * 0.5 * (np.asarray(DIMS) - 1.0)
+    perm = np.concatenate([32 * k + rng.permutation(32) for k in range(rays // 32)])
+    c = rng.normal(size=DIMS[::-1]).astype(np.float32)
+    y = project(env, DIMS, I.RayGeometry(w, s), c, 3)
+    assert np.array_equal(y[perm], project(env, DIMS, I.RayGeometry(w[perm], s[perm]), c, 3))
