@@ -14,10 +14,12 @@ template <class T> __host__ __device__ inline T sel3(int i, const T &a, const T 
 }
 
 // Transverse coordinates are carried as 64-bit fixed point with kLineFrac
-// fraction bits: the start is exact to 2^-41 and the step is off by at most
-// 2^-41 per cell, 2^-30 over the longest ray, so a cell's fraction is its
-// FP32 rounding everywhere on the ray, for one 64-bit add per cell.
-constexpr int kLineFrac = 40;
+// fraction bits (and 15 bits and a sign for cells: the grid has at most 2048,
+// and a ray is marched where it meets it).  The start is the FP64 value, exact
+// to 2^-43, and the step is off by at most 2^-49 per cell, 2^-38 over the
+// longest ray; a cell takes its fraction's upper 32 bits.  One 64-bit add per
+// cell.
+constexpr int kLineFrac = 48;
 
 // The FP32 constants 2/3 and 1/6 of the cubic weights (bweights<3>) are
 // 1.987e-8 and 4.97e-9 too large, so the four weights of an axis sum to

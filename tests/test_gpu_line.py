@@ -296,3 +296,28 @@ def test_warp_mates_in_any_order(env):
     c = rng.normal(size=DIMS[::-1]).astype(np.float32)
     y = project(env, DIMS, I.RayGeometry(w, s), c, 3)
     assert np.array_equal(y[perm], project(env, DIMS, I.RayGeometry(w[perm], s[perm]), c, 3))
+
+
+def test_position_at_the_end_of_a_long_ray(env, orc):
+    """Rays along 2040 cells whose step is no multiple of 2^-40 (2^-48 exactly),
+    to a coefficient whose support they enter g = 1e-4 .. 2e-4 inside one face and
+    leave through it: the projection goes with g^7, so a drift of half a
+    2^-40 per cell, 9e-10, would show as 3e-5 to 6e-5.  Allowed: the 2^-32 to
+    which a cell takes its fraction, 7 * 2^-32 / g = 1.6e-5, and 6e-6 as for the
+    other clipped corners."""
+    rng = np.random.default_rng(24)
+    dims, k = (2048, 9, 9), 2040
+    ra = (np.floor(0.003 * 2.0 ** 40) + 126.0 / 256.0) / 2.0 ** 40
+    g = rng.uniform(1e-4, 2e-4, 500)
+    x0 = -0.5 * (dims[0] - 1)  # the grid's first coefficient
+    w = np.tile([1.0, -ra, 0.0003], (500, 1))
+    s = np.zeros((500, 3))
+    # the low face of the support along x is at k - 2; there y is g above the low face
+    s[:, 0], s[:, 1], s[:, 2] = x0, -2.0 + g + ra * (k - 2), rng.uniform(-0.9, -0.7, 500)
+    geo = I.RayGeometry(w / np.linalg.norm(w, axis=1, keepdims=True), s)
+    c = np.zeros(dims[::-1], dtype=np.float32)
+    c[4, 4, k] = 1.0
+    ref = orc.forward(3, dims, I.centred_origin(dims), c.astype(np.float64), geom_of(orc, geo)).reshape(-1)
+    assert np.all(ref > 0.0)
+    y = project(env, dims, geo, c, 3)
+    assert np.max(np.abs(y - ref) / ref) <= 2.2e-5
