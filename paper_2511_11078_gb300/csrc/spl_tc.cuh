@@ -348,7 +348,10 @@ __device__ __forceinline__ void tc_cols(uint32_t tmem, float (&z)[32])
 // a reciprocal per value was two thirds of its work (a quarter of them by
 // Newton steps on the FMA pipe); now it is a fifth.  Each reciprocal carries
 // four more roundings of 2^-24 than rcp(d) itself, far below the BF16 rounding
-// that follows.  Values below -87 can take the product out of range (`over`
+// that follows in the hidden layers; the output layer, which is FP32, keeps a
+// reciprocal for each value (silu2; a view of the 256^3 cone 32.3 -> 33.4 ms,
+// A^T 32.0 -> 32.6; the shared one with a residual step 33.9 and 33.3).  Values
+// below -87 can take the product out of range (`over`
 // collects the largest; the caller then repeats its values with silu_safe).
 __device__ __forceinline__ void silu4(const float (&z)[4], float (&h)[4], float &over)
 {
@@ -408,7 +411,7 @@ __device__ __forceinline__ void tc_silu_store(TcTile &T, int m, int c0, const fl
         }
     }
     if (over > kSiluOver) {
-        // a value far below zero (not met in practice): again, one by one
+        // some value far below zero: again, one by one
 #pragma unroll 1
         for (int c = 0; c < 32; ++c) {
             float v = z[0];
@@ -435,32 +438,16 @@ template <bool SAVE>
 __device__ __forceinline__ float tc_output(const TcMlpImage &img, int c0, const float (&z)[32], bool save, float *zb, float *hb)
 {
     float2 acc = make_float2(0.0f, 0.0f);
-    float over = 0.0f;
 #pragma unroll
     for (int k = 0; k < 32; k += 4) {
         if (SAVE && save) *reinterpret_cast<float4 *>(zb + c0 + k) = make_float4(z[k], z[k + 1], z[k + 2], z[k + 3]);
-        const float zz[4] = {z[k], z[k + 1], z[k + 2], z[k + 3]};
-        float h[4];
-        silu4(zz, h, over);
-        if (SAVE && save) *reinterpret_cast<float4 *>(hb + c0 + k) = make_float4(h[0], h[1], h[2], h[3]);
+        const float2 h0 = silu2(make_float2(z[k], z[k + 1])), h1 = silu2(make_float2(z[k + 2], z[k + 3]));
+        if (SAVE && save) *reinterpret_cast<float4 *>(hb + c0 + k) = make_float4(h0.x, h0.y, h1.x, h1.y);
         const float4 w = *reinterpret_cast<const float4 *>(img.w4 + c0 + k);
-        acc = __ffma2_rn(make_float2(h[0], h[1]), make_float2(w.x, w.y), acc);
-        acc = __ffma2_rn(make_float2(h[2], h[3]), make_float2(w.z, w.w), acc);
+        acc = __ffma2_rn(h0, make_float2(w.x, w.y), acc);
+        acc = __ffma2_rn(h1, make_float2(w.z, w.w), acc);
     }
-    float o = acc.x + acc.y;
-    if (over > kSiluOver) {  // as in tc_silu_store
-        o = 0.0f;
-#pragma unroll 1
-        for (int c = 0; c < 32; ++c) {
-            float v = z[0];
-#pragma unroll
-            for (int e = 1; e < 32; ++e) v = e == c ? z[e] : v;
-            const float h = silu_safe(v);
-            o = fmaf(h, img.w4[c0 + c], o);
-            if (SAVE && save) hb[c0 + c] = h;
-        }
-    }
-    return o;
+    return acc.x + acc.y;
 }
 
 // f_theta of this thread's row x (5 features) in a tile of 128 rows; every

@@ -514,3 +514,33 @@ def test_mlp_projector_far_negative_in_some_rows(env, orc, adjoint):
     ref = orc.forward_mlp(3, dims, origin, c.astype(np.float64), og, SIZES, prm.astype(np.float64), mode=1)
     got = y.cpu().numpy().astype(np.float64)
     assert np.linalg.norm(got - ref) <= 2e-3 * np.linalg.norm(ref)
+
+
+def test_output_layer_silu_is_fp32(env):
+    """The third layer's activations enter the output layer and the weight
+    gradient in FP32.  W3 = W4 = 0, b3 = z and the target -1/2 make dL/dW4 the
+    activations themselves.  For z in [3, 8] (12 fraction bits: exact in the
+    bias's BF16 split) they carry three roundings: of 1 + e^-z, uniform within
+    2^-24, of its reciprocal, within 2^-24, and of the product, uniform within
+    2^-24 of a mantissa in 1 .. 2: an rms error of at most
+    sqrt(0.58^2 + 0.58^2 + 0.41^2) = 0.91 * 2^-24."""
+    torch, spl, learn = env
+    rng = np.random.default_rng(5900)
+    m = spl.Mlp(3, max_batch=64, seed=8)
+    X = torch.tensor(random_features(rng, 1), device="cuda")
+    Y = torch.full((1,), -0.5, device="cuda")
+    grad, loss = torch.empty(spl.MLP_PARAMS, device="cuda"), torch.empty(1, device="cuda")
+    err = []
+    for _ in range(40):
+        prm = random_params(rng)
+        z = np.round(rng.uniform(3.0, 8.0, 64) * 4096.0) / 4096.0
+        prm[4544:8640] = 0.0
+        prm[8640:8704] = z
+        prm[8704:] = 0.0
+        m.set_params(prm)
+        m.grad(X, Y, grad, loss)
+        h = grad[8704:8768].cpu().numpy().astype(np.float64)
+        ref = z / (1.0 + np.exp(-z))
+        err.append((h - ref) / ref)
+    m.status()
+    assert np.sqrt(np.mean(np.square(err))) <= 0.95 * 2.0 ** -24
