@@ -167,13 +167,8 @@ typedef struct {
  * flat class; explicit rays whose neighbours in the caller's order lie far
  * apart take fewer copies, or one layout in single values, where four copies
  * outgrow the L2) and, for more than 48 views, 2^22 explicit rays or such
- * rays in several batches, an FP64 accumulator (8 nx ny nz bytes).  Scratch of
- * the forward, for geometries
- * with rays outside the flat class: the coefficients resampled along each
- * axis that is the dominant one of some ray, 16 bytes per coefficient and
- * axis on a grid padded by 3 (left out where few rays cross a large grid,
- * where explicit rays would need more than 320 MB, above 24 GB, and when it
- * cannot be allocated: spl_forward then takes the form without scratch).
+ * rays in several batches, an FP64 accumulator (8 nx ny nz bytes).  The forward's
+ * scratch is allocated by spl_prepare.
  * Uses the current CUDA device.
  * Errors: SPL_ERR_ARG, SPL_ERR_NONFINITE, SPL_ERR_UNSUPPORTED, SPL_ERR_OOM,
  * SPL_ERR_CUDA; *out is NULL on error. */
@@ -218,8 +213,16 @@ spl_status spl_geometry_status(const spl_geometry *g, void *stream);
  * One-time device allocation and kernels on `stream`, then a
  * synchronisation; later calls for the same degree return at once.  Until
  * it has run, spl_forward / spl_adjoint refuse such a basis with
- * SPL_ERR_STATE.  Geometries without separable views,
- * basis->separable == SPL_SEP_OFF and the MLP footprint need nothing.  The
+ * SPL_ERR_STATE.  It also allocates the scratch of spl_forward (exact
+ * footprint, degrees 1 to 3, geometries with rays outside the flat class): the
+ * coefficients resampled along each axis that is the dominant one of some ray,
+ * 16 bytes per coefficient and axis (8 for degree 1) on a grid padded by the
+ * degree, one block for the largest degree asked for.  It is left out where
+ * few rays cross a large grid, where explicit rays far apart would read it from
+ * beyond the L2, above 24 GB or a quarter of the free memory, when it cannot be
+ * allocated, and on a stream that captures; without it, also before
+ * spl_prepare, spl_forward takes the form without scratch.  The adjoint,
+ * the MLP footprint and degree 0 have no use for it.  The
  * plane buffers include the scratch of S and of its adjoint; which calls on
  * one geometry may overlap is said at spl_forward.
  * Errors: SPL_ERR_ARG; SPL_ERR_OOM (plane matrices: the path stays off for

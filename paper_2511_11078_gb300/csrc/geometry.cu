@@ -540,10 +540,10 @@ extern "C" spl_status spl_make_geometry(const spl_geometry_desc *desc, spl_geome
             return fail(SPL_ERR_OOM, "cudaMalloc of the adjoint accumulator (%lld doubles) failed", nk);
         }
     }
-    line_create(g, d.ray_omega);
+    spl_status sync = line_create(g, d.ray_omega);
     // The uploads and clears above went to the default stream; a first call on
     // a stream that does not synchronise with it would run beside them.
-    spl_status sync = cuda_check(cudaStreamSynchronize(0), "geometry upload");
+    if (sync == SPL_OK) sync = cuda_check(cudaStreamSynchronize(0), "geometry upload");
     if (sync == SPL_OK && (g->line || g->plane)) sync = turn_create(g);
     if (sync != SPL_OK) {
         spl_destroy_geometry(g);

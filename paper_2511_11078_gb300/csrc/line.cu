@@ -456,27 +456,34 @@ __global__ void __launch_bounds__(128, LineBlocks<N>::value)
 }
 
 // ---------------------------------------------------------------- host side
-// The resampled arrays of a geometry; forwards take turns on them
-// (ForwardTurn).
+// The resampled arrays of a geometry, one block for the largest degree that
+// spl_prepare has been asked for; forwards take turns on it (ForwardTurn).
 struct LineScratch {
-    LineArrays arr;
+    unsigned mask;   // axes that can be the dominant one of a ray
+    size_t need[4];  // bytes of a degree's arrays, 0 where it keeps the footprint form
     void *block;
+    size_t bytes;
 };
 
 // Where the resampled form is the faster one (both sides measured on GB300):
 //  * the arrays are written once per call, 4.7e-12 s a vector, and a piece of
 //    a view's ray costs 2.9e-11 s in the footprint form and 1.9e-11 s here:
 //    it pays from half a piece per vector on, and a ray crosses about half of
-//    nx + ny + nz cells (20 000 rays through 256^3: 1.46 against 1.22 ms, two
-//    views of 395 x 263 through 293 x 335 x 320: 2.47 against 3.07);
-//  * explicit rays need not lie side by side, and then every lane loads its
-//    own 32-byte sectors: the arrays have to stay mostly in the L2 (300 000
-//    random rays, cubic, 192^3 = 365 MB: 4.6 against 6.0 ms; 256^3 = 850 MB:
-//    12.6 against 7.6; quadratic 192^3: 2.97 against 2.94);
-//  * all three axes of a 512^3 grid take 6.7 GB; beyond 24 GB the scratch is
-//    out of proportion.
+//    nx + ny + nz cells (400^3, rays times nx + ny + nz per vector, footprint form
+//    and this one: cubic 0.54 1.21 and 1.41 ms, 0.95 1.77 and 1.70, 1.9 2.82 and
+//    2.26; linear 0.97 0.53 and 0.66, 1.9 0.79 and 0.80, 3.8 1.44 and 1.18);
+//  * explicit rays that do not lie side by side (spl_geometry::scattered): every
+//    lane loads its own 32-byte sectors, and the arrays have to stay mostly in
+//    the L2 (135 MB).  300 000 and 600 000 random rays, gain over the footprint
+//    form: cubic 176^3 (292 MB) 1.35 1.36, 192^3 (376 MB) 1.23 1.19, 208^3
+//    (475 MB) 0.94 0.84; quadratic 144^3 (161 MB) 1.06 1.07, 160^3 (218 MB) 1.00
+//    1.00, 176^3 (288 MB) 0.93 0.93; linear 208^3 (231 MB) 1.19 1.04, 224^3
+//    (287 MB) 1.11 0.95, 256^3 (425 MB) 0.96 0.81.  Rays side by side gain 1.1 to
+//    2.2 up to 384^3 (2.9 GB), like those of views;
+//  * all three axes of a cubic 512^3 grid take 6.7 GB; beyond 24 GB, or a quarter
+//    of the memory that is free, the scratch is out of proportion.
 constexpr size_t kLineMaxBytes = (size_t)24 << 30;
-constexpr size_t kLineMaxBytesRays = (size_t)320 << 20;
+constexpr double kLineScatteredL2[4] = {0.0, 1.75, 1.5, 3.0};  // most bytes in L2s, per degree
 
 // Axes that can be the dominant one of a line of the geometry (a superset).
 static unsigned line_axes(const spl_geometry *g, const double *ray_dirs)
@@ -493,33 +500,42 @@ static unsigned line_axes(const spl_geometry *g, const double *ray_dirs)
     return mask;
 }
 
-void line_create(spl_geometry *g, const double *ray_dirs)
+// Byte offsets of the axes' arrays; returns their end.
+static size_t line_offsets(const DevGeom &g, unsigned mask, int degree, size_t (&off)[3])
+{
+    size_t end = 0;
+    for (int d = 0; d < 3; ++d) {
+        off[d] = end;
+        if (!((mask >> d) & 1u)) continue;
+        const LineDims L = line_dims(g.n, d, degree);
+        const size_t vec = degree == 1 ? sizeof(float2) : sizeof(float4);
+        end += ((size_t)L.nd * L.np * L.nq * vec + 255) & ~(size_t)255;
+    }
+    return end;
+}
+
+spl_status line_create(spl_geometry *g, const double *ray_dirs)
 {
     const DevGeom &dg = g->dev;
     g->line = nullptr;
     // parallel views of the flat class take the plane matrices or the flat march
-    if (dg.n_rays == 0 || (dg.kind == SPL_PARALLEL && dg.n_flat == dg.n_views)) return;
-    const unsigned mask = line_axes(g, ray_dirs);
-    size_t off[3], total = 0;
-    for (int d = 0; d < 3; ++d) {
-        off[d] = total;
-        if (!((mask >> d) & 1u)) continue;
-        // sized for cubic splines, the largest
-        const LineDims L = line_dims(dg.n, d, 3);
-        total += ((size_t)L.nd * L.np * L.nq * sizeof(float4) + 255) & ~(size_t)255;
-    }
-    if (total == 0 || total > (dg.kind == SPL_RAYS ? kLineMaxBytesRays : kLineMaxBytes)) return;
-    const long long marched = dg.kind == SPL_PARALLEL ? (long long)(dg.n_views - dg.n_flat) * dg.nu * dg.nv : dg.n_rays;
-    if ((double)marched * (dg.n[0] + dg.n[1] + dg.n[2]) < (double)(total / sizeof(float4))) return;
+    if (dg.n_rays == 0 || (dg.kind == SPL_PARALLEL && dg.n_flat == dg.n_views)) return SPL_OK;
     LineScratch *ls = new (std::nothrow) LineScratch();
-    if (!ls) return;
-    if (cudaMalloc(&ls->block, total) != cudaSuccess) {
-        cudaGetLastError();
-        delete ls;
-        return;
+    if (!ls) return fail(SPL_ERR_OOM, "host allocation failed");
+    ls->mask = line_axes(g, ray_dirs);
+    ls->block = nullptr;
+    ls->bytes = 0;
+    const long long marched = dg.kind == SPL_PARALLEL ? (long long)(dg.n_views - dg.n_flat) * dg.nu * dg.nv : dg.n_rays;
+    const double cells = (double)marched * (dg.n[0] + dg.n[1] + dg.n[2]);
+    for (int n = 0; n < 4; ++n) {
+        size_t off[3];
+        const size_t need = n == 0 ? 0 : line_offsets(dg, ls->mask, n, off);
+        const double most = g->scattered ? kLineScatteredL2[n] * (double)l2_bytes() : (double)kLineMaxBytes;
+        const double vectors = (double)need / (n == 1 ? sizeof(float2) : sizeof(float4));
+        ls->need[n] = (double)need <= most && cells >= vectors ? need : 0;
     }
-    for (int d = 0; d < 3; ++d) ls->arr.a[d] = ((mask >> d) & 1u) ? (char *)ls->block + off[d] : nullptr;
     g->line = ls;
+    return SPL_OK;
 }
 
 void line_free(LineScratch *ls)
@@ -529,38 +545,69 @@ void line_free(LineScratch *ls)
     delete ls;
 }
 
+spl_status line_prepare(spl_geometry *g, int degree, cudaStream_t st)
+{
+    LineScratch *ls = g->line;
+    // (no allocation into a capture: a captured forward has no use for it)
+    if (!ls || ls->need[degree] == 0 || stream_captures(st)) return SPL_OK;
+    std::lock_guard<std::mutex> lock(g->turn->mu);
+    if (ls->bytes >= ls->need[degree]) return SPL_OK;
+    // a scratch that takes more than a quarter of what is free is left out
+    size_t free_bytes = 0, total = 0;
+    spl_status s = cuda_check(cudaMemGetInfo(&free_bytes, &total), "memory query");
+    if (s != SPL_OK) return s;
+    if (ls->need[degree] > free_bytes / 4) return SPL_OK;
+    // the block of a lower degree may still be in use
+    if (ls->block && g->turn->used) s = cuda_check(cudaEventSynchronize(g->turn->last), "line scratch wait");
+    if (s != SPL_OK) return s;
+    void *block = nullptr;
+    if (cudaMalloc(&block, ls->need[degree]) != cudaSuccess) {
+        cudaGetLastError();
+        return SPL_OK;
+    }
+    cudaFree(ls->block);
+    ls->block = block;
+    ls->bytes = ls->need[degree];
+    return SPL_OK;
+}
+
 bool line_usable(const spl_geometry *g, int degree, bool captured)
 {
     // a captured call takes no turn against calls outside the graph: it keeps
     // the footprint form, which has no scratch
-    return g->line && degree >= 1 && !captured;
+    const LineScratch *ls = g->line;
+    return ls && !captured && ls->need[degree] > 0 && ls->bytes >= ls->need[degree];
 }
 
 template <int N>
 static spl_status line_forward_n(const spl_geometry *g, int kahan, const float *c, float *y, cudaStream_t st)
 {
     const DevGeom &dg = g->dev;
-    LineScratch &S = *g->line;
+    const LineScratch &S = *g->line;
     const QuadRule qr = quad_rule(N);
+    LineArrays arr;
+    size_t off[3];
+    line_offsets(dg, S.mask, N, off);
+    for (int d = 0; d < 3; ++d) arr.a[d] = ((S.mask >> d) & 1u) ? (char *)S.block + off[d] : nullptr;
     int gx = 0, gy = 0, zc[3];
     for (int d = 0; d < 3; ++d) {
         zc[d] = 0;
-        if (!S.arr.a[d]) continue;
+        if (!arr.a[d]) continue;
         const LineDims L = line_dims(dg.n, d, N);
         zc[d] = (L.nd + kLineChunk - 1) / kLineChunk;
         gx = (L.nq + 31) / 32 > gx ? (L.nq + 31) / 32 : gx;
         gy = (L.np + 7) / 8 > gy ? (L.np + 7) / 8 : gy;
     }
-    k_line_resample<N><<<dim3(gx, gy, zc[0] + zc[1] + zc[2]), 256, 0, st>>>(dg, c, S.arr, make_int3(zc[0], zc[1], zc[2]));
+    k_line_resample<N><<<dim3(gx, gy, zc[0] + zc[1] + zc[2]), 256, 0, st>>>(dg, c, arr, make_int3(zc[0], zc[1], zc[2]));
     if (dg.kind == SPL_RAYS) {
         const int ls = line_split(dg.n_rays, LineBlocks<N>::value);
         const long long blocks = ((dg.n_rays << ls) + 127) / 128;
-        k_line_rays<N><<<(unsigned)blocks, 128, 0, st>>>(dg, S.arr, y, qr, kahan, ls);
+        k_line_rays<N><<<(unsigned)blocks, 128, 0, st>>>(dg, arr, y, qr, kahan, ls);
     } else {
         const int v0 = dg.kind == SPL_PARALLEL ? dg.n_flat : 0, nview = dg.n_views - v0;
         const int *order = dg.kind == SPL_PARALLEL ? dg.view_order + v0 : nullptr;
         const int ls = line_split((long long)nview * dg.nu * dg.nv, LineBlocks<N>::value);
-        k_line_views<N><<<line_grid(dg, nview, ls), 128, 0, st>>>(dg, S.arr, y, qr, kahan, order, ls);
+        k_line_views<N><<<line_grid(dg, nview, ls), 128, 0, st>>>(dg, arr, y, qr, kahan, order, ls);
     }
     return cuda_check(cudaGetLastError(), "line forward launch");
 }

@@ -625,7 +625,8 @@ extern "C" spl_status spl_prepare(spl_geometry *g, const spl_basis_desc *basis, 
     if (s != SPL_OK) return s;
     if (basis->mode == SPL_FP_MLP) return SPL_OK;
     if (basis->mode == SPL_FP_TABLE) return spl::table_build(g, basis->degree, (cudaStream_t)stream);
-    if (basis->separable == SPL_SEP_OFF) return SPL_OK;
+    s = spl::line_prepare(g, basis->degree, (cudaStream_t)stream);
+    if (s != SPL_OK || basis->separable == SPL_SEP_OFF) return s;
     spl_status err;
     spl::plane_ready(g, basis->degree, (cudaStream_t)stream, &err);
     return err;

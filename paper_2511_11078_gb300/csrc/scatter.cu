@@ -662,16 +662,16 @@ spl_status scatter_create(spl_geometry *g, const double *ray_dirs, const double 
 {
     const DevGeom &dg = g->dev;
     g->scatter = nullptr;
+    g->scattered = dg.kind == SPL_RAYS && dg.n_rays > 0 && scattered_rays(dg, ray_dirs, ray_points);
     if (dg.n_rays == 0 || (dg.kind == SPL_PARALLEL && dg.n_flat == dg.n_views)) return SPL_OK;
     const unsigned mask = scatter_axes(g, ray_dirs);
-    const bool scattered = dg.kind == SPL_RAYS && scattered_rays(dg, ray_dirs, ray_points);
     ScatterScratch *S = new (std::nothrow) ScatterScratch();
     if (!S) return fail(SPL_ERR_OOM, "host allocation failed");
     // copies of each layout that some degree takes; the first one also serves form 0
     const int first = (mask & 1u) ? 0 : ((mask & 2u) ? 1 : 2);
     int copies = 0;
     for (int n = 0; n < 4; ++n) {
-        S->form[n] = scatter_form(dg, mask, scattered, n);
+        S->form[n] = scatter_form(dg, mask, g->scattered, n);
         S->batches[n] = scatter_batches(dg, mask, n, S->form[n]);
         copies = S->form[n] > copies ? S->form[n] : copies;
     }

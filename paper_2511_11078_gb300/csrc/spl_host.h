@@ -30,7 +30,8 @@ struct spl_geometry {
     spl::ScatterScratch *scatter; // the scatter adjoint's layout copies of c (scatter.cu), or NULL (no rays;
                                   // parallel geometries whose views are all flat)
     spl::ForwardTurn *turn;       // order of the forwards that use scratch, or NULL (there is none)
-    spl::LineScratch *line;       // the forward's resampled coefficients (line.cu), or NULL (not needed or too large)
+    spl::LineScratch *line;       // the forward's resampled coefficients (line.cu), or NULL (no ray needs them)
+    bool scattered;               // explicit rays whose neighbours lie far apart (scatter.cu)
 };
 
 namespace spl {
@@ -150,10 +151,12 @@ bool stream_captures(cudaStream_t st);
 
 // The forward as line integrals of f on resampled coefficients (line.cu),
 // for explicit rays, cone views and the parallel views outside the flat
-// class.  line_create allocates its arrays with the geometry (leaves
-// g->line NULL when they are not needed, too large or not to be had);
+// class.  line_create finds the axes and sizes of its arrays (g->line stays
+// NULL when no ray has a use for them), line_prepare allocates those of a
+// degree (leaves them out when they are not to be had);
 // line_usable: whether an eager call of this degree takes it.
-void line_create(spl_geometry *g, const double *ray_dirs);
+spl_status line_create(spl_geometry *g, const double *ray_dirs);
+spl_status line_prepare(spl_geometry *g, int degree, cudaStream_t st);
 void line_free(LineScratch *ls);
 bool line_usable(const spl_geometry *g, int degree, bool captured);
 spl_status line_forward(const spl_geometry *g, int degree, int kahan, const float *c, float *y, cudaStream_t st);

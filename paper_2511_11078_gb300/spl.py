@@ -20,6 +20,7 @@ SPL_FP_QUAD, SPL_FP_MLP, SPL_FP_DIRECT, SPL_FP_TABLE = 0, 1, 2, 3
 SPL_ADJ_AUTO, SPL_ADJ_GATHER, SPL_ADJ_SCATTER = 0, 1, 2
 SPL_SEP_AUTO, SPL_SEP_OFF = 0, 1
 MLP_PARAMS = 8769
+_ERR_STATE = 6
 STATUS_NAMES = {0: "SPL_OK", 1: "SPL_ERR_ARG", 2: "SPL_ERR_NONFINITE", 3: "SPL_ERR_CUDA", 4: "SPL_ERR_STEPCAP",
                 5: "SPL_ERR_OOM", 6: "SPL_ERR_STATE", 7: "SPL_ERR_UNSUPPORTED", 8: "SPL_ERR_TIMEOUT"}
 
@@ -224,31 +225,38 @@ def _basis_key(bas: BasisDesc):
 def prepare(geom: Geometry, bas: BasisDesc, stream=None):
     """spl_prepare: build what the projector needs for this basis (the plane
     matrices of slice-separable views, the footprint tables of
-    SPL_FP_TABLE); one-time allocation, then a synchronisation."""
+    SPL_FP_TABLE, the forward's scratch); one-time allocation, then a
+    synchronisation."""
+    import torch
+
     check(lib().spl_prepare(geom.handle, C.byref(bas), _stream(stream)))
-    geom._prepared.add(_basis_key(bas))
-
-
-def _ensure_prepared(geom: Geometry, bas: BasisDesc, stream):
-    # spl_forward / spl_adjoint never allocate and refuse a basis whose
-    # structures are not built (SPL_ERR_STATE); the binding prepares each
-    # (degree, mode, separable) once, before its first use
-    if _basis_key(bas) not in geom._prepared:
-        prepare(geom, bas, stream)
+    with torch.cuda.stream(stream):  # (None: the current one)
+        # a call on a capturing stream leaves the forward's scratch out
+        if not torch.cuda.is_current_stream_capturing():
+            geom._prepared.add(_basis_key(bas))
 
 
 def forward(geom: Geometry, c, y, bas: BasisDesc, stream=None):
     """y = A c (Algorithm 2).  c: float32 CUDA [nz,ny,nx]; y: float32 CUDA (n_rays)."""
     _check_sizes(geom, c, y)
-    _ensure_prepared(geom, bas, stream)
+    # spl_forward never allocates; the binding prepares each (degree, mode,
+    # separable) once, before its first use
+    if _basis_key(bas) not in geom._prepared:
+        prepare(geom, bas, stream)
     check(lib().spl_forward(geom.handle, C.byref(bas), _ptr(c), _ptr(y), _stream(stream)))
 
 
 def adjoint(geom: Geometry, y, c, bas: BasisDesc, stream=None):
     """c = A^T y (matched adjoint)."""
     _check_sizes(geom, c, y)
-    _ensure_prepared(geom, bas, stream)
-    check(lib().spl_adjoint(geom.handle, C.byref(bas), _ptr(y), _ptr(c), _stream(stream)))
+    # prepared only where the adjoint needs it (SPL_ERR_STATE), so that a
+    # geometry used for A^T alone does not hold the forward's scratch
+    args = (geom.handle, C.byref(bas), _ptr(y), _ptr(c), _stream(stream))
+    status = lib().spl_adjoint(*args)
+    if status == _ERR_STATE and _basis_key(bas) not in geom._prepared:
+        prepare(geom, bas, stream)
+        status = lib().spl_adjoint(*args)
+    check(status)
 
 
 def count_work(geom: Geometry, degree: int, stream=None):

@@ -280,6 +280,53 @@ def test_large_and_infinite_coefficients(env, orc, degree):
     assert np.all(np.isposinf(y[ref > 1e-3])) and np.all(np.isfinite(y[ref == 0.0]))
 
 
+def test_scratch_comes_with_prepare(env):
+    """The resampled arrays are allocated by spl_prepare for the degree asked
+    for: a geometry that is only made, or used for A^T, holds none, degree 1 takes
+    half of a cubic array's bytes, and a first call that is captured takes none
+    and leaves them to the next eager one.  Degrees in turn on one geometry share
+    the block: the values are those of a fresh geometry, bit for bit."""
+    torch, spl = env
+    rng = np.random.default_rng(25)
+    dims = (256, 250, 240)
+    geo = I.circular_cone(12, 700.0, 1000.0, 260, 250, 1.4)
+    cubic = sum((dims[d] + 3) * (dims[p] + 6) * ((dims[q] + 6 + 7) // 8 * 8 + 3) * 16 for d, p, q in
+                ((0, 1, 2), (1, 0, 2)))  # no ray has z as its dominant axis
+
+    def free():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return torch.cuda.mem_get_info()[0]
+
+    c = torch.tensor(rng.normal(size=dims[::-1]).astype(np.float32), device="cuda")
+    y, b = torch.zeros(geo.n_rays, device="cuda"), torch.empty(dims[::-1], device="cuda")
+    fresh = {}
+    for degree in (1, 2, 3):
+        g = spl.Geometry(dims, I.centred_origin(dims), geo)
+        spl.forward(g, c, y, spl.basis(degree))
+        fresh[degree] = y.clone()
+        g.close()
+    g = spl.Geometry(dims, I.centred_origin(dims), geo)
+    made = free()
+    spl.adjoint(g, y, b, spl.basis(3))
+    assert made - free() < 16 << 20
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        spl.forward(g, c, y, spl.basis(1))
+    graph.replay()
+    del graph
+    assert made - free() < 32 << 20
+    assert float((y - fresh[1]).norm() / y.norm()) <= TOL
+    used = {}
+    for degree in (1, 3, 2, 1, 3):
+        spl.forward(g, c, y, spl.basis(degree))
+        g.status()
+        assert torch.equal(y, fresh[degree]), degree
+        used.setdefault(degree, made - free())
+    assert 0.4 * cubic < used[1] < 0.6 * cubic + (32 << 20)
+    assert 0.95 * cubic < used[3] < 1.05 * cubic + (32 << 20) and abs(used[2] - used[3]) < 16 << 20
+
+
 def test_warp_mates_in_any_order(env):
     """The Gauss rule of a cubic ray depends on which rays share its warp and on
     nothing else: rays put in another order within each group of 32 keep their
