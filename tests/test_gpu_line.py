@@ -300,21 +300,27 @@ def test_scratch_comes_with_prepare(env):
 
     c = torch.tensor(rng.normal(size=dims[::-1]).astype(np.float32), device="cuda")
     y, b = torch.zeros(geo.n_rays, device="cuda"), torch.empty(dims[::-1], device="cuda")
+
+    def captured(g):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            spl.forward(g, c, y, spl.basis(1))
+        graph.replay()
+        torch.cuda.synchronize()
+
     fresh = {}
     for degree in (1, 2, 3):
         g = spl.Geometry(dims, I.centred_origin(dims), geo)
         spl.forward(g, c, y, spl.basis(degree))
         fresh[degree] = y.clone()
+        spl.adjoint(g, y, b, spl.basis(3))
+        captured(g)  # (loads its kernels, which takes memory too)
         g.close()
     g = spl.Geometry(dims, I.centred_origin(dims), geo)
     made = free()
     spl.adjoint(g, y, b, spl.basis(3))
     assert made - free() < 16 << 20
-    graph = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(graph):
-        spl.forward(g, c, y, spl.basis(1))
-    graph.replay()
-    del graph
+    captured(g)
     assert made - free() < 32 << 20
     assert float((y - fresh[1]).norm() / y.norm()) <= TOL
     used = {}
@@ -368,3 +374,81 @@ def test_position_at_the_end_of_a_long_ray(env, orc):
     assert np.all(ref > 0.0)
     y = project(env, dims, geo, c, 3)
     assert np.max(np.abs(y - ref) / ref) <= 2.2e-5
+
+
+def check_forms(env, orc, geo, degree, dims, modes, line):
+    """A geometry that spl_prepare has not seen takes the forms without
+    scratch (SPL_FP_QUAD: footprints, SPL_FP_DIRECT: the direct march), also in a
+    captured call; a prepared one the resampled arrays, whose sums round
+    otherwise (`line`: some bit differs).  All against the oracle."""
+    import ctypes as C
+
+    torch, spl = env
+    rng = np.random.default_rng(31)
+    origin = I.centred_origin(dims)
+    c = rng.normal(size=dims[::-1]).astype(np.float32)
+    ct = torch.tensor(c, device="cuda")
+    ref = orc.forward(degree, dims, origin, c.astype(np.float64), geom_of(orc, geo)).reshape(-1)
+    out = {}
+    for mode in modes:
+        g, b = spl.Geometry(dims, origin, geo), spl.basis(degree, mode)
+        out[mode], captured, prepared = (torch.full((g.n_rays,), float("nan"), device="cuda") for _ in range(3))
+        st = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        spl.check(spl.lib().spl_forward(g.handle, C.byref(b), spl._ptr(ct), spl._ptr(out[mode]), st))
+        spl.forward(g, ct, prepared, b)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            spl.forward(g, ct, captured, b)
+        graph.replay()
+        torch.cuda.synchronize()
+        g.status()
+        for y in (out[mode], prepared):
+            err = np.linalg.norm(y.cpu().numpy() - ref) / np.linalg.norm(ref)
+            assert err <= TOL, (mode, err)
+        assert torch.equal(captured, out[mode])
+        assert torch.equal(prepared, out[mode]) != line
+    if len(modes) == 2 and degree > 0:
+        assert not torch.equal(*out.values())  # two forms
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+@pytest.mark.parametrize("kind", ["parallel", "cone", "rays"])
+def test_forms_with_and_without_scratch(env, orc, kind, degree):
+    torch, spl = env
+    rng = np.random.default_rng(32)
+    if kind == "parallel":
+        geo = I.parallel_views(I.random_directions(rng, 9), 23, 21, 1.1, center=(0.3, -0.2, 0.1))
+    elif kind == "cone":
+        geo = I.helical_cone(9, 50.0, 80.0, 23, 21, 1.4, turns=1.3, table_feed=6.0)
+    else:
+        w = I.random_directions(rng, 3000)
+        geo = I.RayGeometry(w, rng.uniform(-0.6, 0.6, size=w.shape) * np.asarray(DIMS))
+    check_forms(env, orc, geo, degree, DIMS, (spl.SPL_FP_QUAD, spl.SPL_FP_DIRECT), True)
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+@pytest.mark.parametrize("rays", [2000, 9000])
+def test_eight_threads_a_ray_on_resampled_arrays(env, orc, rays, degree):
+    """Few rays, yet enough for the resampled form: 8 threads a ray at every
+    degree, with flat rays and short ones whose parts are empty."""
+    torch, spl = env
+    rng = np.random.default_rng(rays + degree)
+    w = I.random_directions(rng, rays)
+    w[::7, rng.integers(3)] = 0.0
+    w /= np.linalg.norm(w, axis=1, keepdims=True)
+    s = rng.uniform(-1.15, 1.15, size=(rays, 3)) * 0.5 * (np.asarray(DIMS) - 1.0)
+    check_forms(env, orc, I.RayGeometry(w, s), degree, DIMS, (spl.SPL_FP_QUAD,), True)
+
+
+@pytest.mark.parametrize("degree", [1, 2, 3])
+@pytest.mark.parametrize("dims", [(33, 2, 65), (2, 64, 33), (70, 31, 3)])
+def test_chunks_of_the_resampling(env, orc, dims, degree):
+    """Axes just beyond one and two chunks of 32 cells, with enough rays for the
+    resampled form; and too few, which keep the other."""
+    torch, spl = env
+    rng = np.random.default_rng(33)
+    w = I.random_directions(rng, 1500)
+    s = rng.uniform(-0.6, 0.6, size=w.shape) * np.asarray(dims)
+    check_forms(env, orc, I.RayGeometry(w, s), degree, dims, (spl.SPL_FP_QUAD,), True)
+    check_forms(env, orc, I.RayGeometry(w[:60], s[:60]), degree, dims, (spl.SPL_FP_QUAD,), False)
