@@ -64,10 +64,12 @@ typedef enum {
 /* geometry kinds (Eq. 1 lines) */
 enum { SPL_RAYS = 0, SPL_PARALLEL = 1, SPL_CONE = 2 };
 /* footprint evaluators: exact quadrature, or the learned f_theta (Sec. 2.2);
- * SPL_FP_DIRECT: exact too, but spl_forward integrates f itself along the
- * ray (the Gauss nodes of the same pieces, a window of coefficients instead
- * of footprint accumulators) on rays with three nonzero direction
- * components; everything else is as SPL_FP_QUAD (same matrix). */
+ * SPL_FP_DIRECT: exact too (same matrix).  It differs from SPL_FP_QUAD only
+ * where spl_forward has no scratch (see spl_prepare), for degree 0 and in
+ * captured calls: there it integrates f itself along the ray (the Gauss nodes
+ * of the same pieces, a window of coefficients instead of footprint
+ * accumulators) on rays with three nonzero direction components; with the
+ * scratch both modes integrate f on the resampled coefficients. */
 enum { SPL_FP_QUAD = 0, SPL_FP_MLP = 1, SPL_FP_DIRECT = 2, SPL_FP_TABLE = 3 };
 /* SPL_FP_TABLE (parallel-beam geometries only): the splat form, an
  * approximation.  Each view's footprint, one 2-D function on H_w, is
@@ -85,8 +87,8 @@ enum { SPL_FP_QUAD = 0, SPL_FP_MLP = 1, SPL_FP_DIRECT = 2, SPL_FP_TABLE = 3 };
  * this GPU (the scatter form); SPL_ADJ_GATHER walks coefficient bricks and
  * accumulates in shared memory (no global atomics); SPL_ADJ_SCATTER walks
  * rays like spl_forward and adds with float atomics to global memory.  Both
- * visit the same pairs with the same footprint values; both add in an
- * order that varies between runs (float atomics in shared or global
+ * visit the same pairs with the same footprints to FP32 rounding, and both add
+ * in an order that varies between runs (float atomics in shared or global
  * memory), so results agree to rounding, not bit for bit. */
 enum { SPL_ADJ_AUTO = 0, SPL_ADJ_GATHER = 1, SPL_ADJ_SCATTER = 2 };
 /* slice-separable parallel views (see spl_prepare): SPL_SEP_AUTO uses the
@@ -131,8 +133,8 @@ typedef struct {
 /* Basis and footprint choice.
  *   degree: n in 0..3 (B-spline degree of the tensor-product basis).
  *   mode:   SPL_FP_QUAD (exact piecewise Gauss-Legendre footprint),
- *           SPL_FP_DIRECT (the same operator; forward as the direct line
- *           integral of f), SPL_FP_TABLE (tabulated footprints, parallel
+ *           SPL_FP_DIRECT (the same operator; forward without scratch as
+ *           the direct line integral of f), SPL_FP_TABLE (tabulated footprints, parallel
  *           beams) or SPL_FP_MLP (learned footprint f_theta, Algorithm 2's
  *           f_theta*);
  *           SPL_FP_MLP needs `mlp` built for the same degree.
@@ -263,8 +265,7 @@ spl_status spl_forward(const spl_geometry *g, const spl_basis_desc *basis, const
 /* Adjoint (back-projection) c = A^T y: the transpose of the matrix of Eq. 6,
  * matched to spl_forward (Sec. 2.3): the exact footprint of every (ray,
  * basis) pair of Eq. 4, integrated over the same pieces (the two agree to
- * FP32 rounding; the footprint form of spl_forward evaluates bit-identical
- * values).  View
+ * FP32 rounding).  View
  * geometries use the form chosen by basis->adjoint (SPL_ADJ_*): a
  * ray-driven scatter with float atomics (the default) or a gather over
  * coefficient bricks that loops over views and the detector window of the
@@ -283,9 +284,11 @@ spl_status spl_adjoint(const spl_geometry *g, const spl_basis_desc *basis, const
  * count_dev[0] += number of contributions of Eq. 4: (ray, basis) pairs whose
  * line meets the open support cube of the basis in a segment of positive
  * length, decided exactly as spl_count_pairs_per_ray does;
- * count_dev[1] += pieces the march integrates with the full Gauss-Legendre
- * rule of ceil((3n+1)/2) nodes (rays with three nonzero direction
- * components, and every cone ray); count_dev[2] += pieces of parallel and
+ * count_dev[1] += pieces of rays with three nonzero direction components and
+ * of every cone ray (ceil((3n+1)/2) Gauss-Legendre nodes each; in A on
+ * resampled coefficients and in the scatter A^T, four instead of five cubic
+ * nodes where that misses less than 2^-28 of a footprint per piece);
+ * count_dev[2] += pieces of parallel and
  * explicit rays with a zero component (n+1 nodes each: the third factor is
  * constant along the ray). */
 spl_status spl_count_pairs(const spl_geometry *g, int degree, unsigned long long *count_dev, void *stream);
