@@ -547,7 +547,7 @@ struct ScatterScratch {
     size_t bytes;
     int form[4];     // per degree (scatter_form)
     int batches[4];  // per degree (scatter_batches)
-    bool dirty;      // a launch failed between scatter and fold: clear before the next call
+    bool dirty;      // to be cleared before the next call: new, or a launch failed between scatter and fold
 };
 
 // Axes that can be the smallest component of a line of the geometry (a
@@ -686,18 +686,13 @@ spl_status scatter_create(spl_geometry *g, const double *ray_dirs, const double 
         if ((mask >> b) & 1u) floats += cs * (copies > 0 ? copies : (b == first ? 1 : 0));
     }
     S->bytes = floats * sizeof(float);
-    cudaError_t ce = cudaMalloc(&S->block, S->bytes);
-    if (ce == cudaSuccess) {
-        ce = cudaMemset(S->block, 0, S->bytes);
-        if (ce != cudaSuccess) cudaFree(S->block);
-    }
-    if (ce != cudaSuccess) {
+    if (cudaMalloc(&S->block, S->bytes) != cudaSuccess) {
         const size_t bytes = S->bytes;
         cudaGetLastError();
         delete S;
         return fail(SPL_ERR_OOM, "cudaMalloc of the adjoint's layout copies (%zu bytes) failed", bytes);
     }
-    S->dirty = false;
+    S->dirty = true;
     S->T.cs = cs;
     S->T.one = first;
     for (int b = 0; b < 3; ++b)

@@ -254,3 +254,29 @@ def test_scattered_rays_in_batches(env, dims):
             parts.append(c.double())
             g.close()
         assert float((parts[0] - sum(parts[1:])).norm() / parts[0].norm()) <= TOL
+
+
+def test_first_adjoint_captured(env):
+    """A geometry's layouts are cleared by its first eager adjoint; a captured
+    call before it records its own clear.  Layouts in memory that held NaN."""
+    torch, spl = env
+    rng = np.random.default_rng(17)
+    dims = (120, 110, 100)
+    w = I.random_directions(rng, 3000)
+    s = rng.uniform(-0.4, 0.4, size=w.shape) * np.asarray(dims)
+    y = torch.randn(len(w), device="cuda")
+    poison = torch.full((1 << 27,), float("nan"), device="cuda")
+    torch.cuda.synchronize()
+    del poison
+    torch.cuda.empty_cache()
+    g = spl.Geometry(dims, I.centred_origin(dims), I.RayGeometry(w, s))
+    replayed, eager = (torch.full(dims[::-1], float("nan"), device="cuda") for _ in range(2))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        spl.adjoint(g, y, replayed, spl.basis(3))
+    spl.adjoint(g, y, eager, spl.basis(3))
+    graph.replay()
+    torch.cuda.synchronize()
+    g.status()
+    assert bool(torch.isfinite(eager).all())
+    assert float((replayed - eager).norm() / eager.norm()) <= TOL
