@@ -482,7 +482,7 @@ struct LineScratch {
 //    2.2 up to 384^3 (2.9 GB), like those of views;
 //  * all three axes of a cubic 512^3 grid take 6.7 GB; beyond 24 GB, or a quarter
 //    of the memory that is free, the scratch is out of proportion.
-constexpr size_t kLineMaxBytes = (size_t)24 << 30;
+constexpr size_t kLineMaxBytes = (size_t)24 << 30, kLineSmallBytes = (size_t)1 << 30;
 constexpr double kLineScatteredL2[4] = {0.0, 1.75, 1.5, 3.0};  // most bytes in L2s, per degree
 
 // Axes that can be the dominant one of a line of the geometry (a superset).
@@ -552,11 +552,15 @@ spl_status line_prepare(spl_geometry *g, int degree, cudaStream_t st)
     if (!ls || ls->need[degree] == 0 || stream_captures(st)) return SPL_OK;
     std::lock_guard<std::mutex> lock(g->turn->mu);
     if (ls->bytes >= ls->need[degree]) return SPL_OK;
-    // a scratch that takes more than a quarter of what is free is left out
-    size_t free_bytes = 0, total = 0;
-    spl_status s = cuda_check(cudaMemGetInfo(&free_bytes, &total), "memory query");
-    if (s != SPL_OK) return s;
-    if (ls->need[degree] > free_bytes / 4) return SPL_OK;
+    // a large scratch that takes more than a quarter of what is free is left out
+    // (the query takes 0.2 ms)
+    spl_status s = SPL_OK;
+    if (ls->need[degree] > kLineSmallBytes) {
+        size_t free_bytes = 0, total = 0;
+        s = cuda_check(cudaMemGetInfo(&free_bytes, &total), "memory query");
+        if (s != SPL_OK) return s;
+        if (ls->need[degree] > free_bytes / 4) return SPL_OK;
+    }
     // the block of a lower degree may still be in use
     if (ls->block && g->turn->used) s = cuda_check(cudaEventSynchronize(g->turn->last), "line scratch wait");
     if (s != SPL_OK) return s;

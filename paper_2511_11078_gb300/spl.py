@@ -230,10 +230,14 @@ def prepare(geom: Geometry, bas: BasisDesc, stream=None):
     import torch
 
     check(lib().spl_prepare(geom.handle, C.byref(bas), _stream(stream)))
-    with torch.cuda.stream(stream):  # (None: the current one)
-        # a call on a capturing stream leaves the forward's scratch out
-        if not torch.cuda.is_current_stream_capturing():
-            geom._prepared.add(_basis_key(bas))
+    # (a call on a capturing stream leaves the forward's scratch out)
+    if stream is None:
+        capturing = torch.cuda.is_current_stream_capturing()
+    else:
+        with torch.cuda.stream(stream):
+            capturing = torch.cuda.is_current_stream_capturing()
+    if not capturing:
+        geom._prepared.add(_basis_key(bas))
 
 
 def forward(geom: Geometry, c, y, bas: BasisDesc, stream=None):
