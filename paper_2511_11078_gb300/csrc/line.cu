@@ -36,11 +36,11 @@
 // one before: pieces of one ray may be walked by several threads.
 //
 // Bound by the FMA pipe (64 % busy) and the latency of a piece's loads at 16
-// warps per SM; 8 views of the 512^3 helical workload take 43 ms and 10.3 warp
-// instructions a piece (the footprint form 73 ms and 22.7), 120 views of the
-// 256^3 cone 85 ms (149), 64 general parallel views of 128^3 4.9 ms (8.9; linear
-// 1.0 and 2.2), quadratic 180 x 180 x 50 4.2 ms (5.0).  The relative error
-// against FP64 is 2.8e-8 (1.25e-7 cubic, 4.3e-8 linear and quadratic).
+// warps per SM; 8 views of the 512^3 helical workload take 44.5 ms with the
+// resampling (the footprint form 73 ms), 120 views of the 256^3 cone 86 ms (149),
+// 64 general parallel views of 128^3 5.0 ms (8.9; linear 0.97 and 2.2), quadratic
+// 180 x 180 x 50 4.2 ms (5.0).  The relative error against FP64 is 2.7e-8 (1.25e-7
+// cubic, 4.3e-8 linear and quadratic).
 #include <math.h>
 
 #include <new>

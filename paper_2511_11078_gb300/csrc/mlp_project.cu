@@ -121,7 +121,9 @@ template <int N> struct MlpSmem {
 // 45 %, tensor pipe 15 % (one view of the 256^3 cone).  6 such views: 282 ms
 // (A), 274 (A^T) with one group of 168 registers per CTA, three CTAs per SM,
 // and a reciprocal per SiLU; 239 with the shared reciprocal (silu4), 228 and
-// 225 with two groups sharing the operands at 128 registers, 16 warps per SM.
+// 225 with two groups sharing the operands at 128 registers, 16 warps per SM,
+// 217 and 215 with the slabs divided (mlp_split); 225 and 221 with a reciprocal
+// for each value of the output layer (silu4's comment).
 // Measured and not kept: both halves of a row loaded before either is
 // evaluated, with the ray's enumeration state parked in TMEM (228).
 //

@@ -1,8 +1,9 @@
 // project.cu -- forward projection A (Algorithm 2, Eq. 4) and its matched
-// adjoint A^T (Sec. 2.3: the adjoint is matched exactly to the forward),
-// exact quadrature footprint.
+// adjoint A^T (Sec. 2.3: the same matrix, to FP32 rounding), exact quadrature
+// footprint: dispatch, and the forms that need no scratch.
 //
-// Forward: one thread per ray; the 128 threads of a block cover a 16 x 8
+// Forward of degrees 1 to 3 with the geometry's scratch: line.cu.  Without it
+// (degree 0, captured calls, geometries not prepared): one thread per ray; the 128 threads of a block cover a 16 x 8
 // detector tile of one view (a warp is an 8 x 4 sub-tile), so neighbouring
 // lanes walk neighbouring lines and gather neighbouring coefficients (L1
 // hits).  Each ray is walked with the cell march (one Gauss node set per

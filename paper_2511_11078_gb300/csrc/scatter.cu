@@ -13,7 +13,7 @@
 // on both sides, so no entry of a face needs a bounds test, and rows are
 // a multiple of 4 floats apart, so the copy is chosen once per b crossing and
 // not once per row.  The values of a b event are single ones and go to copy 0
-// (8 helical views 56.2 -> 55.6 ms against the ray's current copy).  k_fold_*
+// (8 helical views 1 % faster than with the ray's current copy).  k_fold_*
 // add the layouts into c (or the FP64 total of the batches) and leave them
 // cleared for the next call.  Explicit rays that do not lie side by side take
 // fewer copies, or single values into one layout (scatter_form).
@@ -25,8 +25,8 @@
 // on 8 views of the 256^3 cone, the L2's tag lookups at 66 %) and by those tag
 // lookups on the 512^3 helical views (86 %).  Against
 // the mirrored march with bounds tests and double-float positions at 3 blocks
-// per SM: 8 such views 9.5 -> 7.3 ms, 8 helical views of 512^3 71.2 -> 56.2, 64
-// general parallel views of 128^3 8.4 -> 5.9, quadratic 180 x 180 x 50 8.5 ->
+// per SM: 8 such views 9.5 -> 7.35 ms, 8 helical views of 512^3 71.2 -> 54.9, 64
+// general parallel views of 128^3 8.4 -> 6.0, quadratic 180 x 180 x 50 8.5 ->
 // 5.3 (rows of three were scalar atomics), 24^3 0.18 -> 0.08.  Measured and not
 // kept: b events in a branch of their own, which leaves one select per entry
 // instead of two (the register allocation spills: 7.3 -> 9.5 ms); 3 blocks per
