@@ -11,10 +11,10 @@
 //   quadratic: x = y = c_1, z = (c_0 - c_1) / 2, w = (c_2 - c_1) / 2, g(q) = q;
 //   linear:    x = c_0, y = c_1, z = w = 0.
 // k_line_resample writes x, y, z, w of every cell and column as one float4
-// (x, y as a float2 for n = 1; no y for n = 2).  A ray is cut into the pieces of the piece march
-// (spl_march.cuh: cells along its dominant axis, split at the knot planes of
-// the other two, r <= 1) and each piece is integrated with the same
-// Gauss-Legendre rule; a node needs two weight sets instead of three and
+// (x, y as a float2 for n = 1; no y for n = 2).  A ray is cut into the pieces
+// of the piece march (spl_march.cuh: cells along its dominant axis, split at
+// the knot planes of the other two, r <= 1) and each piece is integrated with
+// a Gauss-Legendre rule; a node needs two weight sets instead of three and
 // contracts (n+1)^2 columns:
 //   f(t) = (s, t) . sum_i wa_i sum_k wb_k ((x, y) + (g(s), g(t)) (z, w)),
 // the two terms as one packed FP32x2 value.
