@@ -12,10 +12,8 @@
 // for n = 1) into the copy in which it starts a group.  Every axis is padded
 // on both sides, so no entry of a face needs a bounds test, and rows are
 // a multiple of 4 floats apart, so the copy is chosen once per b crossing and
-// not once per row.  The values of a b event are single ones and go to copy 0
-// (8 helical views 1 % faster than with the ray's current copy).  k_fold_*
-// add the layouts into c (or the FP64 total of the batches) and leave them
-// cleared for the next call.  Explicit rays that do not lie side by side take
+// not once per row.  k_fold_* add the layouts into c (or the FP64 total of the
+// batches) and leave them cleared for the next call.  Explicit rays that do not lie side by side take
 // fewer copies, or single values into one layout (scatter_form).
 //
 // The march keeps, next to its 64 accumulators, only what every piece needs
@@ -205,8 +203,10 @@ __device__ __forceinline__ void row_add(float *p, const float (&v)[N + 1], int s
 }
 
 // March over part `seg` of 2^ls equal parts of the ray's cells.  Returns
-// false if the event bound was reached.
-template <int N, int CP>
+// false if the event bound was reached.  HOME: the single values of a b event,
+// which need no alignment, go to copy 0 and not to the ray's current copy
+// (ScatterScratch::home).
+template <int N, int CP, bool HOME>
 __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int ls, size_t cs, const QuadRule &qr)
 {
     constexpr int M = GL<N>::M, C1 = CP > 0 ? CP : 1;
@@ -286,10 +286,10 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
         const bool evA = ta <= tb && ta <= 1.0f, evB = !evA && tb <= 1.0f, evD = !evA && !evB;
         const int2 st = make_int2(R.sd, R.sa);
         // the face that leaves: D: (0, x, .), A: (x, 0, .): rows along b;
-        // B: (x, y, 0): single values, into copy 0
+        // B: (x, y, 0): single values
         if (in) {
             if (evB) {
-                float *w0 = wp - (-(QB + kLo) & (C1 - 1)) * (long long)(cs + 1);
+                float *w0 = HOME ? wp - (-(QB + kLo) & (C1 - 1)) * (long long)(cs + 1) : wp;
 #pragma unroll
                 for (int x = 0; x <= N; ++x)
 #pragma unroll
@@ -354,7 +354,7 @@ __device__ __forceinline__ bool scatter_march(const ScatterRay &R, int seg, int 
 template <int N> struct ScatterBlocks { static constexpr int value = N == 3 ? 4 : (N == 2 ? 5 : 8); };
 
 // rays r0 .. r1 - 1, 2^ls threads each
-template <int N, int CP>
+template <int N, int CP, bool HOME>
 __global__ void __launch_bounds__(128, ScatterBlocks<N>::value)
     k_scatter_rays(DevGeom g, ScatterTarget T, const float *__restrict__ y, QuadRule qr, long long r0, long long r1, int ls)
 {
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(128, ScatterBlocks<N>::value)
         }
     }
     __syncthreads();
-    if (!scatter_march<N, CP>(rays[t >> ls], t & ((1 << ls) - 1), ls, T.cs, qr)) atomicOr(g.err, 1);
+    if (!scatter_march<N, CP, HOME>(rays[t >> ls], t & ((1 << ls) - 1), ls, T.cs, qr)) atomicOr(g.err, 1);
 }
 
 // Whether a warp's eight consecutive lanes run along detector v: along the
@@ -393,7 +393,7 @@ __device__ __forceinline__ bool scatter_lanes_along_v(const DevGeom &g, int k)
 
 // views v0 + blockIdx.z (of order[], when given); the block's pixels form the
 // tiles of line_tile
-template <int N>
+template <int N, bool HOME>
 __global__ void __launch_bounds__(128, ScatterBlocks<N>::value)
     k_scatter_views(DevGeom g, ScatterTarget T, const float *__restrict__ y, QuadRule qr, const int *order, int v0, int ls)
 {
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(128, ScatterBlocks<N>::value)
         }
     }
     __syncthreads();
-    if (!scatter_march<N, kCopies<N>>(rays[t >> ls], t & ((1 << ls) - 1), ls, T.cs, qr)) atomicOr(g.err, 1);
+    if (!scatter_march<N, kCopies<N>, HOME>(rays[t >> ls], t & ((1 << ls) - 1), ls, T.cs, qr)) atomicOr(g.err, 1);
 }
 
 // ---------------------------------------------------------------- fold
@@ -547,6 +547,12 @@ struct ScatterScratch {
     size_t bytes;
     int form[4];     // per degree (scatter_form)
     int batches[4];  // per degree (scatter_batches)
+    // per degree: single values go to copy 0.  Where the copies outgrow the L2,
+    // that makes the target smaller (8 helical views 55.5 -> 54.9 ms); otherwise
+    // many rays through a small grid would meet at one address (300 000 through
+    // 12^3: 0.53 ms, 0.39 in the rays' copies).  Linear splines: always (64
+    // general parallel views of 128^3 1.61 -> 1.53 ms).
+    bool home[4];
     bool dirty;      // to be cleared before the next call: new, or a launch failed between scatter and fold
 };
 
@@ -673,6 +679,10 @@ spl_status scatter_create(spl_geometry *g, const double *ray_dirs, const double 
     for (int n = 0; n < 4; ++n) {
         S->form[n] = scatter_form(dg, mask, g->scattered, n);
         S->batches[n] = scatter_batches(dg, mask, n, S->form[n]);
+        size_t bytes = 0;
+        for (int b = 0; b < 3; ++b)
+            bytes += ((mask >> b) & 1u) ? scatter_dims(dg.n, b).total * sizeof(float) * S->form[n] : 0;
+        S->home[n] = n == 1 || bytes > l2_bytes();
         copies = S->form[n] > copies ? S->form[n] : copies;
     }
     size_t cs = 0, floats = 0, off[3];
@@ -749,13 +759,18 @@ static spl_status scatter_n(const spl_geometry *g, const float *y, long long i0,
         const unsigned blocks = (unsigned)((((i1 - i0) << ls) + 127) / 128);
         const ScatterTarget T = scatter_target(S, N);
         auto launch = [&](auto kernel) { kernel<<<blocks, 128, 0, st>>>(dg, T, y, qr, i0, i1, ls); };
-        if (form == 0) launch(k_scatter_rays<N, 0>);
-        else if (N >= 2 && form == 2) launch(k_scatter_rays<N, N >= 2 ? 2 : kCopies<N>>);
-        else launch(k_scatter_rays<N, kCopies<N>>);
+        if (form == 0) launch(k_scatter_rays<N, 0, false>);
+        else if (N >= 2 && form == 2) launch(k_scatter_rays<N, N >= 2 ? 2 : kCopies<N>, false>);
+        else if (S.home[N]) launch(k_scatter_rays<N, kCopies<N>, true>);
+        else launch(k_scatter_rays<N, kCopies<N>, false>);
     } else {
         const int views = (int)(i1 - i0), ls = line_split((long long)views * dg.nu * dg.nv, ScatterBlocks<N>::value);
-        k_scatter_views<N><<<line_grid(dg, views, ls), 128, 0, st>>>(
-            dg, scatter_target(S, N), y, qr, dg.kind == SPL_PARALLEL ? dg.view_order : nullptr, (int)i0, ls);
+        auto launch = [&](auto kernel) {
+            kernel<<<line_grid(dg, views, ls), 128, 0, st>>>(dg, scatter_target(S, N), y, qr,
+                                                             dg.kind == SPL_PARALLEL ? dg.view_order : nullptr, (int)i0, ls);
+        };
+        if (S.home[N]) launch(k_scatter_views<N, true>);
+        else launch(k_scatter_views<N, false>);
     }
     const spl_status s = cuda_check(cudaGetLastError(), "adjoint launch");
     if (s != SPL_OK) S.dirty = true;
