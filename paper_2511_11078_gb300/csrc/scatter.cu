@@ -13,8 +13,9 @@
 // on both sides, so no entry of a face needs a bounds test, and rows are
 // a multiple of 4 floats apart, so the copy is chosen once per b crossing and
 // not once per row.  k_fold_* add the layouts into c (or the FP64 total of the
-// batches) and leave them cleared for the next call.  Explicit rays that do not lie side by side take
-// fewer copies, or single values into one layout (scatter_form).
+// batches) and leave them cleared for the next call.  Explicit rays that do not
+// lie side by side take fewer copies, or single values into one layout
+// (scatter_form).
 //
 // The march keeps, next to its 64 accumulators, only what every piece needs
 // in registers (4 blocks of 128 threads per SM); the ray's constants sit in
